@@ -494,7 +494,7 @@ attend_prefix_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
     }
   } else if (warp == 0) {
     // ---------------------------------------------------------------- producer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint64_t pol = policy_evict_first();
       uint32_t k_issued = 0, k_par = 0, v_issued = 0, v_par = 0, q_issued = 0, q_par = 0;
       int Tk = 0, Tv = 0, v = 0;  // K and V tiles issued so far, items processed so far
@@ -591,7 +591,7 @@ attend_prefix_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t id_s = idesc_bf16_f32(kBV, kBN);
       const uint32_t id_o = idesc_bf16_f32(kBV, DH) | (1u << 16);  // B (V) is MN-major
       const uint32_t qs = smem_u32(smem);

@@ -270,7 +270,7 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint64_t pol_w = policy_evict_first(), pol_h = policy_evict_last();
       // the weight bytes one stage brings: bf16 or e4m3 tile, or packed
       // 4-bit codes (half the unpacked tile) and their scale-factor chunk;
@@ -321,7 +321,7 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = F8 ? idesc_e4m3_f32(kBM, a.Nt) : idesc_bf16_f32(kBM, a.Nt);
       int s = 0, local = 0;
       uint32_t ph = 0;
@@ -343,6 +343,9 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           tc_fence_after();
           const uint32_t sa = smem_u32(smem + size_t(s) * stage_bytes);
           const uint32_t sb = sa + a_bytes;
+          // descriptors built once per stage, stepped along K by adding to
+          // their start-address field (16-byte units)
+          const uint64_t da = desc_k_sw128(sa), db = desc_k_sw128(sb);
           if (W4 || MX) {
             // the slice's weight scale factors into this stage's 4 columns
             // (mxfp8: the hidden states' too, 4 columns per 128 token rows);
@@ -356,18 +359,16 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-              mma_mx(d_tmem, desc_k_sw128(sa + 32 * k), desc_k_sw128(sb + 32 * k),
+              mma_mx(d_tmem, da + 2 * k, db + 2 * k,
                      idesc_mx(W4 ? 5u : 0u, kBM, a.Nt, k), sfa, sfb, (kb | k) != 0);
           } else {
             // 32 bytes of K per instruction: 16 bf16 or 32 e4m3 elements
 #pragma unroll
             for (int k = 0; k < kBKBytes / 32; ++k) {
               if (F8)
-                mma_e4m3(d_tmem, desc_k_sw128(sa + 32 * k), desc_k_sw128(sb + 32 * k), idesc,
-                         (kb | k) != 0);
+                mma_e4m3(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
               else
-                mma_f16(d_tmem, desc_k_sw128(sa + 32 * k), desc_k_sw128(sb + 32 * k), idesc,
-                        (kb | k) != 0);
+                mma_f16(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
             }
           }
           mma_commit(empty + s);  // frees the stage once these MMAs have read it

@@ -136,7 +136,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint64_t pol_w = policy_evict_first(), pol_x = policy_evict_last();
       int s = 0;
       uint32_t ph = 0, issued = 0, issued_par = 0;
@@ -186,7 +186,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0 && rank == 0) {
+    if (elect_one() && rank == 0) {
       const uint32_t idesc = idesc_bf16_f32(2 * kBM, a.Nt);
       int s = 0, local = 0;
       uint32_t ph = 0;

@@ -32,7 +32,8 @@
 //
 // One CTA per (request, head); 8 warps: lane c of TMEM (value column c, and
 // key column c of W) belongs to thread c of each warpgroup, which split the
-// per-column work between them; thread 0 issues the MMAs and the TMA copies.
+// per-column work between them; thread 0 issues the TMA copies and warp 0's
+// elected thread the MMAs.
 // The next chunk's K goes into a second buffer while the current chunk runs;
 // Q and V are refilled as soon as the current chunk no longer reads them.
 #include <cuda.h>
@@ -414,7 +415,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     qph ^= 1u;
     if (tid == 0) pend &= ~((1u << odd) | 4u);
     // ---- [K; Q] K^T (even chunks) or [Q; K] K^T (odd): k.k and q.k in float32
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {
       tc_fence_after();
 #pragma unroll
       for (int st = 0; st < 8; ++st) {
@@ -526,7 +527,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       // ---- U^T = V^T T'^T (TMEM at X, for the first state MMA to accumulate
       // onto) and W^T = K^T T''^T: V and K are MN-major A operands (exact in
       // bf16), T' and T'' enter as hi + lo
-      if (tid == 0) {
+      if (warp == 0 && elect_one()) {
         tc_fence_after();
         const uint32_t idesc = idesc_bf16_f32(128, 64) | (1u << 15);
 #pragma unroll
@@ -580,7 +581,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     // ---- X = U^T + S0^T [-W | g Q] (delta rule) or O^T = S0^T (g Q)
     // (gated linear attention, X = U^T as stored): three hi/lo passes; the B
     // operand is MN-major (dk rows of 128 tokens)
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {
       tc_fence_after();
 #pragma unroll
       for (int pass = 0; pass < 3; ++pass) {
@@ -646,7 +647,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     __syncthreads();
     // ---- O^T += d^T (M o G)^T (three passes); state^T += (d G[C-1])^T K (two:
     // K is exact in bf16)
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {
       tc_fence_after();
 #pragma unroll
       for (int pass = 0; pass < 3; ++pass) {
@@ -725,6 +726,9 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         if (pend & (1u << b)) mbar_wait(bar_k + b, (kph >> b) & 1u, kDrainNs, nullptr);
       if (pend & 4u) mbar_wait(bar_q, qph, kDrainNs, nullptr);
       if (pend & 8u) mbar_wait(bar_v, vph, kDrainNs, nullptr);
+    }
+    __syncwarp();
+    if (warp == 0 && elect_one()) {
       mma_commit(bar_mma);
       mbar_wait(bar_mma, mph, kDrainNs, nullptr);
     }

@@ -117,6 +117,24 @@ __device__ __forceinline__ bool warp_mbar_wait(uint64_t* bar, uint32_t parity, u
   return __all_sync(0xffffffffu, ok);
 }
 
+// True in one lane of a converged warp (always the same lane for the full
+// mask). The MMA and TMA issuing branches are guarded by it and not by a lane
+// number: tcgen05 and TMA instructions take their operands from uniform
+// registers, and only under elect.sync does the compiler know that a single
+// thread runs the branch and keep them there. With `lane == 0` the issuing
+// thread bounded the tensor-core kernels: 4-bit LM head (139 x 5120 x 151936)
+// 135 -> 107 us, prefill attention (13k positions) 228 -> 198 us, four-layer
+// stack (355 rows) 810 -> 718 us, bf16 LM head (355 x 4096) 370 -> 353 us.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t pred;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(pred));
+  return pred != 0;
+}
+
 __device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
