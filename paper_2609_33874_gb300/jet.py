@@ -168,7 +168,10 @@ def _addr(x) -> Optional[int]:
 def _stream(stream) -> Optional[int]:
     if stream is None:
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        # the current device's current stream as a raw handle: 0.3 us a call,
+        # where building a torch.cuda.Stream object for it takes 3 us (a small
+        # call's whole host time is 8 to 11 us)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
