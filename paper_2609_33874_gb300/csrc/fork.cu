@@ -280,9 +280,312 @@ fork_kernel(const int32_t* __restrict__ cand_offset, const int32_t* __restrict__
   }
 }
 
+// The fork's outputs alone (no forked state written: a decoder stack's linear
+// layers, or a step that does not keep the states), bf16, for candidates of at
+// most kRowTok fed tokens. With no state to write, the prefix state is only
+// read through products: with g_t = a_1 ... a_t and G(i, t) = a_{i+1} ... a_t
+// over a candidate's tokens,
+//   u_t = S_{t-1}^T k_t = g_{t-1} S0^T k_t + sum_{i<t} G(i, t-1) (k_i . k_t) w_i
+//   w_t = b_t (v_t - a_t u_t)              (u = 0 for gated linear attention)
+//   o_t = g_t S0^T q_t + sum_{i<=t} G(i, t) (k_i . q_t) w_i
+// so one pass over S0 serves the k and q of kRowTok tokens at a time (any
+// number of whole candidates), and what is left is a scalar recurrence per
+// column. Stepping a state per candidate instead costs two block-wide
+// reductions and four barriers a token, one token after another (48 us for 355
+// rows of 32 requests x 16 heads, against 5 us of HBM time for the 33.5 MB of
+// prefix states); the products on the CUDA cores took 44 us, bound by
+// instruction issue and shared-memory latency. Here they run as warp-level MMAs
+// (a 16-column tile of S0 per warp: too small a tile for a TMEM accumulator to
+// pay): S0 enters as the exact sum of three bf16 numbers, k and q are bf16, so
+// every product is exact and the sums are float32: 23 us for those rows (two
+// CTAs an SM, 512 CTAs: two rounds of about 10 us, bound by their chains of
+// loads), the four-layer stack around it 713 -> 646 us.
+// A CTA owns 128 value columns of one head of one request. Infinite inputs
+// give non-finite outputs, where the stepped form may give an infinity instead
+// of a NaN.
+constexpr int kRowTok = 16;         // fed tokens of a batch
+constexpr int kRowCols = 128;       // value columns per CTA
+constexpr int kRowThreads = 256;
+constexpr int kXW = kDK / 2 + 4;    // row stride of the staged k and q (32-bit words)
+constexpr int kUW = kRowCols + 8;   // row stride of the products (floats)
+
+struct RowSmem {
+  uint32_t xk[kRowTok][kXW];                // bf16 pairs
+  uint32_t xq[kRowTok + 8][kXW];            // row kRowTok: the shared row's q, then zeros
+  float up[2 * kRowTok + 1][kUW];           // S0^T k, S0^T q, S0^T (the shared row's q)
+  float w[kRowTok][kRowCols];
+  __nv_bfloat16 xv[kRowTok][kRowCols];
+  float kk[kRowTok][kRowTok + 1], kq[kRowTok][kRowTok + 1];  // [t][i]
+  float a[kRowTok], b[kRowTok];
+  int tok[kRowTok], first[kRowTok];  // fed token of a slot; its candidate's first slot
+  int count, next;                   // tokens of the batch; the next batch's candidate
+};
+
+// D += A B: A 16 x 16 (row-major fragments), B 16 x 8, bf16 in, float32 out
+__device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
+                                          uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// the upper halves of two float32 as a bf16 pair (x in the low half)
+__device__ __forceinline__ uint32_t upper_pair(float x, float y) {
+  return __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
+}
+
+// what is left of x below its upper half (exact; 0 for an infinity)
+__device__ __forceinline__ float below_upper(float x) {
+  const float hi = __uint_as_float(__float_as_uint(x) & 0xffff0000u);
+  return x == hi ? 0.f : x - hi;
+}
+
+template <bool DELTA>
+__global__ void __launch_bounds__(kRowThreads, 2)
+fork_rows_kernel(const int32_t* __restrict__ cand_offset,
+                 const int32_t* __restrict__ cand_row_offset,
+                 const int32_t* __restrict__ tgt_offset, const int32_t* __restrict__ row_offset,
+                 int R, int C, int F, int Hl, int dv, const float* __restrict__ s_prefix,
+                 const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
+                 const __nv_bfloat16* __restrict__ v, const float* __restrict__ alpha,
+                 const float* __restrict__ beta, const __nv_bfloat16* __restrict__ q_rows,
+                 __nv_bfloat16* __restrict__ o, int* status) {
+  pdl_begin();
+  extern __shared__ __align__(16) uint8_t row_smem[];
+  RowSmem& sm = *reinterpret_cast<RowSmem*>(row_smem);
+  const int r = blockIdx.z, h = blockIdx.y, j0 = blockIdx.x * kRowCols;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int g4 = lane >> 2, t4 = lane & 3;
+  if (r >= R) return;
+  const int c0 = cand_offset[r], c1 = cand_offset[r + 1];
+  const int n0 = row_offset[r];
+  const int f_begin = n0 - r;  // the request's first fed token
+  const int f_end = f_begin + row_offset[r + 1] - n0 - 1;
+  if (c0 < 0 || c1 < c0 || c1 > C || f_begin < 0 || f_end < f_begin || f_end > F) {
+    if (tid == 0) flag(status, JET_ERR_DEVICE);
+    return;
+  }
+  // this warp's 16 columns of the prefix state in the order of the MMA's A
+  // fragments, float32: A rows g4 and g4 + 8 are columns 2 g4 and 2 g4 + 1 (one
+  // 8-byte load, 64 contiguous bytes per row of S0), A columns the rows of S0.
+  // The layout reads above go first: the staging below waits on them, not on S0.
+  float2 S[8][4];
+  {
+    const float* sp = s_prefix + (size_t(r) * Hl + h) * kDK * size_t(dv) + j0 + 16 * warp + 2 * g4;
+#pragma unroll
+    for (int ks = 0; ks < 8; ++ks)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int kr = 16 * ks + 2 * t4 + (e & 1) + 4 * (e & 2);
+        S[ks][e] = *reinterpret_cast<const float2*>(sp + size_t(kr) * dv);
+      }
+  }
+  const float rs = rsqrtf(float(kDK));
+  // with q_rows, fed token f is written at row f + r + 1
+  const size_t o_shift = q_rows ? size_t(r) + 1 : 0;
+  bool shared_row = q_rows != nullptr;
+  for (int c = c0; c < c1 || shared_row;) {
+    // ---- the batch: whole candidates from c on, at most kRowTok tokens
+    if (warp == 0) {
+      const int cc = c + lane;
+      int cnt = 0, f0 = 0;
+      if (cc < c1) {
+        cnt = tgt_offset[cc + 1] - tgt_offset[cc] - 1;
+        f0 = cand_row_offset[cc] - r - 1;  // fed-token index of y_{c,1}
+        if (cnt < 0 || cnt > kRowTok || f0 < f_begin || f0 + cnt > f_end) {
+          flag(status, JET_ERR_DEVICE);
+          cnt = 0;
+        }
+      }
+      int inc = cnt;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc += y;
+      }
+      const unsigned in = __ballot_sync(0xffffffffu, cc < c1 && inc <= kRowTok);
+      if (in & (1u << lane)) {
+        for (int i = 0; i < cnt; ++i) {
+          sm.tok[inc - cnt + i] = f0 + i;
+          sm.first[inc - cnt + i] = inc - cnt;
+        }
+      }
+      const int taken = __popc(in);  // the inclusive sums grow: a prefix of the lanes
+      const int total = __shfl_sync(0xffffffffu, inc, taken > 0 ? taken - 1 : 0);
+      if (lane == 0) {
+        sm.count = taken > 0 ? total : 0;
+        sm.next = c + taken;
+      }
+    }
+    __syncthreads();
+    const int nt = sm.count;
+    c = sm.next;
+    // ---- stage k, q, this slice's v and the gates: one 16-byte piece of each
+    // per thread (16 tokens x 16 pieces); rows past the batch's are zeros, so
+    // that no stale value enters the MMAs
+    {
+      const int s = tid >> 4, pc = tid & 15;
+      uint4 pk = make_uint4(0, 0, 0, 0), pq = pk, pv = pk, pr = pk;
+      float ga = 0.f, gb = 0.f;
+      if (s < nt) {
+        const size_t row = size_t(sm.tok[s]) * Hl + h;
+        pk = *reinterpret_cast<const uint4*>(k + row * kDK + 8 * pc);
+        pq = *reinterpret_cast<const uint4*>(q + row * kDK + 8 * pc);
+        pv = *reinterpret_cast<const uint4*>(v + row * dv + j0 + 8 * pc);
+        if (pc == 0) {
+          ga = alpha[row];
+          gb = beta[row];
+        }
+      }
+      if (shared_row && s == 0)
+        pr = *reinterpret_cast<const uint4*>(q_rows + (size_t(n0) * Hl + h) * kDK + 8 * pc);
+      *reinterpret_cast<uint4*>(&sm.xk[s][4 * pc]) = pk;
+      *reinterpret_cast<uint4*>(&sm.xq[s][4 * pc]) = pq;
+      *reinterpret_cast<uint4*>(&sm.xv[s][8 * pc]) = pv;
+      if (s < 8) *reinterpret_cast<uint4*>(&sm.xq[kRowTok + s][4 * pc]) = pr;
+      if (pc == 0) {
+        sm.a[s] = ga;
+        sm.b[s] = gb;
+      }
+    }
+    __syncthreads();
+    // ---- S0^T k and S0^T q: this warp's 16 columns x (two tiles of 8 tokens of
+    // each, and the shared row's)
+    {
+      float acc[5][4];
+#pragma unroll
+      for (int i = 0; i < 5; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[i][e] = 0.f;
+#pragma unroll
+      for (int ks = 0; ks < 8; ++ks) {
+        uint32_t bf[5][2];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+          const uint32_t* x = i < 2 ? sm.xk[8 * i + g4] : sm.xq[8 * (i - 2) + g4];
+          bf[i][0] = x[8 * ks + t4];
+          bf[i][1] = x[8 * ks + t4 + 4];
+        }
+        float2 rest[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) rest[e] = S[ks][e];
+        // S0 = the sum of its upper 8, middle 8 and last 8 significand bits
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+          const uint32_t af[4] = {upper_pair(rest[0].x, rest[1].x), upper_pair(rest[0].y, rest[1].y),
+                                  upper_pair(rest[2].x, rest[3].x), upper_pair(rest[2].y, rest[3].y)};
+#pragma unroll
+          for (int i = 0; i < 5; ++i) {
+            const bool live = i == 4 ? shared_row : (i & 1) ? nt > 8 : nt > 0;
+            if (live && (DELTA || i >= 2)) mma_16816(acc[i], af, bf[i][0], bf[i][1]);
+          }
+          if (p < 2) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              rest[e] = make_float2(below_upper(rest[e].x), below_upper(rest[e].y));
+          }
+        }
+      }
+      // acc[i]: columns 2 g4 (0, 1) and 2 g4 + 1 (2, 3) of the warp, tokens 2 t4
+      // and 2 t4 + 1 of the tile
+      const int col = 16 * warp + 2 * g4;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int u = 8 * i + 2 * t4;
+        *reinterpret_cast<float2*>(&sm.up[u][col]) = make_float2(acc[i][0], acc[i][2]);
+        *reinterpret_cast<float2*>(&sm.up[u + 1][col]) = make_float2(acc[i][1], acc[i][3]);
+      }
+      if (t4 == 0)
+        *reinterpret_cast<float2*>(&sm.up[2 * kRowTok][col]) = make_float2(acc[4][0], acc[4][2]);
+    }
+    // ---- k_i . k_t (warp 0) and k_i . q_t (warp 1) of all the batch's tokens
+    if (warp < 2 && (DELTA || warp == 1)) {
+      const uint32_t(*xa)[kXW] = warp == 0 ? sm.xk : sm.xq;
+      float acc[2][4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[0][e] = acc[1][e] = 0.f;
+#pragma unroll
+      for (int ks = 0; ks < 8; ++ks) {
+        const int x = 8 * ks + t4;
+        const uint32_t af[4] = {xa[g4][x], xa[g4 + 8][x], xa[g4][x + 4], xa[g4 + 8][x + 4]};
+        mma_16816(acc[0], af, sm.xk[g4][x], sm.xk[g4][x + 4]);
+        mma_16816(acc[1], af, sm.xk[g4 + 8][x], sm.xk[g4 + 8][x + 4]);
+      }
+      float(*dst)[kRowTok + 1] = warp == 0 ? sm.kk : sm.kq;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        dst[g4][8 * i + 2 * t4] = acc[i][0];
+        dst[g4][8 * i + 2 * t4 + 1] = acc[i][1];
+        dst[g4 + 8][8 * i + 2 * t4] = acc[i][2];
+        dst[g4 + 8][8 * i + 2 * t4 + 1] = acc[i][3];
+      }
+    }
+    __syncthreads();
+    // ---- the recurrence of this thread's column: the block's halves take the
+    // batch's candidates in turn
+    const int col = tid & (kRowCols - 1), half = tid >> 7;
+    int turn = 0;
+    for (int s0 = 0; s0 < nt;) {
+      int s1 = s0 + 1;
+      while (s1 < nt && sm.first[s1] == s0) ++s1;
+      if ((turn++ & 1) == half) {
+        for (int t = s0; t < s1; ++t) {
+          const float a = sm.a[t];
+          float u = 0.f;
+          if (DELTA) {
+            float g = 1.f;
+            for (int i = t - 1; i >= s0; --i) {
+              u = fmaf(g * sm.kk[t][i], sm.w[i][col], u);
+              g *= sm.a[i];
+            }
+            u = fmaf(g, sm.up[t][col], u);
+          }
+          const float w = sm.b[t] * (__bfloat162float(sm.xv[t][col]) - a * u);
+          float acc = sm.kq[t][t] * w, g = a;
+          for (int i = t - 1; i >= s0; --i) {
+            acc = fmaf(g * sm.kq[t][i], sm.w[i][col], acc);
+            g *= sm.a[i];
+          }
+          acc = fmaf(g, sm.up[kRowTok + t][col], acc);
+          sm.w[t][col] = w;  // read by this thread alone
+          o[((size_t(sm.tok[t]) + o_shift) * Hl + h) * dv + j0 + col] =
+              __float2bfloat16_rn(acc * rs);
+        }
+      }
+      s0 = s1;
+    }
+    if (shared_row && half == 1)
+      o[(size_t(n0) * Hl + h) * dv + j0 + col] =
+          __float2bfloat16_rn(sm.up[2 * kRowTok][col] * rs);
+    shared_row = false;
+    __syncthreads();  // the next batch refills the staging buffers
+  }
+}
+
 }  // namespace
 
 namespace {
+
+template <bool DELTA>
+cudaError_t launch_rows(const jet_layout& lay, const jet_dims& d, const float* s_prefix,
+                        const void* q, const void* k, const void* v, const float* alpha,
+                        const float* beta, const void* q_rows, void* o, int* status,
+                        cudaStream_t st) {
+  const jet_sizes& n = lay.n;
+  auto kern = fork_rows_kernel<DELTA>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             int(sizeof(RowSmem)));
+  if (e != cudaSuccess) return e;
+  dim3 grid(unsigned(d.dv / kRowCols), unsigned(d.Hl), unsigned(n.R));
+  return launch_pdl(kern, grid, dim3(kRowThreads), sizeof(RowSmem), st, lay.cand_offset,
+                    lay.cand_row_offset, lay.tgt_offset, lay.row_offset, n.R, n.C, n.N - n.R, d.Hl,
+                    d.dv, s_prefix, static_cast<const __nv_bfloat16*>(q),
+                    static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(v),
+                    alpha, beta, static_cast<const __nv_bfloat16*>(q_rows),
+                    static_cast<__nv_bfloat16*>(o), status);
+}
 
 template <bool DELTA>
 cudaError_t launch_rule(const jet_layout& lay, const jet_dims& d, const float* s_prefix,
@@ -292,6 +595,11 @@ cudaError_t launch_rule(const jet_layout& lay, const jet_dims& d, const float* s
   const jet_sizes& n = lay.n;
   dim3 grid(unsigned(d.dv / kCols), unsigned(d.Hl), unsigned(n.R));
   const int F = n.N - n.R;
+  // No states to write: the prefix state is read once for 16 fed tokens at a
+  // time (23 us against 48 at 355 rows of 32 requests x 16 heads), as long as no
+  // candidate is longer than such a batch and the value width fills its columns.
+  if (!s_fork && d.dtype == JET_DTYPE_BF16 && n.max_len - 1 <= kRowTok && d.dv % kRowCols == 0)
+    return launch_rows<DELTA>(lay, d, s_prefix, q, k, v, alpha, beta, q_rows, o, status, st);
   if (d.dtype == JET_DTYPE_F32) {
     return launch_pdl(fork_kernel<float, DELTA>, grid, dim3(kThreads), 0, st, lay.cand_offset,
                       lay.cand_row_offset, lay.tgt_offset, lay.row_offset, n.R, n.C, F, d.Hl,
