@@ -766,8 +766,11 @@ attend_prefix_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
           ok = false;
           break;
         }
-        if (mt > m_used + kRescaleLog2) {
-          const float m_new = mt;
+        // the whole warp takes the branch when one of its vectors needs it: the
+        // TMEM accesses and the wait below are warp-wide
+        const bool grow = mt > m_used + kRescaleLog2;
+        if (__any_sync(0xffffffffu, grow)) {
+          const float m_new = grow ? mt : m_used;
           if (j >= 1) {
             // O holds this item's P V so far: wait for the last one, rescale in TMEM
             if (!warp_mbar_wait(p_free + ((Tj - 1) & 1), ((Tj - 1) >> 1) & 1, a.wait_ns,
@@ -776,7 +779,7 @@ attend_prefix_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
               break;
             }
             tc_fence_after();
-            const float f = ex2(m_used - m_new);
+            const float f = grow ? ex2(m_used - m_new) : 1.f;
 #pragma unroll 1
             for (int c0 = 0; c0 < DH; c0 += 32) {
               float ov[32];
