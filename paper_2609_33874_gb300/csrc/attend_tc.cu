@@ -1176,8 +1176,8 @@ cudaError_t launch_prefill_tc(const jet_layout& lay, const jet_dims& d, const vo
                               const void* k, const void* v, void* o, void* ws, int* status,
                               cudaStream_t st) {
   if (d.d == 64) return launch_prefill_dh<64>(lay, d, q, k, v, o, ws, status, st);
-  if (d.d == 128) return launch_prefill_dh<128>(lay, d, q, k, v, o, ws, status, st);
-  if (d.d == 256) return launch_prefill_dh<256>(lay, d, q, k, v, o, ws, status, st);
+  if (d.d == 128) return launch_prefill_pair<128>(lay, d, q, k, v, o, status, st);
+  if (d.d == 256) return launch_prefill_pair<256>(lay, d, q, k, v, o, status, st);
   return cudaErrorInvalidValue;
 }
 

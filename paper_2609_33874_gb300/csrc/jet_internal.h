@@ -130,6 +130,12 @@ cudaError_t launch_prefill_tc(const jet_layout& lay, const jet_dims& d, const vo
                               const void* k, const void* v, void* o, void* ws, int* status,
                               cudaStream_t st);
 
+// the same on pairs of SMs (prefill_tc.cu), head dimensions 128 and 256; no work list
+template <int DH>
+cudaError_t launch_prefill_pair(const jet_layout& lay, const jet_dims& d, const void* q,
+                                const void* k, const void* v, void* o, int* status,
+                                cudaStream_t st);
+
 // q_rows (optional, every row's q [N, Hl, dk]): o then covers all N rows, the
 // shared rows reading the prefix states (o = S_r^T q / sqrt(dk)) and fed token
 // f at row f + r + 1; without it o holds the fed tokens only
