@@ -90,6 +90,7 @@ struct TcArgs {
   int* status;
   int N, T, V, D;
   int Nt, n_tt, units, nkb, stages, vtiles;
+  int nblk;              // 16-row blocks the token tiles share out (0: tiles of Nt rows)
   uint32_t tmem_cols;
   uint32_t buf_cols;     // columns of one accumulator
   uint32_t sfb_col;      // the hidden side's scale factors: w4 one slot (all 1),
@@ -98,6 +99,30 @@ struct TcArgs {
   uint64_t wait_ns;  // budget of one bounded wait (jet_set_wait_budget_ns)
   int hold_first;    // test hook (jet_set_test_stall): withhold the first stage's loads
 };
+
+// unit u of `workers` (CTAs or CTA pairs): a vocabulary tile (of a pair: two)
+// and a token tile [t0, t0 + cols). The token tiles of one vocabulary tile are
+// consecutive units, so they share its weights through L2; they are as even as
+// 16-row blocks allow, and the order rotates from round to round, so that every
+// worker gets its share of the larger ones.
+struct Unit {
+  int vg, tt, t0, cols;
+};
+__device__ __forceinline__ Unit unit_of(const TcArgs& a, int u, int workers) {
+  Unit x;
+  x.vg = u / a.n_tt;
+  if (a.nblk) {
+    const int rot = int((long long)x.vg * a.n_tt / workers);
+    x.tt = (u % a.n_tt + rot) % a.n_tt;
+    x.t0 = 16 * int((long long)x.tt * a.nblk / a.n_tt);
+    x.cols = 16 * int((long long)(x.tt + 1) * a.nblk / a.n_tt) - x.t0;
+  } else {
+    x.tt = u % a.n_tt;
+    x.t0 = x.tt * a.Nt;
+    x.cols = a.Nt;
+  }
+  return x;
+}
 
 __device__ __forceinline__ void combine(float& m, float& s, float m2, float s2) {
   const float M = fmaxf(m, m2);
@@ -131,6 +156,17 @@ __device__ __forceinline__ void mma_e4m3(uint32_t d_tmem, uint64_t a_desc, uint6
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// the same on a CTA pair (issued by the even CTA)
+__device__ __forceinline__ void mma_e4m3_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+                                              uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
       "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
@@ -195,7 +231,7 @@ __device__ __forceinline__ void tmem_st_8cols(uint32_t taddr, uint32_t v) {
       : "memory");
 }
 
-template <int FMT>
+template <int FMT, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
 lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmH,
                  const TcArgs a) {
@@ -204,10 +240,11 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   constexpr bool MX = FMT == kFmtMx8;    // e4m3 blocks on both sides, block-scaled MMA
   constexpr bool ROWSC = FMT == kFmtE4m3 || W4;  // float32 scales per weight row and token
   constexpr int kBKe = F8 ? kBKBytes : kBK;  // elements of one K slice
+  static_assert(!PAIR || !(W4 || MX), "the block-scaled formats run on single CTAs");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
-  const uint32_t a_bytes = kBM * 128, b_bytes = uint32_t(a.Nt) * 128;
+  const uint32_t a_bytes = kBM * 128, b_bytes = uint32_t(PAIR ? a.Nt / 2 : a.Nt) * 128;
   // a stage holds the weight and hidden tiles of one K slice (w4: the weight
   // tile as the TMA unpacks it, 1 byte per code) and the slice's scale-factor
   // chunks: w4 the weights' 512 bytes (in a 1 KB slot), mxfp8 also the hidden
@@ -227,6 +264,10 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   volatile int* epi_abort = abort_flag + 1;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // this CTA's rank in its pair, its worker number and the number of workers
+  const uint32_t rank = PAIR ? cluster_rank() : 0;
+  const int wid = int(PAIR ? blockIdx.x >> 1 : blockIdx.x);
+  const int workers = int(PAIR ? gridDim.x >> 1 : gridDim.x);
   if (threadIdx.x == 0) {
     for (int s = 0; s < a.stages; ++s) {
       mbar_init(full + s, 1);
@@ -234,7 +275,7 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull + b, 1);
-      mbar_init(tempty + b, 4);
+      mbar_init(tempty + b, PAIR ? 8 : 4);  // (both CTAs') epilogue warps
     }
     mbar_init(drain, 1);
     *abort_flag = 0;
@@ -248,11 +289,17 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   // global memory and TMEM only after the previous kernel of the stream is done
   pdl_begin();
   if (warp == 1) {
-    tmem_alloc(tmem_slot, a.tmem_cols);
-    tmem_relinquish();
+    if (PAIR) {
+      tmem_alloc_pair(tmem_slot, a.tmem_cols);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(tmem_slot, a.tmem_cols);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync();  // the even CTA's barriers are initialised
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   const uint32_t buf_cols = a.buf_cols;
@@ -280,8 +327,10 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       int s = 0;
       uint32_t ph = 0, issued = 0, issued_par = 0;
       bool ok = true, hold = a.hold_first != 0;
-      for (int u = blockIdx.x; ok && u < a.units; u += gridDim.x) {
-        const int vt = u / a.n_tt, v0 = vt * kBM, t0 = (u % a.n_tt) * a.Nt;
+      for (int u = wid; ok && u < a.units; u += workers) {
+        const Unit x = unit_of(a, u, workers);
+        const int vt = PAIR ? 2 * x.vg + int(rank) : x.vg, v0 = vt * kBM;
+        const int t0 = x.t0 + (PAIR ? int(rank) * (x.cols / 2) : 0);
         for (int kb = 0; kb < a.nkb; ++kb) {
           if (!mbar_wait(empty + s, ph ^ 1u, a.wait_ns, abort_flag)) {
             ok = false;
@@ -290,6 +339,15 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           uint8_t* sa = smem + size_t(s) * stage_bytes;
           if (hold) {
             hold = false;  // test hook: this stage never fills
+          } else if (PAIR) {
+            // both CTAs' bytes complete on the even CTA's barrier, which
+            // expects them all; the odd CTA's may land before that arrive
+            const uint32_t bar = mapa_shared(full + s, 0);
+            if (rank == 0) mbar_arrive_expect_tx(full + s, 2 * stage_bytes);
+            tma_load_2d_pair(sa, &tmW, bar, kb * kBKe, v0, pol_w);
+            tma_load_2d_pair(sa + a_bytes, &tmH, bar, kb * kBKe, t0, pol_h);
+            issued |= 1u << s;
+            issued_par = (issued_par & ~(1u << s)) | (ph << s);
           } else {
             mbar_arrive_expect_tx(full + s, w_tx + b_bytes);
             tma_load_2d(sa, &tmW, full + s, kb * kBKe, v0, pol_w);
@@ -300,7 +358,7 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                         full + s, pol_w);
             if (MX)
               bulk_load(sa + a_bytes + b_bytes + kW4ScaleBytes,
-                        a.h_sf + (size_t(u % a.n_tt) * a.nkb + kb) * 2 * kW4ScaleBytes,
+                        a.h_sf + (size_t(x.tt) * a.nkb + kb) * 2 * kW4ScaleBytes,
                         2 * kW4ScaleBytes, full + s, pol_h);
             issued |= 1u << s;
             issued_par = (issued_par & ~(1u << s)) | (ph << s);
@@ -314,21 +372,31 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       if (!ok) {
         *abort_flag = 1;
         flag(a.status, JET_ERR_TIMEOUT);
-        // let every copy already issued land before the CTA can exit
-        for (int t = 0; t < a.stages; ++t)
-          if (issued & (1u << t)) mbar_wait(full + t, (issued_par >> t) & 1u, kDrainNs, nullptr);
+        // let every copy already issued land before the CTA can exit (of a
+        // pair, the even CTA's barriers count both CTAs' bytes; the odd CTA
+        // waits out a fixed bounded time)
+        if (rank == 0) {
+          for (int t = 0; t < a.stages; ++t)
+            if (issued & (1u << t)) mbar_wait(full + t, (issued_par >> t) & 1u, kDrainNs, nullptr);
+        } else if (issued) {
+          const uint64_t t0 = global_timer_ns();
+          while (global_timer_ns() - t0 < kDrainNs / 16) {
+          }
+        }
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (elect_one()) {
-      const uint32_t idesc = F8 ? idesc_e4m3_f32(kBM, a.Nt) : idesc_bf16_f32(kBM, a.Nt);
+    if (rank == 0 && elect_one()) {
+      constexpr int kM = PAIR ? 2 * kBM : kBM;
       int s = 0, local = 0;
       uint32_t ph = 0;
       bool ok = true;
-      for (int u = blockIdx.x; ok && u < a.units; u += gridDim.x, ++local) {
+      for (int u = wid; ok && u < a.units; u += workers, ++local) {
         const int buf = local & 1;
         const uint32_t tph = (local >> 1) & 1;
+        const int cols = unit_of(a, u, workers).cols;
+        const uint32_t idesc = F8 ? idesc_e4m3_f32(kM, cols) : idesc_bf16_f32(kM, cols);
         if (!mbar_wait(tempty + buf, tph ^ 1u, a.wait_ns, abort_flag)) {
           ok = false;
           break;
@@ -355,35 +423,49 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             tmem_cp_32x128(sfa, sb + b_bytes);
             if (MX) {
               tmem_cp_32x128(sfb, sb + b_bytes + kW4ScaleBytes);
-              if (a.Nt > 128) tmem_cp_32x128(sfb + 4, sb + b_bytes + 2 * kW4ScaleBytes);
+              if (cols > 128) tmem_cp_32x128(sfb + 4, sb + b_bytes + 2 * kW4ScaleBytes);
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k)
               mma_mx(d_tmem, da + 2 * k, db + 2 * k,
-                     idesc_mx(W4 ? 5u : 0u, kBM, a.Nt, k), sfa, sfb, (kb | k) != 0);
+                     idesc_mx(W4 ? 5u : 0u, kBM, cols, k), sfa, sfb, (kb | k) != 0);
           } else {
             // 32 bytes of K per instruction: 16 bf16 or 32 e4m3 elements
 #pragma unroll
             for (int k = 0; k < kBKBytes / 32; ++k) {
-              if (F8)
+              if (PAIR && F8)
+                mma_e4m3_pair(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
+              else if (PAIR)
+                mma_f16_pair(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
+              else if (F8)
                 mma_e4m3(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
               else
                 mma_f16(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
             }
           }
-          mma_commit(empty + s);  // frees the stage once these MMAs have read it
+          // frees the stage (in both CTAs) once these MMAs have read it
+          if (PAIR)
+            mma_commit_pair(empty + s, 0x3);
+          else
+            mma_commit(empty + s);
           if (++s == a.stages) {
             s = 0;
             ph ^= 1u;
           }
         }
         if (!ok) break;
-        mma_commit(tfull + buf);  // accumulator complete
+        if (PAIR)  // accumulator complete
+          mma_commit_pair(tfull + buf, 0x3);
+        else
+          mma_commit(tfull + buf);
       }
       if (!ok) {
         *abort_flag = 1;
         flag(a.status, JET_ERR_TIMEOUT);
-        mma_commit(drain);
+        if (PAIR)
+          mma_commit_pair(drain, 0x1);
+        else
+          mma_commit(drain);
         mbar_wait(drain, 0, kDrainNs, nullptr);
       }
     }
@@ -392,12 +474,15 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
     const int q = warp & 3;          // TMEM lane quadrant this warp may access
     const int et = threadIdx.x - 64;  // 0..127
     const int vrow = q * 32 + lane;   // vocabulary row within the tile
+    // the odd CTA's warps release the accumulator on the even CTA's barrier
+    const uint32_t tempty_even = PAIR ? mapa_shared(tempty, 0) : 0;
     int local = 0;
-    for (int u = blockIdx.x; u < a.units; u += gridDim.x, ++local) {
+    for (int u = wid; u < a.units; u += workers, ++local) {
       const int buf = local & 1;
       const uint32_t tph = (local >> 1) & 1;
-      const int vt = u / a.n_tt;
-      const int v0 = vt * kBM, t0 = (u % a.n_tt) * a.Nt;
+      const Unit x = unit_of(a, u, workers);
+      const int vt = PAIR ? 2 * x.vg + int(rank) : x.vg;
+      const int v0 = vt * kBM, t0 = x.t0;
       const bool ok = warp_mbar_wait(tfull + buf, tph, a.wait_ns, abort_flag);
       if (!ok || *abort_flag) *epi_abort = 1;
       named_bar_sync(1, 128);
@@ -405,7 +490,7 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       tc_fence_after();
       const uint32_t tcol = tmem_base + buf * buf_cols;
       const uint32_t tl = tcol + (uint32_t(32 * q) << 16);
-      const int ncols = min(a.Nt, a.N - t0);
+      const int ncols = min(x.cols, a.N - t0);
       const bool row_valid = v0 + vrow < a.V;
       // e4m3, w4: this row's weight scale, and the unit's token scales in
       // shared memory (mxfp8 needs none: its block scales are in the MMA)
@@ -480,9 +565,15 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       // the accumulator can be overwritten now
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(tempty + buf);
+      if (lane == 0) {
+        if (PAIR)
+          mbar_arrive_remote(tempty_even + 8u * buf);
+        else
+          mbar_arrive(tempty + buf);
+      }
       named_bar_sync(1, 128);
-      for (int c = et; c < ncols; c += 128) {
+      // (an odd number of vocabulary tiles leaves the last pair's odd CTA none)
+      for (int c = et; c < ncols && vt < a.vtiles; c += 128) {
         float M = red[c].x, S = red[c].y;
 #pragma unroll
         for (int w = 1; w < 4; ++w) combine(M, S, red[w * kMaxNt + c].x, red[w * kMaxNt + c].y);
@@ -495,9 +586,15 @@ lmhead_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 
   tc_fence_before();
   __syncthreads();
+  // neither CTA of a pair leaves (or frees its TMEM) while the partner's MMAs or
+  // copies may still use its shared memory or TMEM
+  if (PAIR) cluster_sync();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, a.tmem_cols);
+    if (PAIR)
+      tmem_dealloc_pair(tmem_base, a.tmem_cols);
+    else
+      tmem_dealloc(tmem_base, a.tmem_cols);
   }
 }
 
@@ -558,9 +655,34 @@ int sm_count() {
 
 namespace {
 
+// clusters of two CTAs of `kern` that can be resident at once; asked once per kernel
+template <typename K>
+int max_pairs(K kern, size_t smem) {
+  static int cached = 0;
+  if (cached > 0) return cached;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(2);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute cl{};
+  cl.id = cudaLaunchAttributeClusterDimension;
+  cl.val.clusterDim.x = 2;
+  cl.val.clusterDim.y = 1;
+  cl.val.clusterDim.z = 1;
+  cfg.attrs = &cl;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    return std::max(1, sm_count() / 2);
+  }
+  cached = n;
+  return n;
+}
+
 // one launch of the LM head on bf16 operands, or e4m3 hidden codes with e4m3
 // or block-scaled 4-bit weights, per-row weight scales and per-token hidden scales
-template <int FMT>
+template <int FMT, bool PAIR>
 cudaError_t launch_head(const jet_layout& lay, const jet_dims& d, const ScorePlan& plan,
                         const void* hidden, const float* h_scale, const void* w_lm,
                         const float* w_scale, void* ws, int* status, cudaStream_t st,
@@ -595,10 +717,13 @@ cudaError_t launch_head(const jet_layout& lay, const jet_dims& d, const ScorePla
   a.D = d.D;
   a.Nt = Nt;
   a.n_tt = n_tt;
-  a.units = plan.vtiles * n_tt;
+  // mxfp8 lays the hidden states' scale factors out by tiles of Nt rows
+  a.nblk = MX ? 0 : (n.N + 15) / 16;
+  a.units = (PAIR ? (plan.vtiles + 1) / 2 : plan.vtiles) * n_tt;
   a.vtiles = plan.vtiles;
   a.nkb = (d.D * esize + kBKBytes - 1) / kBKBytes;
-  const int a_bytes = kBM * kBKBytes, b_bytes = Nt * kBKBytes;
+  const int b_rows = PAIR ? Nt / 2 : Nt;  // token-tile rows one CTA loads
+  const int a_bytes = kBM * kBKBytes, b_bytes = b_rows * kBKBytes;
   const int stage_bytes = a_bytes + b_bytes + (W4 ? 1024 : MX ? 2048 : 0);
   a.stages = std::min(8, (kSmemLimit - 1024 - kFixedSmem) / stage_bytes);
   if (a.stages < 2) return cudaErrorInvalidValue;
@@ -623,7 +748,7 @@ cudaError_t launch_head(const jet_layout& lay, const jet_dims& d, const ScorePla
   const size_t smem = 1024 + size_t(a.stages) * stage_bytes + kFixedSmem;
 
   CUtensorMap tmW, tmH;
-  if (!encode_kmajor(&tmH, hidden, n.N, d.D, Nt, esize)) return cudaErrorInvalidValue;
+  if (!encode_kmajor(&tmH, hidden, n.N, d.D, b_rows, esize)) return cudaErrorInvalidValue;
   if (W4) {
     // the code region covers whole tiles: ceil(V / 128) * 128 rows of
     // ceil(D / 128) * 128 codes; the scale-factor region follows it
@@ -637,14 +762,28 @@ cudaError_t launch_head(const jet_layout& lay, const jet_dims& d, const ScorePla
     a.w_sf = w_sf;
     a.h_sf = h_sf;
   }
-  cudaError_t e = cudaFuncSetAttribute(lmhead_tc_kernel<FMT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  auto kern = lmhead_tc_kernel<FMT, PAIR>;
+  cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
   int sms = sm_count();
   if (d.max_sms > 0) sms = std::min(sms, d.max_sms);
+  if (PAIR) {
+    const int pairs = std::max(1, std::min(a.units, std::min(sms / 2, max_pairs(kern, smem))));
+    return launch_pdl_pairs(kern, dim3(unsigned(2 * pairs)), dim3(kThreads), smem, st, tmW, tmH,
+                            a);
+  }
   const int grid = std::max(1, std::min(a.units, sms));
-  return launch_pdl(lmhead_tc_kernel<FMT>, dim3(grid), dim3(kThreads), smem, st,
-                    tmW, tmH, a);
+  return launch_pdl(kern, dim3(grid), dim3(kThreads), smem, st, tmW, tmH, a);
+}
+
+// More than one token tile: on CTA pairs (tcgen05 cta_group::2, 256 vocabulary
+// rows), which halves the hidden-state bytes each SM takes in: 2,405 rows x 2048
+// x 151,936 in the whole step 1,492 -> 1,370 us, 355 rows x 4096 353 -> 326 us.
+// With a single tile the weights' stream from HBM sets the pace (93 % of the
+// copy rate on single CTAs). A limit of one SM (jet_dims.max_sms) leaves no pair.
+bool use_pairs(const jet_layout& lay, const jet_dims& d) {
+  return lay.n.N > kMaxNt && d.max_sms != 1;
 }
 
 }  // namespace
@@ -652,19 +791,25 @@ cudaError_t launch_head(const jet_layout& lay, const jet_dims& d, const ScorePla
 cudaError_t launch_lmhead_tc(const jet_layout& lay, const jet_dims& d, const ScorePlan& plan,
                              const void* hidden, const void* w_lm, void* ws, int* status,
                              cudaStream_t st) {
-  return launch_head<kFmtBf16>(lay, d, plan, hidden, nullptr, w_lm, nullptr, ws, status, st);
+  if (use_pairs(lay, d))
+    return launch_head<kFmtBf16, true>(lay, d, plan, hidden, nullptr, w_lm, nullptr, ws, status,
+                                       st);
+  return launch_head<kFmtBf16, false>(lay, d, plan, hidden, nullptr, w_lm, nullptr, ws, status,
+                                      st);
 }
 
 cudaError_t launch_lmhead_e4m3(const jet_layout& lay, const jet_dims& d, const ScorePlan& plan,
                                const uint8_t* h_q, const float* h_scale, const uint8_t* w_q,
                                const float* w_scale, void* ws, int* status, cudaStream_t st) {
-  return launch_head<kFmtE4m3>(lay, d, plan, h_q, h_scale, w_q, w_scale, ws, status, st);
+  if (use_pairs(lay, d))
+    return launch_head<kFmtE4m3, true>(lay, d, plan, h_q, h_scale, w_q, w_scale, ws, status, st);
+  return launch_head<kFmtE4m3, false>(lay, d, plan, h_q, h_scale, w_q, w_scale, ws, status, st);
 }
 
 cudaError_t launch_lmhead_mx(const jet_layout& lay, const jet_dims& d, const ScorePlan& plan,
                              const uint8_t* h_q, const uint8_t* h_sf, const uint8_t* w_q,
                              const uint8_t* w_sf, void* ws, int* status, cudaStream_t st) {
-  return launch_head<kFmtMx8>(lay, d, plan, h_q, nullptr, w_q, nullptr, ws, status, st, w_sf,
+  return launch_head<kFmtMx8, false>(lay, d, plan, h_q, nullptr, w_q, nullptr, ws, status, st, w_sf,
                               h_sf);
 }
 
@@ -678,7 +823,7 @@ void mx_token_tiling(int N, int* Nt, int* n_tt) {
 cudaError_t launch_lmhead_w4(const jet_layout& lay, const jet_dims& d, const ScorePlan& plan,
                              const uint8_t* h_q, const float* h_scale, const uint8_t* w4,
                              const float* w_scale, void* ws, int* status, cudaStream_t st) {
-  return launch_head<kFmtW4>(lay, d, plan, h_q, h_scale, w4, w_scale, ws, status, st);
+  return launch_head<kFmtW4, false>(lay, d, plan, h_q, h_scale, w4, w_scale, ws, status, st);
 }
 
 }  // namespace jet
