@@ -26,6 +26,7 @@ constexpr int kThreads = 256;
 constexpr long long kTargetCtas = 608;  // about four CTAs per SM on 152 SMs
 constexpr int kPlanSMs = 152;           // GB300
 constexpr int kMinChunkTc = 640;        // keys
+constexpr int kFewGroups = 22, kFewItems = 44, kLeastChunk = 192;
 
 template <int DH>
 constexpr size_t prefix_smem_bytes() {
@@ -265,7 +266,16 @@ AttnPlan attn_plan(const jet_sizes& n, const jet_dims& d) {
     // of one SM's share of all key tiles, so that the schedule can balance
     const double avg_tiles = double(n.total_prefix) / n.R / 64.0 + 0.5;
     const double share = double(groups) * avg_tiles / kPlanSMs;  // tiles per SM
-    chunk = std::max(kMinChunkTc, int(share / 2.0 + 0.999) * 64);
+    int least = kMinChunkTc;
+    // a few long prefixes leave most SMs idle at that length: then about
+    // kFewItems chunks in all, of at least kLeastChunk keys (one 6,000-key request
+    // with two kv heads: 320 keys 20 us, 640 keys 23 us, 128 keys 23 us; 32
+    // groups of 512 keys: unsplit 17.3 us, halves 18.1 us with the combine)
+    if (groups <= kFewGroups) {
+      const long long even = (long long)(double(groups) * avg_tiles / kFewItems + 0.999) * 64;
+      least = int(std::max<long long>(kLeastChunk, std::min<long long>(kMinChunkTc, even)));
+    }
+    chunk = std::max(least, int(share / 2.0 + 0.999) * 64);
     chunk = std::min(chunk, max_splits * 64);  // one chunk holds the longest prefix
   } else {
     // about four CTAs per SM
