@@ -52,7 +52,8 @@ using namespace sm100;
 
 constexpr int kC = 64;         // tokens per chunk
 constexpr int kD = 128;        // dk = dv handled by this kernel
-constexpr int kThreads = 256;
+constexpr int kGroup = 256;    // threads of one group (solve or state)
+constexpr int kThreads = 2 * kGroup;
 constexpr uint64_t kDrainNs = 200000000ull;
 
 // Shared memory (offsets from the 1024-byte aligned base). Operand tiles are
@@ -65,28 +66,30 @@ constexpr uint32_t kKQSlice = 3 * 8192;
 constexpr uint32_t kOffKQ = 0;
 constexpr uint32_t kOffV = 2 * kKQSlice;            // V: 64 rows x 2 dv-slices
 constexpr uint32_t kVSlice = 8192;
-// 65536 .. 131071: free (the state's hi/lo operand lives in TMEM)
 // [-W | g Q] hi, lo: MN-major (dk rows of 64 tokens), two N slices (-W, then
 // g Q) of 128 rows; the first slices hold T diag(b) and T diag(b g) until W
-constexpr uint32_t kOffWQh = 131072, kOffWQl = 163840;
+constexpr uint32_t kOffWQh = 65536, kOffWQl = 98304;
 constexpr uint32_t kWQSlice = 16384;
-// once the first state MMA has read [-W | g Q]: d^T and (d G[C-1])^T, hi and
-// lo, 128 rows (value column) x 64 tokens each
-constexpr uint32_t kOffDh = 131072, kOffDl = 147456, kOffDGh = 163840, kOffDGl = 180224;
-constexpr uint32_t kOffMh = 196608;     // (M o G) hi, lo: 64 rows (output token) x 64 tokens
-constexpr uint32_t kOffMl = 204800;
-constexpr uint32_t kOffA = 212992;      // A of the solve, 64 x 64 f32 (a_off)
-constexpr uint32_t kOffVec = 229376;    // a[64], b[64], g[64], G[C-1][64], g_{C-1}
-constexpr uint32_t kOffBar = kOffVec + 4 * 64 * 4 + 64;
-constexpr uint32_t kSmemBytes = kOffBar + 64 + 1024;
+// (M o G) hi, lo: 64 rows (output token) x 64 tokens, one pair per chunk parity
+constexpr uint32_t kOffM = 131072;
+constexpr uint32_t kMBuf = 16384, kMLo = 8192;
+constexpr uint32_t kOffA = 163840;      // A of the solve, 64 x 64 f32 (a_off)
+constexpr uint32_t kOffOut = 180224;    // a chunk's outputs [64 tokens][kD] bf16
+// a[64], b[64], g[64], then per chunk parity G[C-1][64] and g_{C-1}
+constexpr uint32_t kOffVec = 196608;
+constexpr uint32_t kOffBar = kOffVec + 5 * 64 * 4 + 64;
+constexpr uint32_t kSmemBytes = kOffBar + 128 + 1024;
 static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
 
-// TMEM columns: [K; Q] K^T at 0 (64), X = [d^T | O^T] at 64 (128), the state
-// at 256 (128), the state's hi and lo bf16 operand at 384 and 448 (64 each)
-constexpr uint32_t kColGM = 0, kColX = 64, kColO = 128, kColSt = 256;
+// TMEM columns: [K; Q] K^T, then W^T, at 0 (64); U^T at 64 (64); X =
+// [S0^T (-W) | O^T] at 128 (128); the state at 256 (128)
+constexpr uint32_t kColGM = 0, kColU = 64, kColX = 128, kColO = 192, kColSt = 256;
 // the state as the X MMA's A operand: bf16 pairs (dk elements 2k, 2k + 1 of
-// lane c in column k), hi then lo
+// lane c in column k), hi then lo (64 columns each); once X has read it, d^T and
+// (d G[C-1])^T, hi and lo (pairs of tokens, 32 columns each), as the A operands
+// of the last MMAs
 constexpr uint32_t kColS0h = 384, kColS0l = 448;
+constexpr uint32_t kColDh = 384, kColDl = 416, kColDGh = 448, kColDGl = 480;
 
 // byte offset of element (row, k) in a 128-byte swizzled K-major tile
 __device__ __forceinline__ uint32_t sw_off(int row, int k, uint32_t slice_bytes) {
@@ -148,10 +151,21 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
       : "memory");
 }
 
-// every thread waits (bounded); true when all of them saw the phase complete
-__device__ __forceinline__ bool all_wait(uint64_t* bar, uint32_t par, uint64_t ns) {
-  const bool ok = mbar_wait(bar, par, ns, nullptr);
-  return __syncthreads_and(ok) != 0;
+// barrier of one group's 256 threads (id 1: solve, 2: state)
+__device__ __forceinline__ void group_sync(uint32_t id) { named_bar_sync(id, kGroup); }
+
+// the same, returning whether `ok` holds for every thread of the group
+__device__ __forceinline__ bool group_and(uint32_t id, bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "barrier.cta.red.and.pred q, %2, %3, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(uint32_t(ok)), "r"(id), "n"(kGroup)
+      : "memory");
+  return r != 0;
 }
 
 // A[r][i] (i < r) of the solve, row-major in f32 (a float index), the 16-byte
@@ -225,7 +239,7 @@ __device__ __forceinline__ void invert_unit_lower(const float* __restrict__ A, u
 #pragma unroll
     for (int r = 0; r < 16; ++r) *t_at(sm, 16 * kb + r, 16 * ib + col) = x[r];
   }
-  __syncthreads();
+  group_sync(1);
   // then the blocks below the diagonal level by level (d = i - j = 1, 2, 3):
   // T_ij = -sum_{k=j}^{i-1} (T_ii A_ik) T_kj, one barrier a level
 #pragma unroll
@@ -254,7 +268,7 @@ __device__ __forceinline__ void invert_unit_lower(const float* __restrict__ A, u
       *reinterpret_cast<float4*>(t_at(sm, 16 * ib + r, 16 * jb + 4 * c4)) =
           make_float4(-acc.x, -acc.y, -acc.z, -acc.w);
     }
-    __syncthreads();
+    group_sync(1);
   }
 }
 
@@ -272,22 +286,34 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   float* va = reinterpret_cast<float*>(sm + kOffVec);  // a of the chunk's tokens (1 past its end)
   float* vb = va + 64;                                 // b (0 past its end)
   float* vg = vb + 64;                                 // g_r = a_0 ... a_r
-  float* vgc = vg + 64;                                // G[C-1][i]
-  float* gC = vgc + 64;                                // g_{C-1}
+  float* vgc2 = vg + 64;                               // [2][64]: G[C-1][i], by chunk parity
+  float* gC2 = vgc2 + 128;                             // [2]: g_{C-1}
   float* Am = reinterpret_cast<float*>(sm + kOffA);
-  // the chunk's outputs [64 tokens][kD] bf16, staged in the A buffer
-  __nv_bfloat16* ost = reinterpret_cast<__nv_bfloat16*>(sm + kOffA);
+  __nv_bfloat16* ost = reinterpret_cast<__nv_bfloat16*>(sm + kOffOut);
   uint64_t* bar_k = reinterpret_cast<uint64_t*>(sm + kOffBar);  // K buffers 0 and 1
   uint64_t* bar_q = bar_k + 2;
   uint64_t* bar_v = bar_k + 3;
-  uint64_t* bar_mma = bar_k + 4;
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar_k + 5);
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int grp = tid >> 7;   // warpgroup
+  uint64_t* bar_a = bar_k + 4;    // the solve group's MMAs
+  uint64_t* bar_x = bar_k + 5;    // X of a chunk is done: [-W | g Q] may be replaced
+  uint64_t* bar_so = bar_k + 6;   // the state and output MMAs of a chunk
+  uint64_t* ready = bar_k + 7;    // a chunk's U, [-W | g Q] and M o G are ready
+  uint64_t* u_free = bar_k + 8;   // a chunk's U has been read
+  uint64_t* drain = bar_k + 9;    // [2]
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 2);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int role = warp >> 3;             // 0: solve, 1: state
+  const int tid = threadIdx.x & (kGroup - 1);  // within the group
+  const int grp = tid >> 7;   // warpgroup of the group
   const int c = tid & 127;    // TMEM lane: value column c (and key column c of W)
   const int h = blockIdx.x, r = blockIdx.y;
-  if (tid == 0) {
-    for (int b = 0; b < 5; ++b) mbar_init(bar_k + b, 1);
+  if (threadIdx.x == 0) {
+    for (int b = 0; b < 7; ++b) mbar_init(bar_k + b, 1);
+    mbar_init(ready, kGroup / 32);
+    mbar_init(u_free, kGroup / 32);
+    mbar_init(drain, 1);
+    mbar_init(drain + 1, 1);
+    *abort_flag = 0;
     fence_barrier_init();
     tma_prefetch_desc(&tmQ);
     tma_prefetch_desc(&tmK);
@@ -309,430 +335,445 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     p1 = prefix_offset[r + 1];
   }
   if (r >= R || p0 < 0 || p1 < p0 || p1 > total) {
-    if (tid == 0) flag(status, JET_ERR_DEVICE);
+    if (threadIdx.x == 0) flag(status, JET_ERR_DEVICE);
     p1 = p0 = 0;
   }
   const int nch = (p1 - p0 + kC - 1) / kC;
   const size_t head = (size_t(r) * Hl + h) * kD;  // row 0 of this (request, head)'s state
   const uint64_t pol = policy_evict_first();
 
-  // TMA copies of chunk j's K (into buffer j & 1), Q and V, issued by thread 0;
-  // `pend` marks the barriers with a copy in flight (bits 0, 1: K buffers, 2:
-  // Q, 3: V)
-  uint32_t pend = 0;
+  // TMA copies of chunk j's K (into buffer j & 1), Q and V. K of the first two
+  // chunks, Q and V are issued by the solve group's thread 0, later K by the
+  // state group's. `pend` / `par` remember the barriers this thread armed (bits
+  // 0, 1: K buffers, 2: Q, 3: V) and the parity of their last phase, for the
+  // wait after an abort.
+  uint32_t pend = 0, par = 0;
+  auto armed = [&](int bit, int phase) {
+    pend |= 1u << bit;
+    par = (par & ~(1u << bit)) | (uint32_t(phase & 1) << bit);
+  };
   auto load_k = [&](int j) {
     uint64_t* b = bar_k + (j & 1);
     mbar_arrive_expect_tx(b, 2 * 8192);
     for (int sl = 0; sl < 2; ++sl)
       tma_load_3d(sm + kOffKQ + sl * kKQSlice + (j & 1) * 16384, &tmK, b, sl * 64, h,
                   p0 + j * kC, pol);
-    pend |= 1u << (j & 1);
+    armed(j & 1, j >> 1);
   };
   auto load_q = [&](int j) {
     mbar_arrive_expect_tx(bar_q, 2 * 8192);
     for (int sl = 0; sl < 2; ++sl)
       tma_load_3d(sm + kOffKQ + sl * kKQSlice + 8192, &tmQ, bar_q, sl * 64, h, p0 + j * kC, pol);
-    pend |= 4u;
+    armed(2, j);
   };
   auto load_v = [&](int j) {
     mbar_arrive_expect_tx(bar_v, 2 * 8192);
     for (int sl = 0; sl < 2; ++sl)
       tma_load_3d(sm + kOffV + sl * kVSlice, &tmV, bar_v, sl * 64, h, p0 + j * kC, pol);
-    pend |= 8u;
+    armed(3, j);
   };
-  if (tid == 0 && nch > 0 && !hold_first) {
-    load_k(0);
-    load_q(0);
-    load_v(0);
-    if (nch > 1) load_k(1);
-  }
-  // the gates of the first chunk (thread t < 64: token t of the chunk)
-  float na = 1.f, nb = 0.f;
-  if (tid < kC && p0 + tid < p1) {
-    na = alpha[size_t(p0 + tid) * Hl + h];
-    nb = beta[size_t(p0 + tid) * Hl + h];
-  }
-
-  // the initial state: into TMEM (lane c holds S0^T[c][.] = S0[.][c]; this
-  // warpgroup's 64 columns) and as the bf16 hi/lo operand of the first state MMA
-  for (int i0 = 64 * grp; i0 < 64 * grp + 64; i0 += 32) {
-    float v[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = s_init ? s_init[(head + i0 + i) * kD + c] : 0.f;
-    tmem_st_32cols(tmem + lane_off + kColSt + i0, v);
-    put32_tmem(tmem + lane_off + kColS0h + (i0 >> 1), tmem + lane_off + kColS0l + (i0 >> 1), v);
-  }
-  tmem_wait_st();
-  fence_proxy_async_shared();
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-
-  const float rs = rsqrtf(float(kD));
-  uint32_t kph = 0, qph = 0, vph = 0, mph = 0;  // kph: bit b = parity of K buffer b
   bool ok = true;
-  for (int j = 0; ok && j < nch; ++j) {
-    const int c0 = p0 + j * kC;
-    const int n = min(kC, p1 - c0);
-    const bool last = j + 1 == nch;
-    const int odd = j & 1;
-    uint8_t* const kt = sm + kOffKQ + odd * 16384;  // this chunk's K (dk-slices kKQSlice apart)
-    // ---- gates and decay products
-    if (tid < kC) {
-      va[tid] = na;
-      vb[tid] = nb;
+
+  if (role == 0) {
+    // ================================================================ solve
+    if (tid == 0 && nch > 0 && !hold_first) {
+      load_k(0);
+      load_q(0);
+      load_v(0);
+      if (nch > 1) load_k(1);
     }
-    __syncthreads();
-    if (tid < kC && !last) {
-      const int t = c0 + kC + tid;
-      na = t < p1 ? alpha[size_t(t) * Hl + h] : 1.f;
-      nb = t < p1 ? beta[size_t(t) * Hl + h] : 0.f;
+    // the gates of the first chunk (thread t < 64: token t of the chunk)
+    float na = 1.f, nb = 0.f;
+    if (tid < kC && p0 + tid < p1) {
+      na = alpha[size_t(p0 + tid) * Hl + h];
+      nb = beta[size_t(p0 + tid) * Hl + h];
     }
-    // row rr (first warpgroup): G[rr][i] = a_{i+1} .. a_rr (i <= rr), g_rr
-    const int rr = tid & 63;
-    float gam[kC];
-    if (grp == 0) {
-      float g = 1.f;
-#pragma unroll
-      for (int i = kC - 1; i >= 0; --i) {
-        gam[i] = i <= rr ? g : 0.f;
-        if (i <= rr) g *= va[i];
+    uint32_t aph = 0;
+    for (int j = 0; j < nch; ++j) {
+      const int c0 = p0 + j * kC;
+      const bool last = j + 1 == nch;
+      const int odd = j & 1;
+      uint8_t* const kt = sm + kOffKQ + odd * 16384;  // this chunk's K (dk-slices kKQSlice apart)
+      uint8_t* const mt = sm + kOffM + odd * kMBuf;   // this chunk's M o G
+      // ---- gates and decay products: g_t = a_0 .. a_t and G[C-1][t] =
+      // a_{t+1} .. a_63 by scans over two warps (each multiplies in the other's
+      // half)
+      float gsuf = 1.f, gtot = 1.f;
+      if (tid < kC) {
+        va[tid] = na;
+        vb[tid] = nb;
       }
-      if (tid < kC) vg[rr] = g;
-      if (tid == kC - 1) {
-        *gC = g;
+      group_sync(1);
+      if (tid < kC) {
+        const float other = va[tid ^ 32];
+        float pre = na, suf = na, all = other;
 #pragma unroll
-        for (int i = 0; i < kC; ++i) vgc[i] = gam[i];
-      }
-    }
-    {
-      const bool okk = mbar_wait(bar_k + odd, (kph >> odd) & 1u, wait_ns, nullptr) &&
-                       mbar_wait(bar_q, qph, wait_ns, nullptr);
-      ok = __syncthreads_and(okk) != 0;
-    }
-    if (!ok) break;
-    kph ^= 1u << odd;
-    qph ^= 1u;
-    if (tid == 0) pend &= ~((1u << odd) | 4u);
-    // ---- [K; Q] K^T (even chunks) or [Q; K] K^T (odd): k.k and q.k in float32
-    if (warp == 0 && elect_one()) {
-      tc_fence_after();
-#pragma unroll
-      for (int st = 0; st < 8; ++st) {
-        const uint32_t sl = (st >> 2) * kKQSlice + 32 * (st & 3);
-        const uint32_t a = smem_u32(sm + kOffKQ + (odd ? 8192 : 0)) + sl;
-        const uint32_t b = smem_u32(kt) + sl;
-        mma_f16(tmem + kColGM, desc_k_sw128(a), desc_k_sw128(b), idesc_bf16_f32(128, 64), st != 0);
-      }
-      mma_commit(bar_mma);
-    }
-    ok = all_wait(bar_mma, mph, wait_ns);
-    if (!ok) break;
-    mph ^= 1u;
-    tc_fence_after();
-    // ---- the solve's matrix A (k rows) and M o G (q rows) from the first
-    // warpgroup's TMEM lanes; g Q from the second warpgroup
-    if (grp == 0) {
-      // 32 columns of [K; Q] K^T at a time
-#pragma unroll
-      for (int hf = 0; hf < 2; ++hf) {
-        float gr[32];
-        tmem_ld_32cols(tmem + lane_off + kColGM + 32 * hf, gr);
-        tmem_wait_ld();
-        if ((tid >> 6) == odd) {
-          // k row rr: A[rr][i] = b_rr G[rr][i] (k_rr . k_i), i < rr (the
-          // entries from rr on are never read)
-          if (DELTA) {
-            const float b = vb[rr];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              const int i = 32 * hf + 4 * q;
-              float4 w;
-              w.x = i + 0 < rr ? b * gam[i + 0] * gr[4 * q + 0] : 0.f;
-              w.y = i + 1 < rr ? b * gam[i + 1] * gr[4 * q + 1] : 0.f;
-              w.z = i + 2 < rr ? b * gam[i + 2] * gr[4 * q + 2] : 0.f;
-              w.w = i + 3 < rr ? b * gam[i + 3] * gr[4 * q + 3] : 0.f;
-              *reinterpret_cast<float4*>(Am + a_off(rr, 8 * hf + q)) = w;
-            }
-          }
-        } else {
-          // q row rr: (M o G)[rr][i] = (q_rr . k_i) G[rr][i], i <= rr
-          float m[32];
-#pragma unroll
-          for (int i = 0; i < 32; ++i) m[i] = gam[32 * hf + i] * gr[i];  // gam = 0 past rr
-#pragma unroll
-          for (int jj = 0; jj < 4; ++jj)
-            put8(sm + kOffMh, sm + kOffMl, rr, 4 * hf + jj, m + 8 * jj);
+        for (int d = 1; d < 32; d <<= 1) {
+          const float x = __shfl_up_sync(0xffffffffu, pre, d);
+          if (lane >= d) pre *= x;
+          const float y = __shfl_down_sync(0xffffffffu, suf, d);
+          if (lane + d < 32) suf *= y;
+          all *= __shfl_xor_sync(0xffffffffu, all, d);
+        }
+        suf = __shfl_down_sync(0xffffffffu, suf, 1);  // a_{t+1} .. of this warp
+        if (lane == 31) suf = 1.f;
+        gtot = tid >= 32 ? all * pre : pre;
+        gsuf = tid < 32 ? suf * all : suf;
+        vg[tid] = gtot;
+        if (!last) {
+          const int t = c0 + kC + tid;
+          na = t < p1 ? alpha[size_t(t) * Hl + h] : 1.f;
+          nb = t < p1 ? beta[size_t(t) * Hl + h] : 0.f;
         }
       }
-    } else {
-      // g Q as rows 64 .. 127 (the second N slice) of the MN-major [-W | g Q]
-      // operand: thread c writes dk row c, the chunk's 64 tokens contiguous
-      const uint8_t* qt = sm + kOffKQ + 8192;
-      float x[kC];
+      ok = group_and(1, mbar_wait(bar_k + odd, (j >> 1) & 1, wait_ns, abort_flag) &&
+                            mbar_wait(bar_q, j & 1, wait_ns, abort_flag));
+      if (!ok) break;
+      // K of this chunk came after the state group was done with the chunk
+      // before last: its parity's M o G and decays may be replaced
+      if (tid < kC) vgc2[odd * 64 + tid] = gsuf;
+      if (tid == kC - 1) gC2[odd] = gtot;
+      // ---- [K; Q] K^T (even chunks) or [Q; K] K^T (odd): k.k and q.k in float32
+      if (warp == 0 && elect_one()) {
+        tc_fence_after();
 #pragma unroll
-      for (int t = 0; t < kC; ++t) x[t] = vg[t] * bf(qt, sw_off(t, c, kKQSlice));
-#pragma unroll
-      for (int jj = 0; jj < 8; ++jj)
-        put8(sm + kOffWQh + kWQSlice, sm + kOffWQl + kWQSlice, c, jj, x + 8 * jj);
-      if (DELTA) {
-        // O^T starts from zero under the first state MMA's accumulation
-        float z[32];
-#pragma unroll
-        for (int i = 0; i < 32; ++i) z[i] = 0.f;
-        tmem_st_32cols(tmem + lane_off + kColO, z);
-        tmem_st_32cols(tmem + lane_off + kColO + 32, z);
+        for (int st = 0; st < 8; ++st) {
+          const uint32_t sl = (st >> 2) * kKQSlice + 32 * (st & 3);
+          const uint32_t a = smem_u32(sm + kOffKQ + (odd ? 8192 : 0)) + sl;
+          const uint32_t b = smem_u32(kt) + sl;
+          mma_f16(tmem + kColGM, desc_k_sw128(a), desc_k_sw128(b), idesc_bf16_f32(128, 64),
+                  st != 0);
+        }
+        mma_commit(bar_a);
       }
-    }
-    tmem_wait_st();
-    fence_proxy_async_shared();
-    tc_fence_before();
-    __syncthreads();
-    if (DELTA) {
-      // ---- T = (I + A)^{-1}, then T' = T diag(b) and T'' = T diag(b g) as
-      // the hi/lo B operands (row r, 64 tokens i, K-major) of U = T' V and
-      // W = T'' K, in the first N slice of the [-W | g Q] tiles (free until W)
-      invert_unit_lower(Am, sm, tid);
-      {
-        const int row = tid >> 2;
+      __syncwarp();
+      bool okk = true;
+      if (grp == 1) {
+        // g Q as rows 64 .. 127 (the second N slice) of the MN-major [-W | g Q]
+        // operand: thread c writes dk row c, the chunk's 64 tokens contiguous -
+        // once the previous chunk's X has read it
+        okk = j == 0 || mbar_wait(bar_x, (j - 1) & 1, wait_ns, abort_flag);
+        if (okk) {
+          const uint8_t* qt = sm + kOffKQ + 8192;
 #pragma unroll
-        for (int h2 = 0; h2 < 2; ++h2) {
-          const int jj = 2 * (tid & 3) + h2;
-          float x1[8], x2[8];
-          const float4 t0 = *reinterpret_cast<const float4*>(t_at(sm, row, 8 * jj));
-          const float4 t1 = *reinterpret_cast<const float4*>(t_at(sm, row, 8 * jj + 4));
-          const float tv[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+          for (int jj = 0; jj < 8; ++jj) {
+            float x[8];
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const int i = 8 * jj + e;
-            const float t = i <= row ? tv[e] : 0.f;
-            x1[e] = t * vb[i];
-            x2[e] = x1[e] * vg[i];
+            for (int e = 0; e < 8; ++e)
+              x[e] = vg[8 * jj + e] * bf(qt, sw_off(8 * jj + e, c, kKQSlice));
+            put8(sm + kOffWQh + kWQSlice, sm + kOffWQl + kWQSlice, c, jj, x);
           }
-          put8(sm + kOffWQh, sm + kOffWQl, row, jj, x1);
-          put8(sm + kOffWQh + 8192, sm + kOffWQl + 8192, row, jj, x2);
+        }
+      }
+      okk = okk && mbar_wait(bar_a, aph, wait_ns, abort_flag);
+      aph ^= 1u;
+      tc_fence_after();
+      // ---- the solve's matrix A (k rows) and M o G (q rows) from the first
+      // warpgroup's TMEM lanes, 32 columns of [K; Q] K^T at a time from the right
+      // (the decay G[rr][i] = a_{i+1} .. a_rr grows leftwards)
+      if (okk && grp == 0) {
+        const int rr = tid & 63;
+        const bool krow = (tid >> 6) == odd;
+        float g = 1.f;
+#pragma unroll
+        for (int hf = 1; hf >= 0; --hf) {
+          float gr[32];
+          tmem_ld_32cols(tmem + lane_off + kColGM + 32 * hf, gr);
+          tmem_wait_ld();
+          if (krow && !DELTA) continue;
+          const float b = vb[rr];
+#pragma unroll
+          for (int i = 31; i >= 0; --i) {
+            const int col = 32 * hf + i;
+            const float gam = col <= rr ? g : 0.f;
+            if (col <= rr) g *= va[col];
+            // k row rr: A[rr][i] = b_rr G[rr][i] (k_rr . k_i), i < rr (the
+            // entries from rr on are never read); q row rr: (M o G)[rr][i] =
+            // (q_rr . k_i) G[rr][i], i <= rr
+            gr[i] = krow ? (col < rr ? b * gam * gr[i] : 0.f) : gam * gr[i];
+          }
+          if (krow) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+              *reinterpret_cast<float4*>(Am + a_off(rr, 8 * hf + q)) =
+                  make_float4(gr[4 * q], gr[4 * q + 1], gr[4 * q + 2], gr[4 * q + 3]);
+          } else {
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj)
+              put8(mt, mt + kMLo, rr, 4 * hf + jj, gr + 8 * jj);
+          }
         }
       }
       fence_proxy_async_shared();
       tc_fence_before();
-      __syncthreads();
-    }
-    // Q (and T in its slots) is no longer read: the next chunk's Q may land
-    if (tid == 0 && !last) load_q(j + 1);
-    ok = all_wait(bar_v, vph, wait_ns);
-    if (!ok) break;
-    vph ^= 1u;
-    if (tid == 0) pend &= ~8u;
-    if (DELTA) {
-      // ---- U^T = V^T T'^T (TMEM at X, for the first state MMA to accumulate
-      // onto) and W^T = K^T T''^T: V and K are MN-major A operands (exact in
-      // bf16), T' and T'' enter as hi + lo
-      if (warp == 0 && elect_one()) {
-        tc_fence_after();
-        const uint32_t idesc = idesc_bf16_f32(128, 64) | (1u << 15);
+      ok = group_and(1, okk);
+      if (!ok) break;
+      if (DELTA) {
+        // ---- T = (I + A)^{-1}, then T' = T diag(b) and T'' = T diag(b g) as
+        // the hi/lo B operands (row r, 64 tokens i, K-major) of U = T' V and
+        // W = T'' K, in the first N slice of the [-W | g Q] tiles (free until W)
+        invert_unit_lower(Am, sm, tid);
+        {
+          const int row = tid >> 2;
 #pragma unroll
-        for (int pass = 0; pass < 2; ++pass) {
-          const uint32_t b = smem_u32(sm + (pass ? kOffWQl : kOffWQh));
+          for (int h2 = 0; h2 < 2; ++h2) {
+            const int jj = 2 * (tid & 3) + h2;
+            float x1[8], x2[8];
+            const float4 t0 = *reinterpret_cast<const float4*>(t_at(sm, row, 8 * jj));
+            const float4 t1 = *reinterpret_cast<const float4*>(t_at(sm, row, 8 * jj + 4));
+            const float tv[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            mma_f16(tmem + kColX, desc_mn_sw128(smem_u32(sm + kOffV) + k * 2048, kVSlice),
-                    desc_k_sw128(b + 32 * k), idesc, (pass | k) != 0);
-            mma_f16(tmem + kColGM, desc_mn_sw128(smem_u32(kt) + k * 2048, kKQSlice),
-                    desc_k_sw128(b + 8192 + 32 * k), idesc, (pass | k) != 0);
+            for (int e = 0; e < 8; ++e) {
+              const int i = 8 * jj + e;
+              const float t = i <= row ? tv[e] : 0.f;
+              x1[e] = t * vb[i];
+              x2[e] = x1[e] * vg[i];
+            }
+            put8(sm + kOffWQh, sm + kOffWQl, row, jj, x1);
+            put8(sm + kOffWQh + 8192, sm + kOffWQl + 8192, row, jj, x2);
           }
         }
-        mma_commit(bar_mma);
+        fence_proxy_async_shared();
+        tc_fence_before();
+        group_sync(1);
       }
-      ok = all_wait(bar_mma, mph, wait_ns);
-      if (!ok) break;
-      mph ^= 1u;
-      tc_fence_after();
-      // -W as the first N slice of [-W | g Q]: thread c writes key row c
-      if (grp == 1) {
+      // Q (and T in its slots) is no longer read: the next chunk's Q may land
+      if (tid == 0 && !last) load_q(j + 1);
+      okk = mbar_wait(bar_v, j & 1, wait_ns, abort_flag) &&
+            (j == 0 || mbar_wait(u_free, (j - 1) & 1, wait_ns, abort_flag));
+      if (DELTA) {
+        // ---- U^T = V^T T'^T and W^T = K^T T''^T: V and K are MN-major A
+        // operands (exact in bf16), T' and T'' enter as hi + lo
+        ok = group_and(1, okk);
+        if (!ok) break;
+        if (warp == 0 && elect_one()) {
+          tc_fence_after();
+          const uint32_t idesc = idesc_bf16_f32(128, 64) | (1u << 15);
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
+          for (int pass = 0; pass < 2; ++pass) {
+            const uint32_t b = smem_u32(sm + (pass ? kOffWQl : kOffWQh));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              mma_f16(tmem + kColU, desc_mn_sw128(smem_u32(sm + kOffV) + k * 2048, kVSlice),
+                      desc_k_sw128(b + 32 * k), idesc, (pass | k) != 0);
+              mma_f16(tmem + kColGM, desc_mn_sw128(smem_u32(kt) + k * 2048, kKQSlice),
+                      desc_k_sw128(b + 8192 + 32 * k), idesc, (pass | k) != 0);
+            }
+          }
+          mma_commit(bar_a);
+        }
+        __syncwarp();
+        okk = mbar_wait(bar_a, aph, wait_ns, abort_flag);
+        aph ^= 1u;
+        tc_fence_after();
+        // -W as the first N slice of [-W | g Q]: thread c writes key row c, each
+        // warpgroup half of the tokens
+        if (okk) {
           float wv[32];
-          tmem_ld_32cols(tmem + lane_off + kColGM + 32 * hf, wv);
+          tmem_ld_32cols(tmem + lane_off + kColGM + 32 * grp, wv);
           tmem_wait_ld();
 #pragma unroll
           for (int i = 0; i < 32; ++i) wv[i] = -wv[i];
 #pragma unroll
           for (int jj = 0; jj < 4; ++jj)
-            put8(sm + kOffWQh, sm + kOffWQl, c, 4 * hf + jj, wv + 8 * jj);
+            put8(sm + kOffWQh, sm + kOffWQl, c, 4 * grp + jj, wv + 8 * jj);
         }
-      }
-    } else if (grp == 0) {
-      // gated linear attention: U = diag(b) V straight into TMEM
-      const uint8_t* vt = sm + kOffV;
-#pragma unroll
-      for (int i0 = 0; i0 < kC; i0 += 32) {
+      } else if (okk) {
+        // gated linear attention: U = diag(b) V straight into TMEM
+        tc_fence_after();
+        const uint8_t* vt = sm + kOffV;
         float uv[32];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) uv[i] = vb[i0 + i] * bf(vt, sw_off(i0 + i, c, kVSlice));
-        tmem_st_32cols(tmem + lane_off + kColX + i0, uv);
-      }
-      tmem_wait_st();
-    }
-    fence_proxy_async_shared();
-    tc_fence_before();
-    __syncthreads();
-    // V is no longer read
-    if (tid == 0 && !last) load_v(j + 1);
-    // ---- X = U^T + S0^T [-W | g Q] (delta rule) or O^T = S0^T (g Q)
-    // (gated linear attention, X = U^T as stored): three hi/lo passes; the B
-    // operand is MN-major (dk rows of 128 tokens)
-    if (warp == 0 && elect_one()) {
-      tc_fence_after();
-#pragma unroll
-      for (int pass = 0; pass < 3; ++pass) {
-        // A (the state, K = dk) from TMEM: 8 packed columns per K = 16 step
-        const uint32_t a = tmem + (pass == 2 ? kColS0l : kColS0h);
-        const uint32_t b = smem_u32(sm + (pass == 1 ? kOffWQl : kOffWQh));
-#pragma unroll
-        for (int st = 0; st < 8; ++st) {
-          if (DELTA)
-            mma_f16_ta(tmem + kColX, a + 8 * st, desc_mn_sw128(b + st * 2048, kWQSlice),
-                       idesc_bf16_f32(128, 128) | (1u << 16), 1u);
-          else
-            mma_f16_ta(tmem + kColO, a + 8 * st, desc_mn_sw128(b + kWQSlice + st * 2048, kWQSlice),
-                       idesc_bf16_f32(128, 64) | (1u << 16), (pass | st) != 0);
-        }
-      }
-      mma_commit(bar_mma);
-    }
-    ok = all_wait(bar_mma, mph, wait_ns);
-    if (!ok) break;
-    mph ^= 1u;
-    tc_fence_after();
-    // ---- d (column c of d is row c of d^T): the first warpgroup writes d^T,
-    // the second (d G[C-1])^T, as the second MMA group's A operands; each
-    // scales its 64 state columns by g_{C-1} in TMEM for the last MMA to
-    // accumulate onto
-    {
-#pragma unroll
-      for (int hf = 0; hf < 2; ++hf) {
-        float dr[32];
-        tmem_ld_32cols(tmem + lane_off + kColX + 32 * hf, dr);
-        tmem_wait_ld();
-        if (grp == 0) {
-#pragma unroll
-          for (int jj = 0; jj < 4; ++jj) put8(sm + kOffDh, sm + kOffDl, c, 4 * hf + jj, dr + 8 * jj);
-        } else {
-#pragma unroll
-          for (int jj = 0; jj < 4; ++jj) {
-            float dg[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) dg[e] = dr[8 * jj + e] * vgc[32 * hf + 8 * jj + e];
-            put8(sm + kOffDGh, sm + kOffDGl, c, 4 * hf + jj, dg);
-          }
-        }
-      }
-      const float g = *gC;
-      const uint32_t scol = tmem + lane_off + kColSt + 64 * grp;
-      float s0[32], s1[32];
-      tmem_ld_32cols(scol, s0);
-      tmem_ld_32cols(scol + 32, s1);
-      tmem_wait_ld();
-#pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        s0[i] *= g;
-        s1[i] *= g;
-      }
-      tmem_st_32cols(scol, s0);
-      tmem_st_32cols(scol + 32, s1);
-      tmem_wait_st();
-    }
-    fence_proxy_async_shared();
-    tc_fence_before();
-    __syncthreads();
-    // ---- O^T += d^T (M o G)^T (three passes); state^T += (d G[C-1])^T K (two:
-    // K is exact in bf16)
-    if (warp == 0 && elect_one()) {
-      tc_fence_after();
-#pragma unroll
-      for (int pass = 0; pass < 3; ++pass) {
-        const uint32_t a = smem_u32(sm + (pass == 2 ? kOffDl : kOffDh));
-        const uint32_t b = smem_u32(sm + (pass == 1 ? kOffMl : kOffMh));
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          mma_f16(tmem + kColO, desc_k_sw128(a + 32 * k), desc_k_sw128(b + 32 * k),
-                  idesc_bf16_f32(128, 64), 1u);
-      }
-#pragma unroll
-      for (int pass = 0; pass < 2; ++pass) {
-        const uint32_t a = smem_u32(sm + (pass == 1 ? kOffDGl : kOffDGh));
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          mma_f16(tmem + kColSt, desc_k_sw128(a + 32 * k),
-                  desc_mn_sw128(smem_u32(kt) + k * 16 * 128, kKQSlice),
-                  idesc_bf16_f32(128, 128) | (1u << 16), 1u);
-      }
-      mma_commit(bar_mma);
-    }
-    ok = all_wait(bar_mma, mph, wait_ns);
-    if (!ok) break;
-    mph ^= 1u;
-    tc_fence_after();
-    // this chunk's K is no longer read: the chunk after next may land there
-    if (tid == 0 && j + 2 < nch) load_k(j + 2);
-    // ---- outputs of the chunk's tokens (warpgroup g: tokens 32 g ..), and this
-    // warpgroup's 64 columns of the new state as the next chunk's operand (and,
-    // after the last chunk, the result)
-    {
-      float ov[32];
-      tmem_ld_32cols(tmem + lane_off + kColO + 32 * grp, ov);
-      const uint32_t scol = tmem + lane_off + kColSt + 64 * grp;
-      float s0[32], s1[32];
-      tmem_ld_32cols(scol, s0);
-      tmem_ld_32cols(scol + 32, s1);
-      tmem_wait_ld();
-      // the chunk's outputs through the solve's A buffer (free until the next
-      // chunk), [token][value] as they are stored, for 16-byte global stores
-#pragma unroll
-      for (int i = 0; i < 32; ++i) ost[(32 * grp + i) * kD + c] = __float2bfloat16_rn(ov[i] * rs);
-      if (last) {
-        const size_t row0 = head + 64 * grp;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          s_out[(row0 + i) * kD + c] = s0[i];
-          s_out[(row0 + 32 + i) * kD + c] = s1[i];
-        }
-      } else {
-        // this warpgroup's 64 dk columns: packed columns 32 grp .. 32 grp + 31
-        put32_tmem(tmem + lane_off + kColS0h + 32 * grp, tmem + lane_off + kColS0l + 32 * grp, s0);
-        put32_tmem(tmem + lane_off + kColS0h + 32 * grp + 16,
-                   tmem + lane_off + kColS0l + 32 * grp + 16, s1);
+        for (int i = 0; i < 32; ++i) uv[i] = vb[32 * grp + i] * bf(vt, sw_off(32 * grp + i, c, kVSlice));
+        tmem_st_32cols(tmem + lane_off + kColU + 32 * grp, uv);
         tmem_wait_st();
       }
+      fence_proxy_async_shared();
+      tc_fence_before();
+      ok = group_and(1, okk);
+      if (!ok) break;
+      if (lane == 0) mbar_arrive(ready);
+      // V is no longer read
+      if (tid == 0 && !last) load_v(j + 1);
     }
-    fence_proxy_async_shared();
+  } else {
+    // ================================================================ state
+    // the initial state: into TMEM (lane c holds S0^T[c][.] = S0[.][c]; this
+    // warpgroup's 64 columns) and as the bf16 hi/lo operand of the first X
+    for (int i0 = 64 * grp; i0 < 64 * grp + 64; i0 += 32) {
+      float v[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) v[i] = s_init ? s_init[(head + i0 + i) * kD + c] : 0.f;
+      tmem_st_32cols(tmem + lane_off + kColSt + i0, v);
+      put32_tmem(tmem + lane_off + kColS0h + (i0 >> 1), tmem + lane_off + kColS0l + (i0 >> 1), v);
+    }
+    tmem_wait_st();
     tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    // each token's 128 outputs are 256 contiguous bytes of o (the next
-    // chunk's first barrier comes before its A lands in the buffer)
-    for (int e = tid; e < n * (kD / 8); e += kThreads) {
-      const int t = e / (kD / 8), q = e % (kD / 8);
-      *reinterpret_cast<uint4*>(o + (size_t(c0 + t) * Hl + h) * kD + 8 * q) =
-          reinterpret_cast<const uint4*>(ost)[e];
+    group_sync(2);
+    const float rs = rsqrtf(float(kD));
+    for (int j = 0; j < nch; ++j) {
+      const int c0 = p0 + j * kC;
+      const int n = min(kC, p1 - c0);
+      const bool last = j + 1 == nch;
+      const int odd = j & 1;
+      uint8_t* const kt = sm + kOffKQ + odd * 16384;
+      uint8_t* const mt = sm + kOffM + odd * kMBuf;
+      ok = group_and(2, mbar_wait(ready, j & 1, wait_ns, abort_flag));
+      if (!ok) break;
+      // ---- X = S0^T [-W | g Q] (delta rule) or O^T = S0^T (g Q) (gated linear
+      // attention): three hi/lo passes; A (the state, K = dk) from TMEM, 8 packed
+      // columns per K = 16 step; the B operand is MN-major (dk rows of 128 tokens)
+      if (warp == 8 && elect_one()) {
+        tc_fence_after();
+#pragma unroll
+        for (int pass = 0; pass < 3; ++pass) {
+          const uint32_t a = tmem + (pass == 2 ? kColS0l : kColS0h);
+          const uint32_t b = smem_u32(sm + (pass == 1 ? kOffWQl : kOffWQh));
+#pragma unroll
+          for (int st = 0; st < 8; ++st) {
+            if (DELTA)
+              mma_f16_ta(tmem + kColX, a + 8 * st, desc_mn_sw128(b + st * 2048, kWQSlice),
+                         idesc_bf16_f32(128, 128) | (1u << 16), (pass | st) != 0);
+            else
+              mma_f16_ta(tmem + kColO, a + 8 * st, desc_mn_sw128(b + kWQSlice + st * 2048, kWQSlice),
+                         idesc_bf16_f32(128, 64) | (1u << 16), (pass | st) != 0);
+          }
+        }
+        mma_commit(bar_x);
+      }
+      __syncwarp();
+      // this warpgroup's 64 state columns, scaled by g_{C-1} for the last MMA to
+      // accumulate onto (X reads the hi/lo copy, not these)
+      const float g = gC2[odd];
+      const uint32_t scol = tmem + lane_off + kColSt + 64 * grp;
+      {
+        float s0[32];
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          tmem_ld_32cols(scol + 32 * hf, s0);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 32; ++i) s0[i] *= g;
+          tmem_st_32cols(scol + 32 * hf, s0);
+        }
+      }
+      const bool okx = mbar_wait(bar_x, j & 1, wait_ns, abort_flag);
+      tc_fence_after();
+      // ---- d = U + X (column c of d is row c of d^T): the first warpgroup
+      // writes d^T, the second (d G[C-1])^T, as bf16 hi/lo A operands in TMEM
+      // over the old state's (X has read it)
+      if (okx) {
+        const float* vgc = vgc2 + odd * 64;
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          float dr[32];
+          tmem_ld_32cols(tmem + lane_off + kColU + 32 * hf, dr);
+          if (DELTA) {
+            float xr[32];
+            tmem_ld_32cols(tmem + lane_off + kColX + 32 * hf, xr);
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 32; ++i) dr[i] += xr[i];
+          } else {
+            tmem_wait_ld();
+          }
+          if (grp == 1) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) dr[i] *= vgc[32 * hf + i];
+          }
+          put32_tmem(tmem + lane_off + (grp ? kColDGh : kColDh) + 16 * hf,
+                     tmem + lane_off + (grp ? kColDGl : kColDl) + 16 * hf, dr);
+        }
+      }
+      tmem_wait_st();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(u_free);
+      ok = group_and(2, okx);
+      if (!ok) break;
+      // ---- O^T += d^T (M o G)^T (three passes); state^T += (d G[C-1])^T K (two:
+      // K is exact in bf16)
+      if (warp == 8 && elect_one()) {
+        tc_fence_after();
+#pragma unroll
+        for (int pass = 0; pass < 3; ++pass) {
+          const uint32_t a = tmem + (pass == 2 ? kColDl : kColDh);
+          const uint32_t b = smem_u32(mt + (pass == 1 ? kMLo : 0));
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            mma_f16_ta(tmem + kColO, a + 8 * k, desc_k_sw128(b + 32 * k), idesc_bf16_f32(128, 64),
+                       1u);
+        }
+#pragma unroll
+        for (int pass = 0; pass < 2; ++pass) {
+          const uint32_t a = tmem + (pass == 1 ? kColDGl : kColDGh);
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            mma_f16_ta(tmem + kColSt, a + 8 * k,
+                       desc_mn_sw128(smem_u32(kt) + k * 16 * 128, kKQSlice),
+                       idesc_bf16_f32(128, 128) | (1u << 16), 1u);
+        }
+        mma_commit(bar_so);
+      }
+      __syncwarp();
+      ok = group_and(2, mbar_wait(bar_so, j & 1, wait_ns, abort_flag));
+      if (!ok) break;
+      tc_fence_after();
+      // this chunk's K is no longer read: the chunk after next may land there
+      if (tid == 0 && j + 2 < nch) load_k(j + 2);
+      // ---- this warpgroup's 64 columns of the new state as the next chunk's
+      // operand (after the last chunk, the result), then the chunk's outputs
+      // (tokens 32 grp ..)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        float s0[32];
+        tmem_ld_32cols(scol + 32 * hf, s0);
+        tmem_wait_ld();
+        if (last) {
+          const size_t row0 = head + 64 * grp + 32 * hf;
+#pragma unroll
+          for (int i = 0; i < 32; ++i) s_out[(row0 + i) * kD + c] = s0[i];
+        } else {
+          // packed columns 32 grp + 16 hf ..
+          put32_tmem(tmem + lane_off + kColS0h + 32 * grp + 16 * hf,
+                     tmem + lane_off + kColS0l + 32 * grp + 16 * hf, s0);
+        }
+      }
+      {
+        float ov[32];
+        tmem_ld_32cols(tmem + lane_off + kColO + 32 * grp, ov);
+        tmem_wait_ld();
+        // [token][value] as they are stored, for 16-byte global stores
+#pragma unroll
+        for (int i = 0; i < 32; ++i) ost[(32 * grp + i) * kD + c] = __float2bfloat16_rn(ov[i] * rs);
+      }
+      tmem_wait_st();
+      tc_fence_before();
+      group_sync(2);
+      // each token's 128 outputs are 256 contiguous bytes of o (the next chunk's
+      // staging comes after several of this group's barriers)
+      for (int e = tid; e < n * (kD / 8); e += kGroup) {
+        const int t = e / (kD / 8), q = e % (kD / 8);
+        *reinterpret_cast<uint4*>(o + (size_t(c0 + t) * Hl + h) * kD + 8 * q) =
+            reinterpret_cast<const uint4*>(ost)[e];
+      }
     }
   }
   if (!ok) {
     // a wait ran out: let the copies and tensor-core work already issued
     // finish before the CTA frees its TMEM and ends
+    *abort_flag = 1;
     if (tid == 0) {
       flag(status, JET_ERR_TIMEOUT);
-      for (int b = 0; b < 2; ++b)
-        if (pend & (1u << b)) mbar_wait(bar_k + b, (kph >> b) & 1u, kDrainNs, nullptr);
-      if (pend & 4u) mbar_wait(bar_q, qph, kDrainNs, nullptr);
-      if (pend & 8u) mbar_wait(bar_v, vph, kDrainNs, nullptr);
+      for (int b = 0; b < 4; ++b)
+        if (pend & (1u << b)) mbar_wait(bar_k + b, (par >> b) & 1u, kDrainNs, nullptr);
     }
     __syncwarp();
-    if (warp == 0 && elect_one()) {
-      mma_commit(bar_mma);
-      mbar_wait(bar_mma, mph, kDrainNs, nullptr);
+    if ((warp & 7) == 0 && elect_one()) {
+      mma_commit(drain + role);
+      mbar_wait(drain + role, 0, kDrainNs, nullptr);
     }
-  } else if (p1 == p0 && r < R && s_out != nullptr) {
+  } else if (p1 == p0 && r < R && s_out != nullptr && role == 1) {
     // no prefix tokens: the state is the initial one (zeros without one)
     for (int i = 64 * grp; i < 64 * grp + 64; ++i)
       s_out[(head + i) * kD + c] = s_init ? s_init[(head + i) * kD + c] : 0.f;
