@@ -59,30 +59,37 @@ constexpr uint64_t kDrainNs = 200000000ull;
 // Shared memory (offsets from the 1024-byte aligned base). Operand tiles are
 // K-major with 128-byte swizzling: 64 elements (128 bytes) per row, 8-row
 // atoms of 1024 bytes, the 128-element dimension split into two slices.
-// Each dk-slice of the token tiles holds [K buffer 0 | Q | K buffer 1] (64
-// token rows each), so [K0; Q] (even chunks) and [Q; K1] (odd chunks) are
-// 128-row operands.
-constexpr uint32_t kKQSlice = 3 * 8192;
+// Each dk-slice of the token tiles holds [K0 | Q0 | K1 | Q1] (64 token rows
+// each, buffer = chunk parity), so [K; Q] of a chunk is one 128-row operand.
+constexpr uint32_t kKQSlice = 4 * 8192;
 constexpr uint32_t kOffKQ = 0;
+constexpr uint32_t kKQBuf = 16384;                  // from one parity's K to the other's
 constexpr uint32_t kOffV = 2 * kKQSlice;            // V: 64 rows x 2 dv-slices
 constexpr uint32_t kVSlice = 8192;
 // [-W | g Q] hi, lo: MN-major (dk rows of 64 tokens), two N slices (-W, then
 // g Q) of 128 rows; the first slices hold T diag(b) and T diag(b g) until W
-constexpr uint32_t kOffWQh = 65536, kOffWQl = 98304;
+constexpr uint32_t kOffWQh = 81920, kOffWQl = 114688;
 constexpr uint32_t kWQSlice = 16384;
 // (M o G) hi, lo: 64 rows (output token) x 64 tokens, one pair per chunk parity
-constexpr uint32_t kOffM = 131072;
+constexpr uint32_t kOffM = 147456;
 constexpr uint32_t kMBuf = 16384, kMLo = 8192;
-constexpr uint32_t kOffA = 163840;      // A of the solve, 64 x 64 f32 (a_off)
-constexpr uint32_t kOffOut = 180224;    // a chunk's outputs [64 tokens][kD] bf16
-// a[64], b[64], g[64], then per chunk parity G[C-1][64] and g_{C-1}
-constexpr uint32_t kOffVec = 196608;
-constexpr uint32_t kOffBar = kOffVec + 5 * 64 * 4 + 64;
+// A of the solve and T = (I + A)^{-1}, the 16 x 16 blocks at and below the
+// diagonal in f32 (blk)
+constexpr uint32_t kBlk = 324, kPitch = 20;  // floats of a block and of its rows
+constexpr uint32_t kOffA = 180224;
+constexpr uint32_t kOffT = kOffA + 10 * kBlk * 4;
+constexpr uint32_t kOffOut = kOffT + 10 * kBlk * 4;  // a chunk's outputs [64 tokens][kD] bf16
+// the gates and their products of up to three chunks: a[64], b[64], in-warp
+// products of a[64], g[64], G[C-1][64], g_{C-1}
+constexpr uint32_t kVecFloats = 5 * 64 + 4;
+constexpr uint32_t kOffVec = kOffOut + 16384;
+constexpr uint32_t kOffBar = kOffVec + 3 * kVecFloats * 4;
 constexpr uint32_t kSmemBytes = kOffBar + 128 + 1024;
+static_assert(kOffOut % 16 == 0 && kOffVec % 16 == 0 && kOffBar % 8 == 0, "alignment");
 static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
 
-// TMEM columns: [K; Q] K^T, then W^T, at 0 (64); U^T at 64 (64); X =
-// [S0^T (-W) | O^T] at 128 (128); the state at 256 (128)
+// TMEM columns: [K; Q] K^T at 0 (64); U^T at 64 (64); X = [S0^T (-W) | O^T] at
+// 128 (128), its first half W^T before; the state at 256 (128)
 constexpr uint32_t kColGM = 0, kColU = 64, kColX = 128, kColO = 192, kColSt = 256;
 // the state as the X MMA's A operand: bf16 pairs (dk elements 2k, 2k + 1 of
 // lane c in column k), hi then lo (64 columns each); once X has read it, d^T and
@@ -151,6 +158,12 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
       : "memory");
 }
 
+// eight floats from a 16-byte aligned address
+__device__ __forceinline__ void load8(float* x, const float* p) {
+  *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(p);
+  *reinterpret_cast<float4*>(x + 4) = *reinterpret_cast<const float4*>(p + 4);
+}
+
 // barrier of one group's 256 threads (id 1: solve, 2: state)
 __device__ __forceinline__ void group_sync(uint32_t id) { named_bar_sync(id, kGroup); }
 
@@ -168,108 +181,128 @@ __device__ __forceinline__ bool group_and(uint32_t id, bool ok) {
   return r != 0;
 }
 
-// A[r][i] (i < r) of the solve, row-major in f32 (a float index), the 16-byte
-// chunks of row r permuted by r & 15 so that the rows written by consecutive
-// threads fall in different banks; readers broadcast one chunk to the warp
-__device__ __forceinline__ uint32_t a_off(int r, int chunk) {
-  return uint32_t(r) * kC + (uint32_t(chunk ^ (r & 15)) << 2);
+// Block (i, k), k <= i, of A or T: rows kPitch floats apart and blocks kBlk, so
+// that eight rows of a 16-byte column, or the same place of two blocks, fall in
+// different banks, and every offset inside a block is a constant.
+__device__ __forceinline__ float* blk(float* base, int i, int k) {
+  return base + (i * (i + 1) / 2 + k) * kBlk;
 }
 
-// T = (I + A)^{-1} (unit lower triangular) in f32, 64 floats a row, in the
-// token tiles' two 8 KB Q slots (rows 32 s .. 32 s + 31 in slice s): the Q of
-// the chunk is no longer needed when it is formed. Element (r, col): the
-// 16-byte chunks of row r permuted by r & 15, so that the rows one warp
-// reads or writes at the same columns fall in different banks.
-__device__ __forceinline__ float* t_at(uint8_t* sm, int r, int col) {
-  return reinterpret_cast<float*>(sm + kOffKQ + (r >> 5) * kKQSlice + 8192 + (r & 31) * 256 +
-                                  ((((col >> 2) ^ (r & 15)) << 4) | ((col & 3) << 2)));
-}
-
-// T in 16 x 16 blocks: the diagonal blocks T_ii by substitution (thread
-// (i, j): column j of T_ii) and, in the same step, the products T_ii A_ik
-// (k < i) by substitution too, in the unused blocks above the diagonal; then
-// the blocks below the diagonal level by level (d = i - j = 1, 2, 3):
-// T_ij = -sum_{k=j}^{i-1} (T_ii A_ik) T_kj - four barrier-separated steps. Every block of T at or below the diagonal is
-// written (zeros above the diagonal of T_ii). In the block products a thread
-// forms four adjacent outputs of one row from 16-byte loads.
-__device__ __forceinline__ void invert_unit_lower(const float* __restrict__ A, uint8_t* sm,
-                                                  int tid) {
-  if (tid < 64) {
-    const int bi = tid >> 4, jj = tid & 15;
-    float x[16];
+// x <- the solution of (I + A_bb) x = x for the 16 x 16 diagonal block b, column
+// by column of A (right-looking: the 15 - i updates by x[i] are independent),
+// four columns' rows loaded at a time
+__device__ __forceinline__ void solve_unit_lower16(const float* __restrict__ A, float (&x)[16]) {
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
-      float s = r == jj ? 1.f : 0.f;
+  for (int q = 0; q < 4; ++q) {
+    float4 a[16];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (4 * q < r) {
-          const float4 a4 = *reinterpret_cast<const float4*>(A + a_off(16 * bi + r, 4 * bi + q));
-          const float av[4] = {a4.x, a4.y, a4.z, a4.w};
+    for (int r = 4 * q + 1; r < 16; ++r)
+      a[r] = *reinterpret_cast<const float4*>(A + r * kPitch + 4 * q);
 #pragma unroll
-          for (int e = 0; e < 4; ++e)
-            if (4 * q + e < r) s = fmaf(-av[e], x[4 * q + e], s);
-        }
-      }
-      x[r] = s;
-    }
+    for (int r = 4 * q + 1; r < 16; ++r) x[r] = fmaf(-a[r].x, x[4 * q], x[r]);
 #pragma unroll
-    for (int r = 0; r < 16; ++r) *t_at(sm, 16 * bi + r, 16 * bi + jj) = x[r];
-  } else if (tid < 64 + 6 * 16) {
-    // in the same step, the six products T_ii A_ik (k < i), column by column as
-    // the solutions of (I + A_ii) x = A_ik[:, col], each kept in the unused
-    // block (k, i) above the diagonal
-    const int task = tid - 64, b = task >> 4, col = task & 15;
-    const int ib = b < 1 ? 1 : b < 3 ? 2 : 3, kb = b - ib * (ib - 1) / 2;
-    float x[16];
+    for (int r = 4 * q + 2; r < 16; ++r) x[r] = fmaf(-a[r].y, x[4 * q + 1], x[r]);
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
-      float s = A[a_off(16 * ib + r, 4 * kb + (col >> 2)) + (col & 3)];
+    for (int r = 4 * q + 3; r < 16; ++r) x[r] = fmaf(-a[r].z, x[4 * q + 2], x[r]);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (4 * q < r) {
-          const float4 a4 = *reinterpret_cast<const float4*>(A + a_off(16 * ib + r, 4 * ib + q));
-          const float av[4] = {a4.x, a4.y, a4.z, a4.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e)
-            if (4 * q + e < r) s = fmaf(-av[e], x[4 * q + e], s);
-        }
-      }
-      x[r] = s;
-    }
-#pragma unroll
-    for (int r = 0; r < 16; ++r) *t_at(sm, 16 * kb + r, 16 * ib + col) = x[r];
+    for (int r = 4 * q + 4; r < 16; ++r) x[r] = fmaf(-a[r].w, x[4 * q + 3], x[r]);
   }
-  group_sync(1);
-  // then the blocks below the diagonal level by level (d = i - j = 1, 2, 3):
-  // T_ij = -sum_{k=j}^{i-1} (T_ii A_ik) T_kj, one barrier a level
+}
+
+// First step of T = (I + A)^{-1}: the diagonal blocks T_bb (threads 0 .. 63: a
+// column each) and, on threads 64 .. 159, the products P_bk = T_bb A_bk (k < b)
+// as the solutions of (I + A_bb) x = A_bk[:, col], in the place of A_bk.
+__device__ __forceinline__ void invert_diagonal(float* A, float* T, int tid) {
+  const int jj = tid & 15;
+  float x[16];
+  if (tid < 64) {
+    const int b = tid >> 4;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) x[r] = r == jj ? 1.f : 0.f;
+    solve_unit_lower16(blk(A, b, b), x);
+    float* t = blk(T, b, b) + jj;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) t[r * kPitch] = x[r];
+  } else {
+    const int task = (tid - 64) >> 4, b = task < 1 ? 1 : task < 3 ? 2 : 3;
+    float* t = blk(A, b, task - b * (b - 1) / 2) + jj;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) x[r] = t[r * kPitch];
+    solve_unit_lower16(blk(A, b, b), x);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) t[r * kPitch] = x[r];
+  }
+}
+
+// Then the blocks below the diagonal level by level (d = i - j = 1, 2, 3):
+// T_ij = -sum_{k=j}^{i-1} P_ik T_kj, one barrier a level. A thread forms four
+// outputs of one row for one block k (16 products each), and the d threads of
+// an output add theirs: each level is one pass of 20 independent 16-byte loads.
+// They sit in different half or quarter warps, so that the lanes served together
+// read the same rows (no bank conflicts).
+__device__ __forceinline__ void invert_levels(float* P, float* T, int tid) {
 #pragma unroll
   for (int d = 1; d < 4; ++d) {
+    const int lanes = d == 1 ? 32 : d == 2 ? 16 : 8;  // outputs of a warp
+    const int sp = (tid & 31) / lanes, t = (tid >> 5) * lanes + tid % lanes;
     // task t: block (jb + d, jb), row r, columns 4 c4 .. 4 c4 + 3
-    const int t = tid;
-    const int jb = t >> 6, ib = jb + d, r = (t >> 2) & 15, c4 = t & 3;
-    if (t < (4 - d) * 64) {
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      // 4 d chunks of k (a compile-time count: the loads can all be issued early)
+    const int jb = t >> 6, ib = jb + d, r = (t >> 2) & 15, c4 = t & 3, kb = jb + sp;
+    const bool on = t < (4 - d) * 64 && sp < d;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (on) {
+      const float* pr = blk(P, ib, kb) + r * kPitch;
+      const float* tr = blk(T, kb, jb) + 4 * c4;
 #pragma unroll
-      for (int kk = 0; kk < 4 * d; ++kk) {
-        const int kb = jb + (kk >> 2), k4 = kk & 3;
-        const float4 p4 = *reinterpret_cast<const float4*>(t_at(sm, 16 * kb + r, 16 * ib + 4 * k4));
+      for (int k4 = 0; k4 < 4; ++k4) {
+        const float4 p4 = *reinterpret_cast<const float4*>(pr + 4 * k4);
         const float pv[4] = {p4.x, p4.y, p4.z, p4.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const float4 t4 =
-              *reinterpret_cast<const float4*>(t_at(sm, 16 * kb + 4 * k4 + e, 16 * jb + 4 * c4));
+          const float4 t4 = *reinterpret_cast<const float4*>(tr + (4 * k4 + e) * kPitch);
           acc.x = fmaf(pv[e], t4.x, acc.x);
           acc.y = fmaf(pv[e], t4.y, acc.y);
           acc.z = fmaf(pv[e], t4.z, acc.z);
           acc.w = fmaf(pv[e], t4.w, acc.w);
         }
       }
-      *reinterpret_cast<float4*>(t_at(sm, 16 * ib + r, 16 * jb + 4 * c4)) =
-          make_float4(-acc.x, -acc.y, -acc.z, -acc.w);
     }
+#pragma unroll
+    for (int o = lanes; o < 32; o <<= 1) {
+      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+      acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o);
+      acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
+    }
+    if (on && sp == 0)
+      *reinterpret_cast<float4*>(blk(T, ib, jb) + r * kPitch + 4 * c4) =
+          make_float4(-acc.x, -acc.y, -acc.z, -acc.w);
     group_sync(1);
   }
+}
+
+// The gates of a chunk and their decay products, by two warps (t = 0 .. 63):
+// g_t = a_0 .. a_t and G[C-1][t] = a_{t+1} .. a_63 by scans, each warp
+// multiplying in the other's half
+__device__ __forceinline__ void decays(float* v, int t, int lane, float a, float a_other,
+                                       float b) {
+  float pre = a, suf = a, all = a_other;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const float x = __shfl_up_sync(0xffffffffu, pre, d);
+    if (lane >= d) pre *= x;
+    const float y = __shfl_down_sync(0xffffffffu, suf, d);
+    if (lane + d < 32) suf *= y;
+    all *= __shfl_xor_sync(0xffffffffu, all, d);
+  }
+  suf = __shfl_down_sync(0xffffffffu, suf, 1);  // a_{t+1} .. of this warp
+  if (lane == 31) suf = 1.f;
+  const float g = t >= 32 ? all * pre : pre;
+  v[t] = a;
+  v[64 + t] = b;
+  v[128 + t] = pre;
+  v[192 + t] = g;
+  v[256 + t] = t < 32 ? suf * all : suf;
+  if (t == kC - 1) v[320] = g;
 }
 
 template <bool DELTA>
@@ -283,22 +316,20 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                            ~uintptr_t(1023));
-  float* va = reinterpret_cast<float*>(sm + kOffVec);  // a of the chunk's tokens (1 past its end)
-  float* vb = va + 64;                                 // b (0 past its end)
-  float* vg = vb + 64;                                 // g_r = a_0 ... a_r
-  float* vgc2 = vg + 64;                               // [2][64]: G[C-1][i], by chunk parity
-  float* gC2 = vgc2 + 128;                             // [2]: g_{C-1}
-  float* Am = reinterpret_cast<float*>(sm + kOffA);
+  float* const vec = reinterpret_cast<float*>(sm + kOffVec);  // chunk j's gates at (j % 3) kVecFloats
+  float* const Am = reinterpret_cast<float*>(sm + kOffA);
+  float* const Tm = reinterpret_cast<float*>(sm + kOffT);
   __nv_bfloat16* ost = reinterpret_cast<__nv_bfloat16*>(sm + kOffOut);
-  uint64_t* bar_k = reinterpret_cast<uint64_t*>(sm + kOffBar);  // K buffers 0 and 1
-  uint64_t* bar_q = bar_k + 2;
-  uint64_t* bar_v = bar_k + 3;
-  uint64_t* bar_a = bar_k + 4;    // the solve group's MMAs
-  uint64_t* bar_x = bar_k + 5;    // X of a chunk is done: [-W | g Q] may be replaced
-  uint64_t* bar_so = bar_k + 6;   // the state and output MMAs of a chunk
-  uint64_t* ready = bar_k + 7;    // a chunk's U, [-W | g Q] and M o G are ready
-  uint64_t* u_free = bar_k + 8;   // a chunk's U has been read
-  uint64_t* drain = bar_k + 9;    // [2]
+  uint64_t* bar_k = reinterpret_cast<uint64_t*>(sm + kOffBar);  // [2], by chunk parity
+  uint64_t* bar_q = bar_k + 2;                                  // [2]
+  uint64_t* bar_v = bar_k + 4;
+  uint64_t* bar_g = bar_k + 5;    // [K; Q] K^T of a chunk is done
+  uint64_t* bar_uw = bar_k + 6;   // U and W of a chunk are done
+  uint64_t* bar_x = bar_k + 7;    // X of a chunk is done: [-W | g Q] may be replaced
+  uint64_t* bar_so = bar_k + 8;   // the state and output MMAs of a chunk
+  uint64_t* ready = bar_k + 9;    // the solve group is done with a chunk
+  uint64_t* u_free = bar_k + 10;  // a chunk's U and X have been read
+  uint64_t* drain = bar_k + 11;   // [2]
   uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tslot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -308,7 +339,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   const int c = tid & 127;    // TMEM lane: value column c (and key column c of W)
   const int h = blockIdx.x, r = blockIdx.y;
   if (threadIdx.x == 0) {
-    for (int b = 0; b < 7; ++b) mbar_init(bar_k + b, 1);
+    for (int b = 0; b < 9; ++b) mbar_init(bar_k + b, 1);
     mbar_init(ready, kGroup / 32);
     mbar_init(u_free, kGroup / 32);
     mbar_init(drain, 1);
@@ -342,37 +373,49 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   const size_t head = (size_t(r) * Hl + h) * kD;  // row 0 of this (request, head)'s state
   const uint64_t pol = policy_evict_first();
 
-  // TMA copies of chunk j's K (into buffer j & 1), Q and V. K of the first two
-  // chunks, Q and V are issued by the solve group's thread 0, later K by the
-  // state group's. `pend` / `par` remember the barriers this thread armed (bits
-  // 0, 1: K buffers, 2: Q, 3: V) and the parity of their last phase, for the
-  // wait after an abort.
+  // TMA copies of chunk j's K and Q (into the buffers of its parity) and V. The
+  // first ones are issued by the solve group's thread 0, the later ones by the
+  // thread 0 of the group that last read the buffer. `pend` / `par` remember the
+  // barriers this thread armed (bits 0, 1: K, 2, 3: Q, 4: V) and the parity of
+  // their last phase, for the wait after an abort.
   uint32_t pend = 0, par = 0;
   auto armed = [&](int bit, int phase) {
     pend |= 1u << bit;
     par = (par & ~(1u << bit)) | (uint32_t(phase & 1) << bit);
   };
-  auto load_k = [&](int j) {
-    uint64_t* b = bar_k + (j & 1);
-    mbar_arrive_expect_tx(b, 2 * 8192);
+  auto load = [&](const CUtensorMap* map, uint64_t* bar, uint32_t off, uint32_t slice, int j) {
+    mbar_arrive_expect_tx(bar, 2 * 8192);
     for (int sl = 0; sl < 2; ++sl)
-      tma_load_3d(sm + kOffKQ + sl * kKQSlice + (j & 1) * 16384, &tmK, b, sl * 64, h,
-                  p0 + j * kC, pol);
+      tma_load_3d(sm + off + sl * slice, map, bar, sl * 64, h, p0 + j * kC, pol);
+  };
+  auto load_k = [&](int j) {
+    load(&tmK, bar_k + (j & 1), kOffKQ + (j & 1) * kKQBuf, kKQSlice, j);
     armed(j & 1, j >> 1);
   };
   auto load_q = [&](int j) {
-    mbar_arrive_expect_tx(bar_q, 2 * 8192);
-    for (int sl = 0; sl < 2; ++sl)
-      tma_load_3d(sm + kOffKQ + sl * kKQSlice + 8192, &tmQ, bar_q, sl * 64, h, p0 + j * kC, pol);
-    armed(2, j);
+    load(&tmQ, bar_q + (j & 1), kOffKQ + 8192 + (j & 1) * kKQBuf, kKQSlice, j);
+    armed(2 + (j & 1), j >> 1);
   };
   auto load_v = [&](int j) {
-    mbar_arrive_expect_tx(bar_v, 2 * 8192);
-    for (int sl = 0; sl < 2; ++sl)
-      tma_load_3d(sm + kOffV + sl * kVSlice, &tmV, bar_v, sl * 64, h, p0 + j * kC, pol);
-    armed(3, j);
+    load(&tmV, bar_v, kOffV, kVSlice, j);
+    armed(4, j);
   };
   bool ok = true;
+  // g Q of chunk j as rows 64 .. 127 (the second N slice) of the MN-major
+  // [-W | g Q] operand: thread c writes dk row c, each warpgroup half of the tokens
+  auto write_gq = [&](int j) {
+    const uint8_t* qt = sm + kOffKQ + 8192 + (j & 1) * kKQBuf;
+    const float* vg = vec + (j % 3) * kVecFloats + 192;
+#pragma unroll
+    for (int j4 = 0; j4 < 4; ++j4) {
+      const int jj = 4 * grp + j4;
+      float x[8], gv[8];
+      load8(gv, vg + 8 * jj);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) x[e] = gv[e] * bf(qt, sw_off(8 * jj + e, c, kKQSlice));
+      put8(sm + kOffWQh + kWQSlice, sm + kOffWQl + kWQSlice, c, jj, x);
+    }
+  };
 
   if (role == 0) {
     // ================================================================ solve
@@ -380,154 +423,137 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       load_k(0);
       load_q(0);
       load_v(0);
-      if (nch > 1) load_k(1);
+      if (nch > 1) {
+        load_k(1);
+        load_q(1);
+      }
     }
-    // the gates of the first chunk (thread t < 64: token t of the chunk)
-    float na = 1.f, nb = 0.f;
-    if (tid < kC && p0 + tid < p1) {
-      na = alpha[size_t(p0 + tid) * Hl + h];
-      nb = beta[size_t(p0 + tid) * Hl + h];
+    // a chunk's gates are read two chunks ahead and their products formed one
+    // ahead, by the group's last two warps (token t of the chunk; 1 and 0 past
+    // the prefix's end), beside the first step of the inverse
+    const int gt = tid - (kGroup - kC);
+    float ga = 1.f, go = 1.f, gb = 0.f;  // this token's, and a of the other warp's
+    auto read_gates = [&](int j) {
+      const int t = p0 + j * kC + gt, u = p0 + j * kC + (gt ^ 32);
+      ga = t < p1 ? alpha[size_t(t) * Hl + h] : 1.f;
+      gb = t < p1 ? beta[size_t(t) * Hl + h] : 0.f;
+      go = u < p1 ? alpha[size_t(u) * Hl + h] : 1.f;
+    };
+    if (gt >= 0 && nch > 0) {
+      read_gates(0);
+      decays(vec, gt, lane, ga, go, gb);
+      read_gates(1);
     }
-    uint32_t aph = 0;
+    // [K; Q] K^T of chunk j: k.k and q.k in float32 (one thread; false: its
+    // operands did not come)
+    auto issue_gm = [&](int j) {
+      if (!mbar_wait(bar_k + (j & 1), (j >> 1) & 1, wait_ns, abort_flag) ||
+          !mbar_wait(bar_q + (j & 1), (j >> 1) & 1, wait_ns, abort_flag))
+        return false;
+      tc_fence_after();
+      const uint32_t kq = smem_u32(sm + kOffKQ + (j & 1) * kKQBuf);
+#pragma unroll
+      for (int st = 0; st < 8; ++st) {
+        const uint32_t a = kq + (st >> 2) * kKQSlice + 32 * (st & 3);
+        mma_f16(tmem + kColGM, desc_k_sw128(a), desc_k_sw128(a), idesc_bf16_f32(128, 64), st != 0);
+      }
+      mma_commit(bar_g);
+      return true;
+    };
+    bool issued = true;  // this thread's loads and MMAs went out
+    if (warp == 0 && nch > 0 && elect_one()) issued = issue_gm(0);
+    __syncwarp();
     for (int j = 0; j < nch; ++j) {
-      const int c0 = p0 + j * kC;
       const bool last = j + 1 == nch;
       const int odd = j & 1;
-      uint8_t* const kt = sm + kOffKQ + odd * 16384;  // this chunk's K (dk-slices kKQSlice apart)
-      uint8_t* const mt = sm + kOffM + odd * kMBuf;   // this chunk's M o G
-      // ---- gates and decay products: g_t = a_0 .. a_t and G[C-1][t] =
-      // a_{t+1} .. a_63 by scans over two warps (each multiplies in the other's
-      // half)
-      float gsuf = 1.f, gtot = 1.f;
-      if (tid < kC) {
-        va[tid] = na;
-        vb[tid] = nb;
-      }
-      group_sync(1);
-      if (tid < kC) {
-        const float other = va[tid ^ 32];
-        float pre = na, suf = na, all = other;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          const float x = __shfl_up_sync(0xffffffffu, pre, d);
-          if (lane >= d) pre *= x;
-          const float y = __shfl_down_sync(0xffffffffu, suf, d);
-          if (lane + d < 32) suf *= y;
-          all *= __shfl_xor_sync(0xffffffffu, all, d);
-        }
-        suf = __shfl_down_sync(0xffffffffu, suf, 1);  // a_{t+1} .. of this warp
-        if (lane == 31) suf = 1.f;
-        gtot = tid >= 32 ? all * pre : pre;
-        gsuf = tid < 32 ? suf * all : suf;
-        vg[tid] = gtot;
-        if (!last) {
-          const int t = c0 + kC + tid;
-          na = t < p1 ? alpha[size_t(t) * Hl + h] : 1.f;
-          nb = t < p1 ? beta[size_t(t) * Hl + h] : 0.f;
-        }
-      }
-      ok = group_and(1, mbar_wait(bar_k + odd, (j >> 1) & 1, wait_ns, abort_flag) &&
-                            mbar_wait(bar_q, j & 1, wait_ns, abort_flag));
+      uint8_t* const kt = sm + kOffKQ + odd * kKQBuf;  // this chunk's K (dk-slices kKQSlice apart)
+      uint8_t* const mt = sm + kOffM + odd * kMBuf;    // this chunk's M o G
+      float* const va = vec + (j % 3) * kVecFloats;  // this chunk's gates
+      const float *vb = va + 64, *vh = va + 128, *vg = va + 192;
+      bool okk = mbar_wait(bar_g, j & 1, wait_ns, abort_flag) && issued;
+      ok = group_and(1, okk);  // and the gates are in
       if (!ok) break;
-      // K of this chunk came after the state group was done with the chunk
-      // before last: its parity's M o G and decays may be replaced
-      if (tid < kC) vgc2[odd * 64 + tid] = gsuf;
-      if (tid == kC - 1) gC2[odd] = gtot;
-      // ---- [K; Q] K^T (even chunks) or [Q; K] K^T (odd): k.k and q.k in float32
-      if (warp == 0 && elect_one()) {
-        tc_fence_after();
-#pragma unroll
-        for (int st = 0; st < 8; ++st) {
-          const uint32_t sl = (st >> 2) * kKQSlice + 32 * (st & 3);
-          const uint32_t a = smem_u32(sm + kOffKQ + (odd ? 8192 : 0)) + sl;
-          const uint32_t b = smem_u32(kt) + sl;
-          mma_f16(tmem + kColGM, desc_k_sw128(a), desc_k_sw128(b), idesc_bf16_f32(128, 64),
-                  st != 0);
-        }
-        mma_commit(bar_a);
-      }
-      __syncwarp();
-      bool okk = true;
-      if (grp == 1) {
-        // g Q as rows 64 .. 127 (the second N slice) of the MN-major [-W | g Q]
-        // operand: thread c writes dk row c, the chunk's 64 tokens contiguous -
-        // once the previous chunk's X has read it
-        okk = j == 0 || mbar_wait(bar_x, (j - 1) & 1, wait_ns, abort_flag);
-        if (okk) {
-          const uint8_t* qt = sm + kOffKQ + 8192;
-#pragma unroll
-          for (int jj = 0; jj < 8; ++jj) {
-            float x[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e)
-              x[e] = vg[8 * jj + e] * bf(qt, sw_off(8 * jj + e, c, kKQSlice));
-            put8(sm + kOffWQh + kWQSlice, sm + kOffWQl + kWQSlice, c, jj, x);
-          }
-        }
-      }
-      okk = okk && mbar_wait(bar_a, aph, wait_ns, abort_flag);
-      aph ^= 1u;
       tc_fence_after();
-      // ---- the solve's matrix A (k rows) and M o G (q rows) from the first
-      // warpgroup's TMEM lanes, 32 columns of [K; Q] K^T at a time from the right
-      // (the decay G[rr][i] = a_{i+1} .. a_rr grows leftwards)
-      if (okk && grp == 0) {
-        const int rr = tid & 63;
-        const bool krow = (tid >> 6) == odd;
-        float g = 1.f;
+      float gr[32];
+      tmem_ld_32cols(tmem + lane_off + kColGM + 32 * (1 - grp), gr);
+      // ---- the solve's matrix A (k rows, lanes 0 .. 63) and M o G (q rows): the
+      // first warpgroup columns 32 .. 63, the second columns 0 .. 31; the decay
+      // G[rr][i] = a_{i+1} .. a_rr grows leftwards. This parity's M o G was last
+      // read by the chunk before last, whose state MMAs this chunk's K (its load
+      // came after them) has waited for.
+      {
+        const int rr = tid & 63, hf = 1 - grp;
+        float av[32];
 #pragma unroll
-        for (int hf = 1; hf >= 0; --hf) {
-          float gr[32];
-          tmem_ld_32cols(tmem + lane_off + kColGM + 32 * hf, gr);
-          tmem_wait_ld();
-          if (krow && !DELTA) continue;
-          const float b = vb[rr];
+        for (int q = 0; q < 8; ++q)
+          *reinterpret_cast<float4*>(av + 4 * q) =
+              *reinterpret_cast<const float4*>(va + 32 * hf + 4 * q);
+        float g = hf == 0 && rr >= 32 ? vh[rr] : 1.f;
+        const int top = rr - 32 * hf;  // the last column of this half up to rr
+        tmem_wait_ld();
+        if ((tid & 64) == 0) {
+          if (DELTA) {
+            // k row rr: A[rr][i] = b_rr G[rr][i] (k_rr . k_i), i < rr (what stands
+            // from rr on is never read)
+            g *= vb[rr];
+#pragma unroll
+            for (int i = 31; i >= 0; --i) {
+              gr[i] *= g;
+              if (i <= top) g *= av[i];
+            }
+            const int ib = rr >> 4;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              const int kb = 2 * hf + (q >> 2);
+              if (kb <= ib)
+                *reinterpret_cast<float4*>(blk(Am, ib, kb) + (rr & 15) * kPitch + 4 * (q & 3)) =
+                    make_float4(gr[4 * q], gr[4 * q + 1], gr[4 * q + 2], gr[4 * q + 3]);
+            }
+          }
+        } else {
+          // q row rr: (M o G)[rr][i] = (q_rr . k_i) G[rr][i], i <= rr
 #pragma unroll
           for (int i = 31; i >= 0; --i) {
-            const int col = 32 * hf + i;
-            const float gam = col <= rr ? g : 0.f;
-            if (col <= rr) g *= va[col];
-            // k row rr: A[rr][i] = b_rr G[rr][i] (k_rr . k_i), i < rr (the
-            // entries from rr on are never read); q row rr: (M o G)[rr][i] =
-            // (q_rr . k_i) G[rr][i], i <= rr
-            gr[i] = krow ? (col < rr ? b * gam * gr[i] : 0.f) : gam * gr[i];
+            gr[i] = i <= top ? gr[i] * g : 0.f;
+            if (i <= top) g *= av[i];
           }
-          if (krow) {
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-              *reinterpret_cast<float4*>(Am + a_off(rr, 8 * hf + q)) =
-                  make_float4(gr[4 * q], gr[4 * q + 1], gr[4 * q + 2], gr[4 * q + 3]);
-          } else {
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj)
-              put8(mt, mt + kMLo, rr, 4 * hf + jj, gr + 8 * jj);
-          }
+          for (int jj = 0; jj < 4; ++jj)
+            put8(mt, mt + kMLo, rr, 4 * hf + jj, gr + 8 * jj);
         }
       }
       fence_proxy_async_shared();
       tc_fence_before();
-      ok = group_and(1, okk);
-      if (!ok) break;
+      group_sync(1);
       if (DELTA) {
         // ---- T = (I + A)^{-1}, then T' = T diag(b) and T'' = T diag(b g) as
         // the hi/lo B operands (row r, 64 tokens i, K-major) of U = T' V and
-        // W = T'' K, in the first N slice of the [-W | g Q] tiles (free until W)
-        invert_unit_lower(Am, sm, tid);
-        {
+        // W = T'' K, in the first N slice of the [-W | g Q] tiles, once the
+        // previous chunk's X has read those
+        if (tid < 64 + 6 * 16)
+          invert_diagonal(Am, Tm, tid);
+        else if (gt >= 0 && !last) {
+          decays(vec + (j + 1) % 3 * kVecFloats, gt, lane, ga, go, gb);
+          read_gates(j + 2);
+        }
+        group_sync(1);
+        invert_levels(Am, Tm, tid);
+        okk = j == 0 || mbar_wait(bar_x, (j - 1) & 1, wait_ns, abort_flag);
+        if (okk) {
           const int row = tid >> 2;
 #pragma unroll
           for (int h2 = 0; h2 < 2; ++h2) {
             const int jj = 2 * (tid & 3) + h2;
             float x1[8], x2[8];
-            const float4 t0 = *reinterpret_cast<const float4*>(t_at(sm, row, 8 * jj));
-            const float4 t1 = *reinterpret_cast<const float4*>(t_at(sm, row, 8 * jj + 4));
-            const float tv[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+            float tv[8] = {}, bv[8], gv[8];
+            if ((jj >> 1) <= (row >> 4))
+              load8(tv, blk(Tm, row >> 4, jj >> 1) + (row & 15) * kPitch + 8 * (jj & 1));
+            load8(bv, vb + 8 * jj);
+            load8(gv, vg + 8 * jj);
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-              const int i = 8 * jj + e;
-              const float t = i <= row ? tv[e] : 0.f;
-              x1[e] = t * vb[i];
-              x2[e] = x1[e] * vg[i];
+              x1[e] = tv[e] * bv[e];  // T_ii is zero above the diagonal
+              x2[e] = x1[e] * gv[e];
             }
             put8(sm + kOffWQh, sm + kOffWQl, row, jj, x1);
             put8(sm + kOffWQh + 8192, sm + kOffWQl + 8192, row, jj, x2);
@@ -535,67 +561,67 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         }
         fence_proxy_async_shared();
         tc_fence_before();
-        group_sync(1);
-      }
-      // Q (and T in its slots) is no longer read: the next chunk's Q may land
-      if (tid == 0 && !last) load_q(j + 1);
-      okk = mbar_wait(bar_v, j & 1, wait_ns, abort_flag) &&
-            (j == 0 || mbar_wait(u_free, (j - 1) & 1, wait_ns, abort_flag));
-      if (DELTA) {
-        // ---- U^T = V^T T'^T and W^T = K^T T''^T: V and K are MN-major A
-        // operands (exact in bf16), T' and T'' enter as hi + lo
         ok = group_and(1, okk);
         if (!ok) break;
+        if (lane == 0) mbar_arrive(ready);
+        // ---- U^T = V^T T'^T and W^T = K^T T''^T: V and K are MN-major A
+        // operands (exact in bf16), T' and T'' enter as hi + lo; W^T takes the
+        // first half of X, which (like U) the state group has read by then. The
+        // next chunk's [K; Q] K^T follows at once.
         if (warp == 0 && elect_one()) {
-          tc_fence_after();
-          const uint32_t idesc = idesc_bf16_f32(128, 64) | (1u << 15);
+          issued = mbar_wait(bar_v, j & 1, wait_ns, abort_flag) &&
+                   (j == 0 || mbar_wait(u_free, (j - 1) & 1, wait_ns, abort_flag));
+          if (issued) {
+            tc_fence_after();
+            const uint32_t idesc = idesc_bf16_f32(128, 64) | (1u << 15);
 #pragma unroll
-          for (int pass = 0; pass < 2; ++pass) {
-            const uint32_t b = smem_u32(sm + (pass ? kOffWQl : kOffWQh));
+            for (int pass = 0; pass < 2; ++pass) {
+              const uint32_t b = smem_u32(sm + (pass ? kOffWQl : kOffWQh));
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              mma_f16(tmem + kColU, desc_mn_sw128(smem_u32(sm + kOffV) + k * 2048, kVSlice),
-                      desc_k_sw128(b + 32 * k), idesc, (pass | k) != 0);
-              mma_f16(tmem + kColGM, desc_mn_sw128(smem_u32(kt) + k * 2048, kKQSlice),
-                      desc_k_sw128(b + 8192 + 32 * k), idesc, (pass | k) != 0);
+              for (int k = 0; k < 4; ++k) {
+                mma_f16(tmem + kColU, desc_mn_sw128(smem_u32(sm + kOffV) + k * 2048, kVSlice),
+                        desc_k_sw128(b + 32 * k), idesc, (pass | k) != 0);
+                mma_f16(tmem + kColX, desc_mn_sw128(smem_u32(kt) + k * 2048, kKQSlice),
+                        desc_k_sw128(b + 8192 + 32 * k), idesc, (pass | k) != 0);
+              }
             }
+            mma_commit(bar_uw);
+            if (!last) issued = issue_gm(j + 1);
           }
-          mma_commit(bar_a);
         }
         __syncwarp();
-        okk = mbar_wait(bar_a, aph, wait_ns, abort_flag);
-        aph ^= 1u;
-        tc_fence_after();
-        // -W as the first N slice of [-W | g Q]: thread c writes key row c, each
-        // warpgroup half of the tokens
-        if (okk) {
-          float wv[32];
-          tmem_ld_32cols(tmem + lane_off + kColGM + 32 * grp, wv);
-          tmem_wait_ld();
-#pragma unroll
-          for (int i = 0; i < 32; ++i) wv[i] = -wv[i];
-#pragma unroll
-          for (int jj = 0; jj < 4; ++jj)
-            put8(sm + kOffWQh, sm + kOffWQl, c, 4 * grp + jj, wv + 8 * jj);
-        }
-      } else if (okk) {
+      } else {
         // gated linear attention: U = diag(b) V straight into TMEM
-        tc_fence_after();
-        const uint8_t* vt = sm + kOffV;
-        float uv[32];
+        if (gt >= 0 && !last) {
+          decays(vec + (j + 1) % 3 * kVecFloats, gt, lane, ga, go, gb);
+          read_gates(j + 2);
+        }
+        okk = mbar_wait(bar_v, j & 1, wait_ns, abort_flag) &&
+              (j == 0 || (mbar_wait(bar_x, (j - 1) & 1, wait_ns, abort_flag) &&
+                          mbar_wait(u_free, (j - 1) & 1, wait_ns, abort_flag)));
+        if (okk) {
+          write_gq(j);
+          tc_fence_after();
+          const uint8_t* vt = sm + kOffV;
+          float uv[32];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) uv[i] = vb[32 * grp + i] * bf(vt, sw_off(32 * grp + i, c, kVSlice));
-        tmem_st_32cols(tmem + lane_off + kColU + 32 * grp, uv);
-        tmem_wait_st();
+          for (int i = 0; i < 32; ++i)
+            uv[i] = vb[32 * grp + i] * bf(vt, sw_off(32 * grp + i, c, kVSlice));
+          tmem_st_32cols(tmem + lane_off + kColU + 32 * grp, uv);
+          tmem_wait_st();
+        }
+        fence_proxy_async_shared();
+        tc_fence_before();
+        ok = group_and(1, okk);
+        if (!ok) break;
+        if (lane == 0) mbar_arrive(ready);
+        if (tid == 0 && !last) load_v(j + 1);  // V is no longer read
+        __syncwarp();
+        if (warp == 0 && !last && elect_one()) issued = issue_gm(j + 1);
+        __syncwarp();
       }
-      fence_proxy_async_shared();
-      tc_fence_before();
-      ok = group_and(1, okk);
-      if (!ok) break;
-      if (lane == 0) mbar_arrive(ready);
-      // V is no longer read
-      if (tid == 0 && !last) load_v(j + 1);
     }
+    ok = group_and(1, ok && issued);
   } else {
     // ================================================================ state
     // the initial state: into TMEM (lane c holds S0^T[c][.] = S0[.][c]; this
@@ -616,10 +642,52 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       const int n = min(kC, p1 - c0);
       const bool last = j + 1 == nch;
       const int odd = j & 1;
-      uint8_t* const kt = sm + kOffKQ + odd * 16384;
+      uint8_t* const kt = sm + kOffKQ + odd * kKQBuf;
       uint8_t* const mt = sm + kOffM + odd * kMBuf;
-      ok = group_and(2, mbar_wait(ready, j & 1, wait_ns, abort_flag));
+      bool okk = mbar_wait(ready, j & 1, wait_ns, abort_flag);
+      const uint32_t scol = tmem + lane_off + kColSt + 64 * grp;
+      if (okk) {
+        if (DELTA) write_gq(j);  // while the tensor cores form U and W
+        // this warpgroup's 64 state columns, scaled by g_{C-1} for the last MMA
+        // to accumulate onto (X reads the hi/lo copy, not these)
+        const float g = vec[(j % 3) * kVecFloats + 320];
+        float s0[32], s1[32];
+        tmem_ld_32cols(scol, s0);
+        tmem_ld_32cols(scol + 32, s1);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          s0[i] *= g;
+          s1[i] *= g;
+        }
+        tmem_st_32cols(scol, s0);
+        tmem_st_32cols(scol + 32, s1);
+      }
+      if (DELTA) {
+        // -W as the first N slice: thread c writes key row c, each warpgroup half
+        // of the tokens (T' and T'' have been read)
+        okk = okk && mbar_wait(bar_uw, j & 1, wait_ns, abort_flag);
+        tc_fence_after();
+        if (okk) {
+          float wv[32];
+          tmem_ld_32cols(tmem + lane_off + kColX + 32 * grp, wv);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 32; ++i) wv[i] = -wv[i];
+#pragma unroll
+          for (int jj = 0; jj < 4; ++jj)
+            put8(sm + kOffWQh, sm + kOffWQl, c, 4 * grp + jj, wv + 8 * jj);
+        }
+      }
+      fence_proxy_async_shared();
+      tc_fence_before();
+      ok = group_and(2, okk);
       if (!ok) break;
+      // this chunk's Q (and V, for the delta rule) are no longer read
+      if (tid == 0) {
+        if (j + 2 < nch) load_q(j + 2);
+        if (DELTA && !last) load_v(j + 1);
+      }
       // ---- X = S0^T [-W | g Q] (delta rule) or O^T = S0^T (g Q) (gated linear
       // attention): three hi/lo passes; A (the state, K = dk) from TMEM, 8 packed
       // columns per K = 16 step; the B operand is MN-major (dk rows of 128 tokens)
@@ -642,28 +710,13 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         mma_commit(bar_x);
       }
       __syncwarp();
-      // this warpgroup's 64 state columns, scaled by g_{C-1} for the last MMA to
-      // accumulate onto (X reads the hi/lo copy, not these)
-      const float g = gC2[odd];
-      const uint32_t scol = tmem + lane_off + kColSt + 64 * grp;
-      {
-        float s0[32];
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          tmem_ld_32cols(scol + 32 * hf, s0);
-          tmem_wait_ld();
-#pragma unroll
-          for (int i = 0; i < 32; ++i) s0[i] *= g;
-          tmem_st_32cols(scol + 32 * hf, s0);
-        }
-      }
       const bool okx = mbar_wait(bar_x, j & 1, wait_ns, abort_flag);
       tc_fence_after();
       // ---- d = U + X (column c of d is row c of d^T): the first warpgroup
       // writes d^T, the second (d G[C-1])^T, as bf16 hi/lo A operands in TMEM
       // over the old state's (X has read it)
       if (okx) {
-        const float* vgc = vgc2 + odd * 64;
+        const float* vgc = vec + (j % 3) * kVecFloats + 256;
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
           float dr[32];
@@ -752,11 +805,12 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       group_sync(2);
       // each token's 128 outputs are 256 contiguous bytes of o (the next chunk's
       // staging comes after several of this group's barriers)
-      for (int e = tid; e < n * (kD / 8); e += kGroup) {
-        const int t = e / (kD / 8), q = e % (kD / 8);
-        *reinterpret_cast<uint4*>(o + (size_t(c0 + t) * Hl + h) * kD + 8 * q) =
-            reinterpret_cast<const uint4*>(ost)[e];
-      }
+      __nv_bfloat16* const od = o + (size_t(c0 + (tid >> 4)) * Hl + h) * kD + 8 * (tid & 15);
+#pragma unroll
+      for (int i = 0; i < kC * (kD / 8) / kGroup; ++i)
+        if ((tid >> 4) + 16 * i < n)
+          *reinterpret_cast<uint4*>(od + size_t(16 * i) * Hl * kD) =
+              reinterpret_cast<const uint4*>(ost)[tid + kGroup * i];
     }
   }
   if (!ok) {
@@ -765,7 +819,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     *abort_flag = 1;
     if (tid == 0) {
       flag(status, JET_ERR_TIMEOUT);
-      for (int b = 0; b < 4; ++b)
+      for (int b = 0; b < 5; ++b)
         if (pend & (1u << b)) mbar_wait(bar_k + b, (par >> b) & 1u, kDrainNs, nullptr);
     }
     __syncwarp();
