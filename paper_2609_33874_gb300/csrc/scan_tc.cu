@@ -30,12 +30,19 @@
 // chunk instead of the 64^2 / 2 per column of a substitution for all 256
 // columns of U and W.
 //
-// One CTA per (request, head); 8 warps: lane c of TMEM (value column c, and
-// key column c of W) belongs to thread c of each warpgroup, which split the
-// per-column work between them; thread 0 issues the TMA copies and warp 0's
-// elected thread the MMAs.
-// The next chunk's K goes into a second buffer while the current chunk runs;
-// Q and V are refilled as soon as the current chunk no longer reads them.
+// One CTA per (request, head), two groups of eight warps. The solve group works
+// one chunk ahead of the state: it forms A, M o G, T, T diag(b) and T diag(b g)
+// of chunk j + 1 (none of which needs the state) and issues U and W, while the
+// state group runs X, d, O and the new state of chunk j. Lane c of TMEM (value
+// column c, and key column c of W) belongs to thread c of each warpgroup, which
+// split the columns. What bounds it: the chain of the state group (X, d, O and
+// S, the new operand: 5 to 6 us a chunk) and the instructions of the hi/lo
+// splits (40 % of the issue slots); with one group doing both in turn a chunk
+// took 11 us. 32 requests x 512 tokens x 16 heads: delta rule 338 -> 228 us, gated
+// linear attention 199 -> 147 us; 3 x 2,000 - 4,000 tokens 595 -> 362 and 341 ->
+// 223 us. Where it was lost before: bank conflicts and address arithmetic in the
+// inverse, one chunk's gates scanned inside its chain, outputs written before the
+// next chunk's X.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -615,7 +622,9 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         ok = group_and(1, okk);
         if (!ok) break;
         if (lane == 0) mbar_arrive(ready);
-        if (tid == 0 && !last) load_v(j + 1);  // V is no longer read
+        // neither V nor Q is read any more
+        if (tid == 0 && !last) load_v(j + 1);
+        if (tid == 0 && j + 2 < nch) load_q(j + 2);
         __syncwarp();
         if (warp == 0 && !last && elect_one()) issued = issue_gm(j + 1);
         __syncwarp();
@@ -637,33 +646,31 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     tc_fence_before();
     group_sync(2);
     const float rs = rsqrtf(float(kD));
+    float ov[32];  // a chunk's outputs: value column c of this warpgroup's 32 tokens
+    // chunk j's outputs from ov, through shared memory as they are stored ([token]
+    // [value]): each token's 128 outputs are 256 contiguous bytes of o (the next
+    // chunk's staging comes after several of this group's barriers)
+    auto write_out = [&](int j) {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) ost[(32 * grp + i) * kD + c] = __float2bfloat16_rn(ov[i] * rs);
+      group_sync(2);
+      const int c0 = p0 + j * kC, n = min(kC, p1 - c0);
+      __nv_bfloat16* const od = o + (size_t(c0 + (tid >> 4)) * Hl + h) * kD + 8 * (tid & 15);
+#pragma unroll
+      for (int i = 0; i < kC * (kD / 8) / kGroup; ++i)
+        if ((tid >> 4) + 16 * i < n)
+          *reinterpret_cast<uint4*>(od + size_t(16 * i) * Hl * kD) =
+              reinterpret_cast<const uint4*>(ost)[tid + kGroup * i];
+    };
     for (int j = 0; j < nch; ++j) {
-      const int c0 = p0 + j * kC;
-      const int n = min(kC, p1 - c0);
       const bool last = j + 1 == nch;
       const int odd = j & 1;
       uint8_t* const kt = sm + kOffKQ + odd * kKQBuf;
       uint8_t* const mt = sm + kOffM + odd * kMBuf;
       bool okk = mbar_wait(ready, j & 1, wait_ns, abort_flag);
       const uint32_t scol = tmem + lane_off + kColSt + 64 * grp;
-      if (okk) {
-        if (DELTA) write_gq(j);  // while the tensor cores form U and W
-        // this warpgroup's 64 state columns, scaled by g_{C-1} for the last MMA
-        // to accumulate onto (X reads the hi/lo copy, not these)
-        const float g = vec[(j % 3) * kVecFloats + 320];
-        float s0[32], s1[32];
-        tmem_ld_32cols(scol, s0);
-        tmem_ld_32cols(scol + 32, s1);
-        tmem_wait_ld();
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          s0[i] *= g;
-          s1[i] *= g;
-        }
-        tmem_st_32cols(scol, s0);
-        tmem_st_32cols(scol + 32, s1);
-      }
       if (DELTA) {
+        if (okk) write_gq(j);  // while the tensor cores form U and W
         // -W as the first N slice: thread c writes key row c, each warpgroup half
         // of the tokens (T' and T'' have been read)
         okk = okk && mbar_wait(bar_uw, j & 1, wait_ns, abort_flag);
@@ -679,14 +686,14 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             put8(sm + kOffWQh, sm + kOffWQl, c, 4 * grp + jj, wv + 8 * jj);
         }
       }
+      tmem_wait_st();  // the new state's operand, of the previous chunk
       fence_proxy_async_shared();
       tc_fence_before();
       ok = group_and(2, okk);
       if (!ok) break;
-      // this chunk's Q (and V, for the delta rule) are no longer read
-      if (tid == 0) {
+      if (DELTA && tid == 0) {  // this chunk's Q and V are no longer read
         if (j + 2 < nch) load_q(j + 2);
-        if (DELTA && !last) load_v(j + 1);
+        if (!last) load_v(j + 1);
       }
       // ---- X = S0^T [-W | g Q] (delta rule) or O^T = S0^T (g Q) (gated linear
       // attention): three hi/lo passes; A (the state, K = dk) from TMEM, 8 packed
@@ -710,6 +717,22 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         mma_commit(bar_x);
       }
       __syncwarp();
+      // while X runs: the previous chunk's outputs, and this warpgroup's 64 state
+      // columns scaled by g_{C-1} for the last MMA to accumulate onto (X reads the
+      // hi/lo copy, not these)
+      if (j > 0) write_out(j - 1);
+      {
+        const float g = vec[(j % 3) * kVecFloats + 320];
+        float s0[32];
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          tmem_ld_32cols(scol + 32 * hf, s0);
+          tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 32; ++i) s0[i] *= g;
+          tmem_st_32cols(scol + 32 * hf, s0);
+        }
+      }
       const bool okx = mbar_wait(bar_x, j & 1, wait_ns, abort_flag);
       tc_fence_after();
       // ---- d = U + X (column c of d is row c of d^T): the first warpgroup
@@ -774,9 +797,10 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       tc_fence_after();
       // this chunk's K is no longer read: the chunk after next may land there
       if (tid == 0 && j + 2 < nch) load_k(j + 2);
-      // ---- this warpgroup's 64 columns of the new state as the next chunk's
-      // operand (after the last chunk, the result), then the chunk's outputs
-      // (tokens 32 grp ..)
+      // ---- the outputs (tokens 32 grp ..) into registers, and this warpgroup's 64
+      // columns of the new state as the next chunk's operand (after the last
+      // chunk, the result)
+      tmem_ld_32cols(tmem + lane_off + kColO + 32 * grp, ov);
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {
         float s0[32];
@@ -792,26 +816,8 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                      tmem + lane_off + kColS0l + 32 * grp + 16 * hf, s0);
         }
       }
-      {
-        float ov[32];
-        tmem_ld_32cols(tmem + lane_off + kColO + 32 * grp, ov);
-        tmem_wait_ld();
-        // [token][value] as they are stored, for 16-byte global stores
-#pragma unroll
-        for (int i = 0; i < 32; ++i) ost[(32 * grp + i) * kD + c] = __float2bfloat16_rn(ov[i] * rs);
-      }
-      tmem_wait_st();
-      tc_fence_before();
-      group_sync(2);
-      // each token's 128 outputs are 256 contiguous bytes of o (the next chunk's
-      // staging comes after several of this group's barriers)
-      __nv_bfloat16* const od = o + (size_t(c0 + (tid >> 4)) * Hl + h) * kD + 8 * (tid & 15);
-#pragma unroll
-      for (int i = 0; i < kC * (kD / 8) / kGroup; ++i)
-        if ((tid >> 4) + 16 * i < n)
-          *reinterpret_cast<uint4*>(od + size_t(16 * i) * Hl * kD) =
-              reinterpret_cast<const uint4*>(ost)[tid + kGroup * i];
     }
+    if (ok && nch > 0) write_out(nch - 1);
   }
   if (!ok) {
     // a wait ran out: let the copies and tensor-core work already issued
