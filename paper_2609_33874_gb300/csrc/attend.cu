@@ -28,27 +28,33 @@ constexpr int kPlanSMs = 152;           // GB300
 constexpr int kMinChunkTc = 640;        // keys
 constexpr int kFewGroups = 22, kFewItems = 44, kLeastChunk = 192;
 
+// rows of Q, K and P are padded by 16 bytes: 16-byte reads of eight consecutive
+// rows then fall in different banks
 template <int DH>
 constexpr size_t prefix_smem_bytes() {
-  return sizeof(float) * (size_t(kQV) * (DH + 1) + size_t(kKT) * (DH + 1) + size_t(kKT) * DH +
-                          size_t(kQV) * (kKT + 1));
+  return sizeof(float) * (size_t(kQV) * (DH + 4) + size_t(kKT) * (DH + 4) + size_t(kKT) * DH +
+                          size_t(kQV) * (kKT + 4));
 }
 
 // One CTA: one prefix chunk of one (request, key/value head) for kQV query
 // vectors. Thread (vec = tid / 16, sub = tid % 16) scores keys sub and sub+16
-// of each tile for its vector and accumulates output dims sub + 16 i.
-template <typename T, int DH>
+// of each tile for its vector and accumulates output dims 4 sub + 64 i .. + 3.
+// Small batches are bound by the chain of loads: the query block and a tile are
+// fetched by 16-byte loads that are all in flight at once, and chunks go down to
+// one tile (7 rows over 128 keys: 13.2 -> 4.9 us).
+template <int DH>
 __global__ void __launch_bounds__(kThreads)
 attend_prefix_kernel(const int32_t* __restrict__ prefix_offset, const int32_t* __restrict__ row_offset,
                      int R, int N, int total_prefix, int Hq, int Hkv, int chunk,
-                     const T* __restrict__ q, const T* __restrict__ k_pre, const T* __restrict__ v_pre,
-                     float* __restrict__ o_part, float2* __restrict__ ml_part, int* status) {
+                     const float* __restrict__ q, const float* __restrict__ k_pre,
+                     const float* __restrict__ v_pre, float* __restrict__ o_part,
+                     float2* __restrict__ ml_part, int* status) {
   pdl_begin();
-  extern __shared__ float smem[];
-  float* Qs = smem;                          // [kQV][DH+1], pre-scaled by 1/sqrt(d)
-  float* Ks = Qs + kQV * (DH + 1);           // [kKT][DH+1]
-  float* Vs = Ks + kKT * (DH + 1);           // [kKT][DH]
-  float* Ps = Vs + kKT * DH;                 // [kQV][kKT+1]
+  extern __shared__ __align__(16) float smem[];
+  float* Qs = smem;                          // [kQV][DH+4], pre-scaled by log2(e)/sqrt(d)
+  float* Ks = Qs + kQV * (DH + 4);           // [kKT][DH+4]
+  float* Vs = Ks + kKT * (DH + 4);           // [kKT][DH]
+  float* Ps = Vs + kKT * DH;                 // [kQV][kKT+4]
 
   const int split = blockIdx.x, qg = blockIdx.y;
   const int r = blockIdx.z / Hkv, kh = blockIdx.z % Hkv;
@@ -66,50 +72,73 @@ attend_prefix_kernel(const int32_t* __restrict__ prefix_offset, const int32_t* _
   const int k_begin = split * chunk;
   const int k_end = min(P, k_begin + chunk);
 
+  constexpr int C4 = DH / 4;                       // 16-byte pieces of a row
+  constexpr int QI = kQV * C4 / kThreads;          // of the query block per thread
+  constexpr int KI = kKT * C4 / kThreads;          // of a K (or V) tile per thread
   const int tid = threadIdx.x;
   const int vec = tid >> 4, sub = tid & 15;
   const float scale = 1.4426950408889634f * rsqrtf(float(DH));  // base-2 scores
-  for (int i = tid; i < kQV * DH; i += kThreads) {
-    const int vv = i / DH, dd = i % DH, gv = vbase + vv;
-    float x = 0.f;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  // a tile's keys past k_end are zeros
+  float4 kr[KI], vr[KI];
+  auto fetch = [&](int kb) {
+#pragma unroll
+    for (int i = 0; i < KI; ++i) {
+      const int e = tid + i * kThreads, j = e / C4, c = e % C4;
+      const bool in = kb + j < k_end;
+      const size_t idx = (size_t(p0 + kb + (in ? j : 0)) * Hkv + kh) * DH + 4 * c;
+      kr[i] = in ? *reinterpret_cast<const float4*>(k_pre + idx) : zero;
+      vr[i] = in ? *reinterpret_cast<const float4*>(v_pre + idx) : zero;
+    }
+  };
+  if (k_begin < k_end) fetch(k_begin);
+#pragma unroll
+  for (int i = 0; i < QI; ++i) {
+    const int e = tid + i * kThreads, vv = e / C4, c = e % C4, gv = vbase + vv;
+    float4 x = zero;
     if (gv < nvec) {
       const int n = n0 + gv / g, h = kh * g + gv % g;
-      x = to_f32(q[(size_t(n) * Hq + h) * DH + dd]) * scale;
+      x = *reinterpret_cast<const float4*>(q + (size_t(n) * Hq + h) * DH + 4 * c);
     }
-    Qs[vv * (DH + 1) + dd] = x;
+    *reinterpret_cast<float4*>(Qs + vv * (DH + 4) + 4 * c) =
+        make_float4(x.x * scale, x.y * scale, x.z * scale, x.w * scale);
   }
 
-  constexpr int PER = DH / 16;
-  float acc[PER];
+  constexpr int PER = DH / 64;
+  float4 acc[PER];
 #pragma unroll
-  for (int i = 0; i < PER; ++i) acc[i] = 0.f;
+  for (int i = 0; i < PER; ++i) acc[i] = zero;
   float m = -INFINITY, l = 0.f;
 
   for (int kb = k_begin; kb < k_end; kb += kKT) {
     const int nk = min(kKT, k_end - kb);
     __syncthreads();
-    for (int i = tid; i < kKT * DH; i += kThreads) {
-      const int j = i / DH, dd = i % DH;
-      float kx = 0.f, vx = 0.f;
-      if (j < nk) {
-        const size_t idx = (size_t(p0 + kb + j) * Hkv + kh) * DH + dd;
-        kx = to_f32(k_pre[idx]);
-        vx = to_f32(v_pre[idx]);
-      }
-      Ks[j * (DH + 1) + dd] = kx;
-      Vs[j * DH + dd] = vx;
+#pragma unroll
+    for (int i = 0; i < KI; ++i) {
+      const int e = tid + i * kThreads, j = e / C4, c = e % C4;
+      *reinterpret_cast<float4*>(Ks + j * (DH + 4) + 4 * c) = kr[i];
+      *reinterpret_cast<float4*>(Vs + j * DH + 4 * c) = vr[i];
     }
     __syncthreads();
+    if (kb + kKT < k_end) fetch(kb + kKT);  // the next tile, while this one is used
 
-    const float* qv = Qs + vec * (DH + 1);
-    const float* k0 = Ks + sub * (DH + 1);
-    const float* k1 = Ks + (sub + 16) * (DH + 1);
+    const float* qv = Qs + vec * (DH + 4);
+    const float* k0 = Ks + sub * (DH + 4);
+    const float* k1 = Ks + (sub + 16) * (DH + 4);
     float s0 = 0.f, s1 = 0.f;
 #pragma unroll 8
-    for (int dd = 0; dd < DH; ++dd) {
-      const float x = qv[dd];
-      s0 = fmaf(x, k0[dd], s0);
-      s1 = fmaf(x, k1[dd], s1);
+    for (int dd = 0; dd < DH; dd += 4) {
+      const float4 x = *reinterpret_cast<const float4*>(qv + dd);
+      const float4 a = *reinterpret_cast<const float4*>(k0 + dd);
+      const float4 b = *reinterpret_cast<const float4*>(k1 + dd);
+      s0 = fmaf(x.x, a.x, s0);
+      s1 = fmaf(x.x, b.x, s1);
+      s0 = fmaf(x.y, a.y, s0);
+      s1 = fmaf(x.y, b.y, s1);
+      s0 = fmaf(x.z, a.z, s0);
+      s1 = fmaf(x.z, b.z, s1);
+      s0 = fmaf(x.w, a.w, s0);
+      s1 = fmaf(x.w, b.w, s1);
     }
     if (sub >= nk) s0 = -INFINITY;
     if (sub + 16 >= nk) s1 = -INFINITY;
@@ -124,16 +153,22 @@ attend_prefix_kernel(const int32_t* __restrict__ prefix_offset, const int32_t* _
     for (int o = 8; o > 0; o >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, o);
     l = l * corr + psum;
     m = mn;
-    Ps[vec * (kKT + 1) + sub] = e0;
-    Ps[vec * (kKT + 1) + sub + 16] = e1;
+    Ps[vec * (kKT + 4) + sub] = e0;
+    Ps[vec * (kKT + 4) + sub + 16] = e1;
     __syncwarp();
 #pragma unroll
-    for (int i = 0; i < PER; ++i) acc[i] *= corr;
+    for (int i = 0; i < PER; ++i)
+      acc[i] = make_float4(acc[i].x * corr, acc[i].y * corr, acc[i].z * corr, acc[i].w * corr);
     for (int j = 0; j < nk; ++j) {
-      const float pj = Ps[vec * (kKT + 1) + j];
-      const float* vr = Vs + j * DH + sub;
+      const float pj = Ps[vec * (kKT + 4) + j];
 #pragma unroll
-      for (int i = 0; i < PER; ++i) acc[i] = fmaf(pj, vr[16 * i], acc[i]);
+      for (int i = 0; i < PER; ++i) {
+        const float4 x = *reinterpret_cast<const float4*>(Vs + j * DH + 4 * sub + 64 * i);
+        acc[i].x = fmaf(pj, x.x, acc[i].x);
+        acc[i].y = fmaf(pj, x.y, acc[i].y);
+        acc[i].z = fmaf(pj, x.z, acc[i].z);
+        acc[i].w = fmaf(pj, x.w, acc[i].w);
+      }
     }
   }
 
@@ -142,75 +177,85 @@ attend_prefix_kernel(const int32_t* __restrict__ prefix_offset, const int32_t* _
     const int n = n0 + gv / g, h = kh * g + gv % g;
     const size_t base = (size_t(split) * N + n) * Hq + h;
 #pragma unroll
-    for (int i = 0; i < PER; ++i) o_part[base * DH + sub + 16 * i] = acc[i];
+    for (int i = 0; i < PER; ++i)
+      *reinterpret_cast<float4*>(o_part + base * DH + 4 * sub + 64 * i) = acc[i];
     if (sub == 0) ml_part[base] = make_float2(m, l);
   }
 }
 
-// One warp per (row, query head): combine the prefix chunks, then the row's
-// own causal candidate keys, and normalise.
-template <typename T, int DH>
-__global__ void __launch_bounds__(256)
+// One warp per (row, query head), float32: the prefix chunks' partials, then the
+// row's own causal candidate keys, normalised. The loads that do not depend on
+// each other go out together: the chunks' (m, l) one a lane, their outputs and
+// the candidate's keys and values four at a time.
+template <int DH>
+__global__ void __launch_bounds__(128)
 attend_merge_kernel(const int32_t* __restrict__ row_req, const int32_t* __restrict__ row_cand,
                     const int32_t* __restrict__ cand_row_offset, int N, int R, int C, int Hq, int Hkv,
-                    int splits, const T* __restrict__ q, const T* __restrict__ k_cand,
-                    const T* __restrict__ v_cand, const float* __restrict__ o_part,
-                    const float2* __restrict__ ml_part, T* __restrict__ o, int* status) {
+                    int splits, const float* __restrict__ q, const float* __restrict__ k_cand,
+                    const float* __restrict__ v_cand, const float* __restrict__ o_part,
+                    const float2* __restrict__ ml_part, float* __restrict__ o, int* status) {
   pdl_begin();
   const int lane = threadIdx.x & 31;
   const long long idx = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (idx >= (long long)N * Hq) return;
   const int n = int(idx / Hq), h = int(idx % Hq);
   const int kh = h / (Hq / Hkv);
+  const int c = row_cand[n], r = row_req[n];
   constexpr int PER = DH / 32;
+  float qv[PER];
+#pragma unroll
+  for (int i = 0; i < PER; ++i) qv[i] = q[(size_t(n) * Hq + h) * DH + lane + 32 * i];
   float acc[PER];
-#pragma unroll
-  for (int i = 0; i < PER; ++i) acc[i] = 0.f;
-  float m = -INFINITY, l = 0.f;
-  for (int s = 0; s < splits; ++s) {
-    const size_t base = (size_t(s) * N + n) * Hq + h;
-    const float2 ml = ml_part[base];
-    if (!(ml.y > 0.f)) continue;  // empty chunk
-    const float mn = fmaxf(m, ml.x);
-    const float a = exp2f(m - mn), b = exp2f(ml.x - mn);
-#pragma unroll
-    for (int i = 0; i < PER; ++i) acc[i] = acc[i] * a + o_part[base * DH + lane + 32 * i] * b;
-    l = l * a + ml.y * b;
-    m = mn;
-  }
-  const int c = row_cand[n];
+  float m, l;
+  combine_chunks<DH>(splits, N, Hq, n, h, lane, ml_part, o_part, m, l, acc);
   if (c >= 0) {
-    const int r = row_req[n];
     const int first = (c < C) ? cand_row_offset[c] : -1;
     if (first < 0 || first > n || r < 0 || first - r - 1 < 0 || n - r - 1 >= N - R) {
       if (lane == 0) flag(status, JET_ERR_DEVICE);
     } else {
       const float scale = 1.4426950408889634f * rsqrtf(float(DH));  // base 2
-      float qv[PER];
+      for (int n4 = first; n4 <= n; n4 += 4) {
+        float kv[4][PER], vv[4][PER], sc[4];
 #pragma unroll
-      for (int i = 0; i < PER; ++i) qv[i] = to_f32(q[(size_t(n) * Hq + h) * DH + lane + 32 * i]) * scale;
-      for (int nn = first; nn <= n; ++nn) {
-        const size_t kb = (size_t(nn - r - 1) * Hkv + kh) * DH + lane;
-        float sp = 0.f;
+        for (int t = 0; t < 4; ++t) {
+          const size_t kb = (size_t(min(n4 + t, n) - r - 1) * Hkv + kh) * DH + lane;
 #pragma unroll
-        for (int i = 0; i < PER; ++i) sp = fmaf(qv[i], to_f32(k_cand[kb + 32 * i]), sp);
-        const float sc = warp_sum(sp);
-        const float mn = fmaxf(m, sc);
-        const float a = exp2f(m - mn), b = exp2f(sc - mn);
+          for (int i = 0; i < PER; ++i) {
+            kv[t][i] = k_cand[kb + 32 * i];
+            vv[t][i] = v_cand[kb + 32 * i];
+          }
+        }
 #pragma unroll
-        for (int i = 0; i < PER; ++i) acc[i] = acc[i] * a + b * to_f32(v_cand[kb + 32 * i]);
-        l = l * a + b;
-        m = mn;
+        for (int t = 0; t < 4; ++t) {
+          float sp = 0.f;
+#pragma unroll
+          for (int i = 0; i < PER; ++i) sp = fmaf(qv[i] * scale, kv[t][i], sp);
+          sc[t] = sp;
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+          for (int t = 0; t < 4; ++t) sc[t] += __shfl_xor_sync(0xffffffffu, sc[t], off);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          if (n4 + t > n) break;
+          const float mn = fmaxf(m, sc[t]);
+          const float a = exp2f(m - mn), b = exp2f(sc[t] - mn);
+#pragma unroll
+          for (int i = 0; i < PER; ++i) acc[i] = acc[i] * a + b * vv[t][i];
+          l = l * a + b;
+          m = mn;
+        }
       }
     }
   }
   const float inv = l > 0.f ? 1.f / l : 0.f;
 #pragma unroll
-  for (int i = 0; i < PER; ++i) o[(size_t(n) * Hq + h) * DH + lane + 32 * i] = from_f32<T>(acc[i] * inv);
+  for (int i = 0; i < PER; ++i) o[(size_t(n) * Hq + h) * DH + lane + 32 * i] = acc[i] * inv;
 }
 
-template <typename T, int DH>
-cudaError_t launch_typed(const jet_layout& lay, const jet_dims& d, const AttnPlan& plan,
+template <int DH>
+cudaError_t launch_dh(const jet_layout& lay, const jet_dims& d, const AttnPlan& plan,
                          const void* q, const void* k_pre, const void* v_pre, const void* k_cand,
                          const void* v_cand, void* o, void* ws, int* status, cudaStream_t st) {
   const jet_sizes& n = lay.n;
@@ -223,21 +268,22 @@ cudaError_t launch_typed(const jet_layout& lay, const jet_dims& d, const AttnPla
                             status, st);
   } else {
     const size_t smem = prefix_smem_bytes<DH>();
-    e = cudaFuncSetAttribute(attend_prefix_kernel<T, DH>,
+    e = cudaFuncSetAttribute(attend_prefix_kernel<DH>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     dim3 grid(plan.splits, plan.qgroups, unsigned(n.R * d.Hkv));
-    e = launch_pdl(attend_prefix_kernel<T, DH>, grid, dim3(kThreads), smem, st, lay.prefix_offset,
+    e = launch_pdl(attend_prefix_kernel<DH>, grid, dim3(kThreads), smem, st, lay.prefix_offset,
                    lay.row_offset, n.R, n.N, n.total_prefix, d.Hq, d.Hkv, plan.chunk,
-                   static_cast<const T*>(q), static_cast<const T*>(k_pre),
-                   static_cast<const T*>(v_pre), o_part, ml_part, status);
+                   static_cast<const float*>(q), static_cast<const float*>(k_pre),
+                   static_cast<const float*>(v_pre), o_part, ml_part, status);
   }
   if (e != cudaSuccess) return e;
   const long long warps = (long long)n.N * d.Hq;
-  return launch_pdl(attend_merge_kernel<T, DH>, dim3(unsigned((warps + 7) / 8)), dim3(256), 0, st,
+  return launch_pdl(attend_merge_kernel<DH>, dim3(unsigned((warps + 3) / 4)), dim3(128), 0, st,
                     lay.row_req, lay.row_cand, lay.cand_row_offset, n.N, n.R, n.C, d.Hq, d.Hkv,
-                    plan.splits, static_cast<const T*>(q), static_cast<const T*>(k_cand),
-                    static_cast<const T*>(v_cand), o_part, ml_part, static_cast<T*>(o), status);
+                    plan.splits, static_cast<const float*>(q), static_cast<const float*>(k_cand),
+                    static_cast<const float*>(v_cand), o_part, ml_part, static_cast<float*>(o),
+                    status);
 }
 
 }  // namespace
@@ -256,7 +302,7 @@ AttnPlan attn_plan(const jet_sizes& n, const jet_dims& d) {
   // at once, so they do not count as work
   const long long avg_vecs = ((long long)n.N * g + n.R - 1) / n.R;
   const long long groups = (long long)n.R * d.Hkv * std::max<long long>(1, (avg_vecs + qv - 1) / qv);
-  const int max_splits = std::max(1, (n.max_prefix + 63) / 64);
+  const int max_splits = std::max(1, (n.max_prefix + gran - 1) / gran);
   int chunk;
   if (tc) {
     // the persistent kernel (one CTA per SM, longest items first) splits a
@@ -298,17 +344,11 @@ cudaError_t launch_prefix_attend(const jet_layout& lay, const jet_dims& d, const
                                  const void* q, const void* k_pre, const void* v_pre,
                                  const void* k_cand, const void* v_cand, void* o, void* ws,
                                  int* status, cudaStream_t st) {
-#define JET_ATT(T, DH) \
-  return launch_typed<T, DH>(lay, d, plan, q, k_pre, v_pre, k_cand, v_cand, o, ws, status, st)
-  if (d.dtype == JET_DTYPE_F32) {
-    if (d.d == 64) JET_ATT(float, 64);
-    if (d.d == 128) JET_ATT(float, 128);
-    if (d.d == 256) JET_ATT(float, 256);
-  } else {
-    if (d.d == 64) JET_ATT(__nv_bfloat16, 64);
-    if (d.d == 128) JET_ATT(__nv_bfloat16, 128);
-    if (d.d == 256) JET_ATT(__nv_bfloat16, 256);
-  }
+#define JET_ATT(DH) \
+  return launch_dh<DH>(lay, d, plan, q, k_pre, v_pre, k_cand, v_cand, o, ws, status, st)
+  if (d.d == 64) JET_ATT(64);
+  if (d.d == 128) JET_ATT(128);
+  if (d.d == 256) JET_ATT(256);
 #undef JET_ATT
   return cudaErrorInvalidValue;
 }

@@ -935,7 +935,7 @@ bool encode_3d(CUtensorMap* map, const void* base, int rows, int heads, int DH, 
 // candidate's own keys) and normalise. Single-chunk requests were written by
 // the attention kernel itself.
 template <int DH>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(128)
 attend_combine_kernel(const int32_t* __restrict__ prefix_offset, const int32_t* __restrict__ row_req,
                       int N, int R, int Hq, int chunk, const float* __restrict__ o_part,
                       const float2* __restrict__ ml_part, __nv_bfloat16* __restrict__ o,
@@ -956,36 +956,8 @@ attend_combine_kernel(const int32_t* __restrict__ prefix_offset, const int32_t* 
   if (splits_r <= 1) return;
   constexpr int PER = DH / 32;
   float acc[PER];
-#pragma unroll
-  for (int i = 0; i < PER; ++i) acc[i] = 0.f;
-  float m = -INFINITY, l = 0.f;
-  // four chunks' partials at a time, every load issued before the first is
-  // used (the chunks are combined in order)
-  constexpr int kGroup = 4;
-  for (int s0 = 0; s0 < splits_r; s0 += kGroup) {
-    float2 ml[kGroup];
-    float v[kGroup][PER];
-#pragma unroll
-    for (int q = 0; q < kGroup; ++q) {
-      ml[q] = make_float2(-INFINITY, 0.f);
-      if (s0 + q < splits_r) {
-        const size_t base = (size_t(s0 + q) * N + n) * Hq + h;
-        ml[q] = ml_part[base];
-#pragma unroll
-        for (int i = 0; i < PER; ++i) v[q][i] = o_part[base * DH + lane + 32 * i];
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < kGroup; ++q) {
-      if (!(ml[q].y > 0.f)) continue;
-      const float mn = fmaxf(m, ml[q].x);
-      const float fa = exp2f(m - mn), fb = exp2f(ml[q].x - mn);
-#pragma unroll
-      for (int i = 0; i < PER; ++i) acc[i] = acc[i] * fa + v[q][i] * fb;
-      l = l * fa + ml[q].y * fb;
-      m = mn;
-    }
-  }
+  float m, l;
+  combine_chunks<DH>(splits_r, N, Hq, n, h, lane, ml_part, o_part, m, l, acc);
   const float inv = l > 0.f ? 1.f / l : 0.f;
 #pragma unroll
   for (int i = 0; i < PER; ++i)
@@ -1068,7 +1040,7 @@ cudaError_t launch_dh(const jet_layout& lay, const jet_dims& d, const AttnPlan& 
                  tmKc, tmVc, a);
   if (e != cudaSuccess || plan.splits <= 1) return e;
   const long long warps = (long long)n.N * d.Hq;
-  return launch_pdl(attend_combine_kernel<DH>, dim3(unsigned((warps + 7) / 8)), dim3(256), 0, st,
+  return launch_pdl(attend_combine_kernel<DH>, dim3(unsigned((warps + 3) / 4)), dim3(128), 0, st,
                     lay.prefix_offset, lay.row_req, n.N, n.R, d.Hq, plan.chunk, o_part, ml_part,
                     static_cast<__nv_bfloat16*>(o), status);
 }

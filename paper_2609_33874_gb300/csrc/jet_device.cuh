@@ -67,4 +67,64 @@ __device__ __forceinline__ void ms_combine2(float& m, float& s, float m2, float 
   m = mn;
 }
 
+// A warp combines the base-2 partials (m, l, O) of row n, head h over its prefix
+// chunks: l and acc (elements lane + 32 i of the head) relative to m, the largest
+// of their maxima. The (m, l) of 32 chunks are read one a lane and the chunks'
+// outputs four at a time, the first four beside the (m, l): up to four chunks
+// cost one memory latency (64 requests of 100 - 2,000 keys: the whole call 47.9 ->
+// 46.0 us; eight at a time 48.1 us; one 6,000-key request in 19 chunks 18.9 ->
+// 18.5 us).
+template <int DH>
+__device__ __forceinline__ void combine_chunks(int splits, int N, int Hq, int n, int h, int lane,
+                                               const float2* __restrict__ ml_part,
+                                               const float* __restrict__ o_part, float& m,
+                                               float& l, float (&acc)[DH / 32]) {
+  constexpr int PER = DH / 32, kGroup = 4;
+  const size_t base = size_t(n) * Hq + h, step = size_t(N) * Hq;
+  float v[kGroup][PER];
+  auto load = [&](int s0) {
+#pragma unroll
+    for (int g = 0; g < kGroup; ++g) {
+      if (s0 + g < splits) {
+        const float* p = o_part + (base + size_t(s0 + g) * step) * DH + lane;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) v[g][i] = p[32 * i];
+      }
+    }
+  };
+  m = -INFINITY;
+  l = 0.f;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) acc[i] = 0.f;
+  auto load_ml = [&](int s32) {
+    return s32 + lane < splits ? ml_part[base + size_t(s32 + lane) * step]
+                               : make_float2(-INFINITY, 0.f);
+  };
+  float2 ml = load_ml(0);
+  load(0);
+  for (int s32 = 0; s32 < splits; s32 += 32) {
+    if (s32 > 0) ml = load_ml(s32);
+    if (!(ml.y > 0.f)) ml = make_float2(-INFINITY, 0.f);  // an empty chunk
+    const float mn = fmaxf(m, warp_max(ml.x));
+    const float keep = mn == -INFINITY ? 1.f : exp2f(m - mn);
+    const float w = ml.x == -INFINITY ? 0.f : exp2f(ml.x - mn);
+    l = l * keep + warp_sum(ml.y * w);
+    m = mn;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) acc[i] *= keep;
+    for (int s0 = s32; s0 < min(s32 + 32, splits); s0 += kGroup) {
+      if (s0 > 0) load(s0);
+#pragma unroll
+      for (int g = 0; g < kGroup; ++g) {
+        const float ws = __shfl_sync(0xffffffffu, w, (s0 + g) & 31);
+        // an empty chunk's outputs were not written
+        if (s0 + g < splits && ws > 0.f) {
+#pragma unroll
+          for (int i = 0; i < PER; ++i) acc[i] = fmaf(ws, v[g][i], acc[i]);
+        }
+      }
+    }
+  }
+}
+
 }  // namespace jet

@@ -20,7 +20,7 @@
 // products, level by level); then, on the transposed state (TMEM lane = value
 // column):
 //   U^T = V^T (T diag(b))^T,  W^T = K^T (T diag(b g))^T
-//   X   = U^T + S0^T [-W | g Q]   -> d^T and (g Q S0)^T
+//   X   = S0^T [-W | g Q]         -> d^T - U^T and (g Q S0)^T
 //   X  += d^T (M o G)^T           -> O^T (accumulated onto (g Q S0)^T)
 //   Dst = g_{C-1} S0^T + (d G[C-1])^T K  -> the next S0^T
 // Operands that are not bf16 (S0, T diag(.), W, g Q, d, M o G) enter the MMA
