@@ -207,7 +207,7 @@ attend_merge_kernel(const int32_t* __restrict__ row_req, const int32_t* __restri
   for (int i = 0; i < PER; ++i) qv[i] = q[(size_t(n) * Hq + h) * DH + lane + 32 * i];
   float acc[PER];
   float m, l;
-  combine_chunks<DH>(splits, N, Hq, n, h, lane, ml_part, o_part, m, l, acc);
+  combine_chunks<DH>(true, splits, N, Hq, n, h, lane, ml_part, o_part, m, l, acc);
   if (c >= 0) {
     const int first = (c < C) ? cand_row_offset[c] : -1;
     if (first < 0 || first > n || r < 0 || first - r - 1 < 0 || n - r - 1 >= N - R) {

@@ -22,8 +22,17 @@
 //               they write its output through shared memory (coalesced).
 //   warp 6      scheduler: claims work items one ahead, computes their
 //               geometry and starts their query block on the way into L2.
-// The CTA writes its unnormalised O and (m, l) as a partial; the merge kernel
-// combines the chunks with the candidates' own causal keys.
+// The last chunk also takes the candidates' own keys. A chunk's unnormalised O and
+// (m, l) are a partial that the combine kernel merges; a request of one chunk is
+// written directly.
+//
+// Small calls are bound by a chain of latencies, not by bandwidth: layout -> Q and
+// K -> first S 5.4 us, 0.93 us a 64-key tile, the output 3.3 - 4.3 us, the combine
+// and its launch 5 us. So the scheduler reads up to 32 requests' offsets in one
+// latency, what the output does not need O for is done under the last P V, O leaves
+// TMEM 128 columns at a time, and the chunks' (m, l) tell the combine all it needs
+// (one 6,000-key request 18.4 -> 17.2 us, 16 of 200 - 1,200 keys 24.5 -> 23.2 us,
+// one of 500 keys 14.3 -> 13.1 us, 32 of 2,048 - 8,192 keys 86.0 -> 85.0 us).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -143,6 +152,9 @@ struct ItemGeo {
   bool ok;
 };
 
+__device__ __forceinline__ ItemGeo item_geo_at(const AttArgs& a, int4 it, int n0, int nr, int p0,
+                                               int P);
+
 __device__ __forceinline__ ItemGeo item_geo(const AttArgs& a, int4 it) {
   ItemGeo e{};
   e.r = it.x;
@@ -174,10 +186,25 @@ __device__ __forceinline__ ItemGeo item_geo(const AttArgs& a, int4 it) {
     e.ok = true;
     return e;
   }
-  e.n0 = a.row_offset[e.r];
-  e.nr = a.row_offset[e.r + 1] - e.n0;
-  e.p0 = a.prefix_offset[e.r];
-  e.P = a.prefix_offset[e.r + 1] - e.p0;
+  const int n0 = a.row_offset[e.r], p0 = a.prefix_offset[e.r];
+  return item_geo_at(a, it, n0, a.row_offset[e.r + 1] - n0, p0, a.prefix_offset[e.r + 1] - p0);
+}
+
+// The same of a scoring item whose request's rows [n0, n0 + nr) and prefix
+// [p0, p0 + P) are at hand.
+__device__ __forceinline__ ItemGeo item_geo_at(const AttArgs& a, int4 it, int n0, int nr, int p0,
+                                               int P) {
+  ItemGeo e{};
+  e.r = it.x;
+  e.kh = it.y;
+  const int qb = it.z;
+  e.split = it.w;
+  e.ok = false;
+  if (e.r < 0 || e.r >= a.R || e.kh < 0 || e.kh >= a.Hkv) return e;
+  e.n0 = n0;
+  e.nr = nr;
+  e.p0 = p0;
+  e.P = P;
   if (e.n0 < 0 || e.nr < 1 || e.n0 + e.nr > a.N || e.p0 < 0 || e.P < 1 ||
       e.p0 + e.P > a.total_prefix)
     return e;
@@ -269,25 +296,65 @@ attend_items_kernel(const AttArgs a, int qgroups, int splits) {
   }
 }
 
+// The offsets of the requests a lane stands for: its request in the order, its
+// rows [n0, n0 + nr) and its prefix [p0, p0 + P).
+struct LaneReq {
+  int r, n0, nr, p0, P;
+};
+
+// The requests [base, base + 32) of the order, one a lane.
+__device__ __forceinline__ LaneReq lane_req(const AttArgs& a, int base, int lane) {
+  LaneReq q{-1, 0, 0, 0, 0};
+  const int ri = base + lane;
+  if (a.R <= 32) {
+    // all offsets beside the order, then one lane from another: one memory
+    // latency instead of two before the kernel's first loads
+    int p0 = 0, p1 = 0, n0 = 0, n1 = 0;
+    if (lane < a.R) {
+      q.r = a.req_order[lane];
+      p0 = a.prefix_offset[lane];
+      p1 = a.prefix_offset[lane + 1];
+      n0 = a.row_offset[lane];
+      n1 = a.row_offset[lane + 1];
+    }
+    const bool in = q.r >= 0 && q.r < a.R;
+    const int src = in ? q.r : 0;
+    q.p0 = __shfl_sync(0xffffffffu, p0, src);
+    q.P = __shfl_sync(0xffffffffu, p1 - p0, src);
+    q.n0 = __shfl_sync(0xffffffffu, n0, src);
+    q.nr = __shfl_sync(0xffffffffu, n1 - n0, src);
+    if (!in) q = LaneReq{-1, 0, 0, 0, 0};
+  } else if (ri < a.R) {
+    const int r = a.req_order[ri];
+    if (r >= 0 && r < a.R) {
+      q.r = r;
+      q.p0 = a.prefix_offset[r];
+      q.P = a.prefix_offset[r + 1] - q.p0;
+      q.n0 = a.row_offset[r];
+      q.nr = a.row_offset[r + 1] - q.n0;
+    }
+  }
+  return q;
+}
+
 // The k-th work item of the unsorted order - requests by decreasing prefix
 // length (req_order); within a request kv head, query block and chunk, the
 // chunk fastest - counting only items that have keys and vectors. One warp
 // scans the requests' item counts 32 at a time; false past the last item.
-__device__ __forceinline__ bool nth_item(const AttArgs& a, int k, int lane, int4* out) {
+// The geometry comes with it; `q` holds the requests when `held` (up to 32: read
+// once per CTA).
+__device__ __forceinline__ bool nth_item(const AttArgs& a, int k, int lane, LaneReq& q, bool& held,
+                                         int4* out, ItemGeo* geo) {
   int before = 0;
   for (int base = 0; base < a.R; base += 32) {
-    const int ri = base + lane;
-    int cnt = 0, r = 0, nq = 0, sp = 0;
-    if (ri < a.R) {
-      r = a.req_order[ri];
-      if (r >= 0 && r < a.R) {
-        const int P = a.prefix_offset[r + 1] - a.prefix_offset[r];
-        const int nr = a.row_offset[r + 1] - a.row_offset[r];
-        int per = 0;
-        sp = P >= 1 ? req_splits(P, a.chunk, &per) : 0;
-        nq = nr >= 1 ? (nr + a.rb - 1) / a.rb : 0;
-        cnt = a.Hkv * nq * sp;
-      }
+    if (!held) q = lane_req(a, base, lane);
+    held = a.R <= 32;
+    int cnt = 0, nq = 0, sp = 0;
+    if (q.r >= 0) {
+      int per = 0;
+      sp = q.P >= 1 ? req_splits(q.P, a.chunk, &per) : 0;
+      nq = q.nr >= 1 ? (q.nr + a.rb - 1) / a.rb : 0;
+      cnt = a.Hkv * nq * sp;
     }
     int inc = cnt;
 #pragma unroll
@@ -300,11 +367,14 @@ __device__ __forceinline__ bool nth_item(const AttArgs& a, int k, int lane, int4
       const unsigned hit = __ballot_sync(0xffffffffu, k < before + inc);
       const int src = __ffs(hit) - 1;
       const int kk = k - before - __shfl_sync(0xffffffffu, inc - cnt, src);
-      r = __shfl_sync(0xffffffffu, r, src);
+      const int r = __shfl_sync(0xffffffffu, q.r, src);
       nq = __shfl_sync(0xffffffffu, nq, src);
       sp = __shfl_sync(0xffffffffu, sp, src);
       const int split = kk % sp, rest = kk / sp;
       *out = make_int4(r, rest / nq, rest % nq, split);
+      *geo = item_geo_at(a, *out, __shfl_sync(0xffffffffu, q.n0, src),
+                         __shfl_sync(0xffffffffu, q.nr, src), __shfl_sync(0xffffffffu, q.p0, src),
+                         __shfl_sync(0xffffffffu, q.P, src));
       return true;
     }
     before += total;
@@ -409,6 +479,8 @@ attend_prefix_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
   if (warp == kSchedWarp) {
     // ---------------------------------------------------------------- scheduler
     const int count = a.sorted ? *a.item_count : 0;
+    LaneReq reqs{};
+    bool held = false;
     for (int u = 0;; ++u) {
       const int slot = u & 1;
       bool okw = true;
@@ -448,8 +520,8 @@ attend_prefix_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
         const int n = int(gridDim.x);
         const int k = u * n + ((u & 1) ? n - 1 - int(blockIdx.x) : int(blockIdx.x));
         int4 cand;
-        if (k < a.n_all && nth_item(a, k, lane, &cand)) {
-          const ItemGeo ce = item_geo(a, cand);
+        ItemGeo ce;
+        if (k < a.n_all && nth_item(a, k, lane, reqs, held, &cand, &ce)) {
           if (ce.ok) {
             it = cand;
             e = ce;
@@ -801,81 +873,88 @@ attend_prefix_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
         if (lane == 0) mbar_arrive(p_full + b);
       }
       if (!ok) break;
-      // wait for the item's last P V, then write its output (or its partial)
+      // the item's output (or its partial) goes out once its last P V is done; what
+      // does not depend on that comes first: the destinations of the vectors this
+      // lane stores (4 s + lane / 8, 16 bytes each), as element offsets, -1 past the
+      // block's vectors
+      const bool direct = e.splits_r == 1;  // the whole row in this item: final output
+      long long dst[8];
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        const int gi = q4 * 32 + 4 * s + (lane >> 3);
+        dst[s] = -1;
+        if (gi < e.nv) {
+          const int gv = e.vbase + gi;
+          const int n = e.n0 + gv / g, h = e.kh * g + gv % g;
+          dst[s] = (long long)(size_t(direct ? n : e.split * (long long)a.N + n) * a.Hq + h) * DH;
+        }
+      }
+      if (valid && a.splits > 1) {
+        // this chunk's (m, l); a request's last chunk also marks the chunks that
+        // it does not have as empty, and an output written directly by l = -1, so
+        // that the combine needs nothing else to know
+        const int gv = e.vbase + i;
+        const size_t at = size_t(e.n0 + gv / g) * a.Hq + e.kh * g + gv % g;
+        const size_t step = size_t(a.N) * a.Hq;
+        a.ml_part[at + (direct ? 0 : e.split * step)] =
+            direct ? make_float2(0.f, -1.f) : make_float2(m_used, l);
+        if (!direct && e.split == e.splits_r - 1)
+          for (int sp = e.splits_r; sp < a.splits; ++sp)
+            a.ml_part[at + sp * step] = make_float2(-INFINITY, 0.f);
+      }
+      const float inv = l > 0.f ? 1.f / l : 0.f;
       const int Tl = T + e.ntiles - 1;
       if (!warp_mbar_wait(p_free + (Tl & 1), (Tl >> 1) & 1, a.wait_ns, abort_flag)) {
         ok = false;
         break;
       }
       tc_fence_after();
-      const bool direct = e.splits_r == 1;  // the whole row in this item: final output
-      if (valid) {
-        const int gv = e.vbase + i;
-        const int n = e.n0 + gv / g, h = e.kh * g + gv % g;
-        if (!direct) a.ml_part[(size_t(e.split) * a.N + n) * a.Hq + h] = make_float2(m_used, l);
-      }
-      // the destination of the vectors this lane stores: vector 4 s + lane / 8
-      // (f32 partial, 8 lanes x 16 bytes each) or 8 s + lane / 4 (bf16 output,
-      // 4 lanes x 16 bytes each); element offsets, -1 past the block's vectors
-      long long dst[8];
+      // 128 (or all 64) columns of O per TMEM round trip, written as 128-byte pieces
+      // of each vector (64 bf16 or 32 f32 columns) through this warp's 4 KB stage:
+      // eight 16-byte pieces a row, rotated by the row
+      constexpr int kCols = DH < 128 ? DH : 128;
+      auto put_piece = [&](const uint4(&x)[8], char* base, size_t esize, int col) {
 #pragma unroll
-      for (int s = 0; s < 8; ++s) {
-        const int iv = direct ? 8 * s + (lane >> 2) : 4 * s + (lane >> 3);
-        const int gi = q4 * 32 + iv;
-        dst[s] = -1;
-        if ((!direct || s < 4) && gi < e.nv) {
-          const int gv = e.vbase + gi;
-          const int n = e.n0 + gv / g, h = e.kh * g + gv % g;
-          dst[s] = direct ? (long long)(size_t(n) * a.Hq + h) * DH
-                          : (long long)((size_t(e.split) * a.N + n) * a.Hq + h) * DH;
+        for (int q = 0; q < 8; ++q) stage[lane * 8 + (q ^ (lane & 7))] = x[q];
+        __syncwarp();
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+          const int iv = 4 * s + (lane >> 3), c = lane & 7;
+          const uint4 val = stage[iv * 8 + (c ^ (iv & 7))];
+          if (dst[s] >= 0)
+            *reinterpret_cast<uint4*>(base + (dst[s] + col) * esize + c * 16) = val;
         }
-      }
-      const float inv = l > 0.f ? 1.f / l : 0.f;
-      // 64 columns of O per TMEM round trip, written as two 32-column pieces
+        __syncwarp();
+      };
 #pragma unroll 1
-      for (int c0 = 0; c0 < DH; c0 += 64) {
-        float ovp[2][32];
-        tmem_ld_32cols(tmem + lane_off + G::kOCol + c0, ovp[0]);
-        tmem_ld_32cols(tmem + lane_off + G::kOCol + c0 + 32, ovp[1]);
+      for (int c0 = 0; c0 < DH; c0 += kCols) {
+        float ov[kCols / 32][32];
+#pragma unroll
+        for (int k = 0; k < kCols / 32; ++k)
+          tmem_ld_32cols(tmem + lane_off + G::kOCol + c0 + 32 * k, ov[k]);
         tmem_wait_ld();
+        if (direct) {
 #pragma unroll
-        for (int hp = 0; hp < 2; ++hp) {
-          const float* ov = ovp[hp];
-          const int cc0 = c0 + 32 * hp;
-          if (direct) {
-            // 32 bf16 = four 16-byte pieces per vector; two vectors per 128-byte
-            // row of the stage, pieces rotated so that 8 lanes hit 8 bank groups
+          for (int k = 0; k < kCols / 32; k += 2) {
+            uint4 x[8];
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-              stage[(lane >> 1) * 8 + (lane & 1) * 4 + (q ^ ((lane >> 1) & 3))] =
-                  make_uint4(pack_bf16(ov[8 * q] * inv, ov[8 * q + 1] * inv),
-                             pack_bf16(ov[8 * q + 2] * inv, ov[8 * q + 3] * inv),
-                             pack_bf16(ov[8 * q + 4] * inv, ov[8 * q + 5] * inv),
-                             pack_bf16(ov[8 * q + 6] * inv, ov[8 * q + 7] * inv));
-            __syncwarp();
-#pragma unroll
-            for (int s = 0; s < 4; ++s) {
-              const int iv = 8 * s + (lane >> 2), c = lane & 3;
-              const uint4 val = stage[(iv >> 1) * 8 + (iv & 1) * 4 + (c ^ ((iv >> 1) & 3))];
-              if (dst[s] >= 0) *reinterpret_cast<uint4*>(a.o + dst[s] + cc0 + c * 8) = val;
+            for (int q = 0; q < 8; ++q) {
+              const float* y = ov[k + (q >> 2)] + 8 * (q & 3);
+              x[q] = make_uint4(pack_bf16(y[0] * inv, y[1] * inv), pack_bf16(y[2] * inv, y[3] * inv),
+                                pack_bf16(y[4] * inv, y[5] * inv), pack_bf16(y[6] * inv, y[7] * inv));
             }
-          } else {
-            // 32 f32 = eight 16-byte pieces per vector, one vector per 128-byte
-            // row of the stage, pieces rotated by the row
+            put_piece(x, reinterpret_cast<char*>(a.o), 2, c0 + 32 * k);
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < kCols / 32; ++k) {
+            uint4 x[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q)
-              stage[lane * 8 + (q ^ (lane & 7))] =
-                  make_uint4(__float_as_uint(ov[4 * q]), __float_as_uint(ov[4 * q + 1]),
-                             __float_as_uint(ov[4 * q + 2]), __float_as_uint(ov[4 * q + 3]));
-            __syncwarp();
-#pragma unroll
-            for (int s = 0; s < 8; ++s) {
-              const int iv = 4 * s + (lane >> 3), c = lane & 7;
-              const uint4 val = stage[iv * 8 + (c ^ (iv & 7))];
-              if (dst[s] >= 0) *reinterpret_cast<uint4*>(a.o_part + dst[s] + cc0 + c * 4) = val;
-            }
+              x[q] = make_uint4(__float_as_uint(ov[k][4 * q]), __float_as_uint(ov[k][4 * q + 1]),
+                                __float_as_uint(ov[k][4 * q + 2]), __float_as_uint(ov[k][4 * q + 3]));
+            put_piece(x, reinterpret_cast<char*>(a.o_part), 4, c0 + 32 * k);
           }
-          __syncwarp();
         }
       }
       // O may be overwritten by the next item's first P V; the ring slot is free
@@ -933,11 +1012,13 @@ bool encode_3d(CUtensorMap* map, const void* base, int rows, int heads, int DH, 
 // One warp per (row, query head) of a request whose prefix spans several
 // chunks: combine the chunks' base-2 partials (the last chunk also holds the
 // candidate's own keys) and normalise. Single-chunk requests were written by
-// the attention kernel itself.
+// the attention kernel itself; it also left every chunk's (m, l) in place, empty
+// for the chunks a request does not have, so that nothing here waits for the
+// layout.
 template <int DH>
 __global__ void __launch_bounds__(128)
-attend_combine_kernel(const int32_t* __restrict__ prefix_offset, const int32_t* __restrict__ row_req,
-                      int N, int R, int Hq, int chunk, const float* __restrict__ o_part,
+attend_combine_kernel(const int32_t* __restrict__ row_req, int N, int R, int Hq, int splits,
+                      const float* __restrict__ o_part,
                       const float2* __restrict__ ml_part, __nv_bfloat16* __restrict__ o,
                       int* status) {
   pdl_begin();
@@ -946,18 +1027,23 @@ attend_combine_kernel(const int32_t* __restrict__ prefix_offset, const int32_t* 
   if (idx >= (long long)N * Hq) return;
   const int n = int(idx / Hq), h = int(idx % Hq);
   const int r = row_req[n];
+  // written by the attention kernel itself (l = -1 in the first chunk's place)
+  const bool direct = ml_part[size_t(n) * Hq + h].y < 0.f;
+  // partials read beside their (m, l), wanted or not, while the grid is one that
+  // the chip holds at once: then a memory latency is all that counts (one request
+  // of 500 keys 13.5 -> 13.1 us); in a larger grid the rows of short requests are
+  // traffic (64 requests of 100 - 2,000 keys 46.4 -> 48.2 us)
+  const bool ahead = gridDim.x <= 152 * 8;
+  if (!ahead && direct) return;
+  constexpr int PER = DH / 32;
+  float acc[PER];
+  float m, l;
+  combine_chunks<DH>(ahead, splits, N, Hq, n, h, lane, ml_part, o_part, m, l, acc);
   if (r < 0 || r >= R) {
     if (lane == 0) flag(status, JET_ERR_DEVICE);
     return;
   }
-  const int P = prefix_offset[r + 1] - prefix_offset[r];
-  int per = 0;
-  const int splits_r = req_splits(P, chunk, &per);
-  if (splits_r <= 1) return;
-  constexpr int PER = DH / 32;
-  float acc[PER];
-  float m, l;
-  combine_chunks<DH>(splits_r, N, Hq, n, h, lane, ml_part, o_part, m, l, acc);
+  if (direct) return;
   const float inv = l > 0.f ? 1.f / l : 0.f;
 #pragma unroll
   for (int i = 0; i < PER; ++i)
@@ -1041,7 +1127,7 @@ cudaError_t launch_dh(const jet_layout& lay, const jet_dims& d, const AttnPlan& 
   if (e != cudaSuccess || plan.splits <= 1) return e;
   const long long warps = (long long)n.N * d.Hq;
   return launch_pdl(attend_combine_kernel<DH>, dim3(unsigned((warps + 3) / 4)), dim3(128), 0, st,
-                    lay.prefix_offset, lay.row_req, n.N, n.R, d.Hq, plan.chunk, o_part, ml_part,
+                    lay.row_req, n.N, n.R, d.Hq, plan.splits, o_part, ml_part,
                     static_cast<__nv_bfloat16*>(o), status);
 }
 

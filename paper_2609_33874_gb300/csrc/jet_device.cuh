@@ -75,8 +75,8 @@ __device__ __forceinline__ void ms_combine2(float& m, float& s, float m2, float 
 // 46.0 us; eight at a time 48.1 us; one 6,000-key request in 19 chunks 18.9 ->
 // 18.5 us).
 template <int DH>
-__device__ __forceinline__ void combine_chunks(int splits, int N, int Hq, int n, int h, int lane,
-                                               const float2* __restrict__ ml_part,
+__device__ __forceinline__ void combine_chunks(bool ahead, int splits, int N, int Hq, int n, int h,
+                                               int lane, const float2* __restrict__ ml_part,
                                                const float* __restrict__ o_part, float& m,
                                                float& l, float (&acc)[DH / 32]) {
   constexpr int PER = DH / 32, kGroup = 4;
@@ -101,7 +101,7 @@ __device__ __forceinline__ void combine_chunks(int splits, int N, int Hq, int n,
                                : make_float2(-INFINITY, 0.f);
   };
   float2 ml = load_ml(0);
-  load(0);
+  if (ahead) load(0);
   for (int s32 = 0; s32 < splits; s32 += 32) {
     if (s32 > 0) ml = load_ml(s32);
     if (!(ml.y > 0.f)) ml = make_float2(-INFINITY, 0.f);  // an empty chunk
@@ -112,8 +112,10 @@ __device__ __forceinline__ void combine_chunks(int splits, int N, int Hq, int n,
     m = mn;
 #pragma unroll
     for (int i = 0; i < PER; ++i) acc[i] *= keep;
+    const unsigned some = __ballot_sync(0xffffffffu, w > 0.f);
     for (int s0 = s32; s0 < min(s32 + 32, splits); s0 += kGroup) {
-      if (s0 > 0) load(s0);
+      if (!(some >> (s0 & 31) & ((1u << kGroup) - 1))) continue;  // all empty
+      if (!ahead || s0 > 0) load(s0);
 #pragma unroll
       for (int g = 0; g < kGroup; ++g) {
         const float ws = __shfl_sync(0xffffffffu, w, (s0 + g) & 31);

@@ -1,6 +1,8 @@
 """The scoring attention's split and deal of work against the oracle: a few long
-prefixes cut into many chunks, a prefix just past the shortest chunk, and more
-items than CTAs of uneven length (several a CTA, dealt back and forth)."""
+prefixes cut into many chunks, a prefix just past the shortest chunk, more items
+than CTAs of uneven length (several a CTA, dealt back and forth), and more than 32
+requests of one to many chunks (the combine meets rows that are already written
+and chunks that a request does not have)."""
 import dataclasses
 
 import numpy as np
@@ -16,6 +18,7 @@ CASES = [
     ([193], dict(Hq=8, Hkv=2, d=64)),
     ([2049, 100, 700], dict(Hq=32, Hkv=8, d=128)),
     ([1 + 37 * i % 900 for i in range(90)], dict(Hq=24, Hkv=4, d=64)),
+    ([4000] + [50 + 61 * i for i in range(32)], dict(Hq=32, Hkv=8, d=128)),
 ]
 
 
