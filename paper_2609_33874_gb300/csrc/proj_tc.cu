@@ -53,6 +53,10 @@ constexpr int kSmemLimit = 232448;
 // gate/up exchange (16 columns x 128 lanes f32) + barriers and flags
 constexpr int kFixedSmem = 16 * 128 * 4 + 32 * 8 + 64;
 
+// a K range of a split GEMM: the raw f32 partial. Its own kernel: as a branch of the
+// others' epilogues it took 4.5 us more at 178 rows (11.2 -> 15.7 us).
+constexpr int kPartial = 3;
+
 struct ProjArgs {
   __nv_bfloat16* out;
   const __nv_bfloat16* res;
@@ -63,7 +67,7 @@ struct ProjArgs {
   uint32_t tmem_cols, acc_cols;  // two accumulators of acc_cols columns
   uint64_t wait_ns;  // budget of one bounded wait (jet_set_wait_budget_ns)
   int hold_first;    // test hook (jet_set_test_stall): withhold the first stage's loads
-  int vec;           // out 16-byte aligned and ldo % 8 == 0: 16-byte output stores
+  int vec;           // out and res 16-byte aligned and ldo % 8 == 0: 16-byte accesses
 };
 
 // unit u -> (256-row weight slice, K split, token tile); the token tiles of one
@@ -252,11 +256,25 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       const int ot = 2 * x.ot + int(rank);  // this CTA's 128-row weight tile
       const uint32_t tl = tmem_base + uint32_t(buf) * a.acc_cols + (uint32_t(32 * q) << 16);
       for (int c0 = 0; c0 < ncols; c0 += 32) {
+        const int nc = min(32, ncols - c0);
+        // whole 32-feature pieces go out (and the residual comes in) 16 bytes at a
+        // time through this warp's 2 KB of the exchange buffer
+        const int f0 = ot * kBM + 32 * q;  // the warp's first output feature
+        const bool pieces = (EPI == kProjStore || EPI == kProjResid) && a.vec && f0 + 32 <= a.O;
+        uint4 rv[4];
+        if (EPI == kProjResid && pieces) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int e = lane + 32 * k, row = e >> 2, pc = e & 3;
+            if (row < nc)
+              rv[k] = *reinterpret_cast<const uint4*>(a.res + size_t(t0 + c0 + row) * a.ldo + f0 +
+                                                      8 * pc);
+          }
+        }
         float v[32];
         tmem_ld_32cols(tl + uint32_t(c0), v);
         tmem_wait_ld();
-        const int nc = min(32, ncols - c0);
-        if (a.splits > 1) {
+        if (EPI == kPartial) {
           // a K range of a split GEMM: the raw f32 partial
           const int o = ot * kBM + 32 * q + lane;
           if (o < a.O) {
@@ -293,14 +311,24 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
             }
           }
           named_bar_sync(1, 128);
-        } else if (EPI == kProjStore && a.vec && ot * kBM + 32 * q + 32 <= a.O) {
-          // this warp's 32 features x 32 rows through its 2 KB of the exchange
-          // buffer (unused by this epilogue), then 16-byte pieces of each row
+        } else if (pieces) {
+          // the residual's values go where this thread's own outputs then go
           __nv_bfloat16* stg = reinterpret_cast<__nv_bfloat16*>(upx) + q * 1024;
+          if (EPI == kProjResid) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) stg[i * 32 + lane] = __float2bfloat16_rn(v[i]);
+            for (int k = 0; k < 4; ++k) {
+              const int e = lane + 32 * k, row = e >> 2, pc = e & 3;
+              if (row < nc) *reinterpret_cast<uint4*>(stg + row * 32 + 8 * pc) = rv[k];
+            }
+            __syncwarp();
+          }
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            float y = v[i];
+            if (EPI == kProjResid && i < nc) y += __bfloat162float(stg[i * 32 + lane]);
+            stg[i * 32 + lane] = __float2bfloat16_rn(y);
+          }
           __syncwarp();
-          const int f0 = ot * kBM + 32 * q;  // the warp's first output feature
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const int e = lane + 32 * k, row = e >> 2, pc = e & 3;
@@ -310,15 +338,21 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           }
           __syncwarp();
         } else {
-          const int o = ot * kBM + 32 * q + lane;  // output feature
+          const int o = f0 + lane;  // output feature
           if (o < a.O) {
+            // every residual before the first output, which may be the same memory
+            __nv_bfloat16 r[32];
+            if (EPI == kProjResid) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i)
+                if (i < nc) r[i] = a.res[size_t(t0 + c0 + i) * a.ldo + o];
+            }
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
               if (i < nc) {
-                const size_t at = size_t(t0 + c0 + i) * a.ldo + o;
                 float y = v[i];
-                if (EPI == kProjResid) y += __bfloat162float(a.res[at]);
-                a.out[at] = __float2bfloat16_rn(y);
+                if (EPI == kProjResid) y += __bfloat162float(r[i]);
+                a.out[size_t(t0 + c0 + i) * a.ldo + o] = __float2bfloat16_rn(y);
               }
             }
           }
@@ -561,7 +595,8 @@ cudaError_t launch_epi(const void* x, int N, int K, int ldx, const void* w, int 
   a.O = O;
   a.K = K;
   a.ldo = ldo;
-  a.vec = (ldo % 8 == 0) && (reinterpret_cast<uintptr_t>(out) % 16 == 0);
+  a.vec = ldo % 8 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0 &&
+          reinterpret_cast<uintptr_t>(res) % 16 == 0;
   a.Nt = Nt;
   a.n_tt = n_tt;
   a.units = tl.groups * n_tt * a.splits;
@@ -575,7 +610,7 @@ cudaError_t launch_epi(const void* x, int N, int K, int ldx, const void* w, int 
   CUtensorMap tmW, tmX;
   if (!encode_rows(&tmW, w, O, K, K, kBM) || !encode_rows(&tmX, x, N, K, ldx, b_rows))
     return cudaErrorInvalidValue;
-  auto kern = proj_tc_kernel<EPI>;
+  auto kern = a.splits > 1 ? proj_tc_kernel<kPartial> : proj_tc_kernel<EPI>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
   const int clusters = std::max(1, std::min(a.units, max_pairs(kern, smem)));
