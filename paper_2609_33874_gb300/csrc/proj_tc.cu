@@ -556,25 +556,41 @@ struct Tiling {
   int n_tt, Nt, otiles, groups, nkb, splits;  // groups: 256-row weight slices
 };
 
-// token tiles of at most 256 rows (a multiple of 16: each CTA of a pair holds
+// Token tiles of at most 256 rows (a multiple of 16: each CTA of a pair holds
 // half); units of 256 weight rows on CTA pairs; K split while the units still
 // fit the 76 SM pairs once, keeping at least 8 K slices per unit. A function
 // of the shapes only, so that the workspace planned for a call matches the
 // launch.
+// The number of tiles is the one of least cost: rounds of the SM pairs, times K
+// slices a unit, times a slice's time, which goes as Nt + 80 (the weights' share of
+// the bytes an SM takes in; 64 to 110 in place of 80 choose alike but for a few
+// sizes). Always the fewest tiles left the last round half empty: four layers of
+// D 4,096 and Dff 12,288 took 525 us of 178 rows, now 513; 643 of 355, now 634; 715
+// of 444, now 691; 851 of 555, now 808; 1,802 of 2,800, now 1,688. Splits over more
+// than one round gain up to 1 % there, but 355 rows take 1 - 2 % more.
 constexpr int kPlanSMs = 152;
 Tiling tiling(int N, int O, int K, bool split) {
-  Tiling t{};
-  t.n_tt = (N + kMaxNt - 1) / kMaxNt;
-  t.Nt = ((N + t.n_tt - 1) / t.n_tt + 15) / 16 * 16;
-  t.n_tt = (N + t.Nt - 1) / t.Nt;
-  t.otiles = (O + kBM - 1) / kBM;
-  t.groups = (t.otiles + 1) / 2;
-  t.nkb = (K + kBK - 1) / kBK;
-  const int units = t.groups * t.n_tt;
-  t.splits = 1;
-  while (split && units * (t.splits + 1) <= kPlanSMs / 2 && t.nkb / (t.splits + 1) >= 8)
-    ++t.splits;
-  return t;
+  const int pairs = kPlanSMs / 2, least = (N + kMaxNt - 1) / kMaxNt;
+  Tiling best{};
+  long long best_cost = -1;
+  for (int c = least; c <= 2 * least + 2; ++c) {
+    Tiling t{};
+    t.Nt = ((N + c - 1) / c + 15) / 16 * 16;
+    t.n_tt = (N + t.Nt - 1) / t.Nt;
+    t.otiles = (O + kBM - 1) / kBM;
+    t.groups = (t.otiles + 1) / 2;
+    t.nkb = (K + kBK - 1) / kBK;
+    const int units = t.groups * t.n_tt;
+    t.splits = 1;
+    while (split && units * (t.splits + 1) <= pairs && t.nkb / (t.splits + 1) >= 8) ++t.splits;
+    const long long rounds = (units * t.splits + pairs - 1) / pairs;
+    const long long cost = rounds * ((t.nkb + t.splits - 1) / t.splits) * (t.Nt + 80);
+    if (best_cost < 0 || cost < best_cost) {
+      best = t;
+      best_cost = cost;
+    }
+  }
+  return best;
 }
 
 template <int EPI>
