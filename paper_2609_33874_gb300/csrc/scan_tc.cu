@@ -30,7 +30,8 @@
 // chunk instead of the 64^2 / 2 per column of a substitution for all 256
 // columns of U and W.
 //
-// One CTA per (request, head), two groups of eight warps. The solve group works
+// One CTA per SM works through items (request, head), longest requests first, with
+// two groups of eight warps. The solve group works
 // one chunk ahead of the state: it forms A, M o G, T, T diag(b) and T diag(b g)
 // of chunk j + 1 (none of which needs the state) and issues U and W, while the
 // state group runs X, d, O and the new state of chunk j. Lane c of TMEM (value
@@ -39,10 +40,13 @@
 // S, the new operand: 5 to 6 us a chunk) and the instructions of the hi/lo
 // splits (40 % of the issue slots); with one group doing both in turn a chunk
 // took 11 us. 32 requests x 512 tokens x 16 heads: delta rule 338 -> 228 us, gated
-// linear attention 199 -> 147 us; 3 x 2,000 - 4,000 tokens 595 -> 362 and 341 ->
-// 223 us. Where it was lost before: bank conflicts and address arithmetic in the
-// inverse, one chunk's gates scanned inside its chain, outputs written before the
-// next chunk's X.
+// linear attention 199 -> 147 us; 3 x 2,000 - 4,000 tokens 595 -> 359 and 341 ->
+// 222 us. The groups run on from one item into the next: a CTA per item fills and
+// drains this chain every time, and its lengths come in no order (the above 228 ->
+// 220 and 147 -> 141 us; 64 x 64 tokens 89 -> 62 and 64 -> 43 us; 24 x 100 - 4,000
+// tokens 671 -> 500 and 416 -> 319 us). Where it was lost before: bank conflicts and
+// address arithmetic in the inverse, one chunk's gates scanned inside its chain,
+// outputs written before the next chunk's X.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -61,6 +65,7 @@ constexpr int kC = 64;         // tokens per chunk
 constexpr int kD = 128;        // dk = dv handled by this kernel
 constexpr int kGroup = 256;    // threads of one group (solve or state)
 constexpr int kThreads = 2 * kGroup;
+constexpr int kWalker = 160;   // the solve group's thread that steps through the chunks
 constexpr uint64_t kDrainNs = 200000000ull;
 
 // Shared memory (offsets from the 1024-byte aligned base). Operand tiles are
@@ -91,8 +96,13 @@ constexpr uint32_t kOffOut = kOffT + 10 * kBlk * 4;  // a chunk's outputs [64 to
 constexpr uint32_t kVecFloats = 5 * 64 + 4;
 constexpr uint32_t kOffVec = kOffOut + 16384;
 constexpr uint32_t kOffBar = kOffVec + 3 * kVecFloats * 4;
-constexpr uint32_t kSmemBytes = kOffBar + 128 + 1024;
-static_assert(kOffOut % 16 == 0 && kOffVec % 16 == 0 && kOffBar % 8 == 0, "alignment");
+// chunk descriptors {first token, end of the prefix, head, row of (request, head)}
+// of eight chunks in turn; an empty one (no tokens) ends the CTA's sequence
+constexpr uint32_t kOffRing = kOffBar + 128;
+constexpr int kRing = 8;
+constexpr uint32_t kOffWalk = kOffRing + kRing * 16;
+constexpr uint32_t kSmemBytes = kOffWalk + 32 + 1024;
+static_assert(kOffOut % 16 == 0 && kOffVec % 16 == 0 && kOffRing % 16 == 0, "alignment");
 static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
 
 // TMEM columns: [K; Q] K^T at 0 (64); U^T at 64 (64); X = [S0^T (-W) | O^T] at
@@ -312,11 +322,15 @@ __device__ __forceinline__ void decays(float* v, int t, int lane, float a, float
   if (t == kC - 1) v[320] = g;
 }
 
-template <bool DELTA>
+// MANY: more items (request, head) than CTAs, so that a CTA works through several;
+// otherwise CTA i has item i, its chunks are known from its prefix alone, and the
+// walk through the items is left out (with it, one 1,000-token request takes 67.1 us
+// instead of 65.7 under gated linear attention).
+template <bool DELTA, bool MANY>
 __global__ void __launch_bounds__(kThreads, 1)
 scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const int32_t* __restrict__ prefix_offset,
-               int R, int total, int Hl, const float* __restrict__ s_init,
+               const int32_t* __restrict__ req_order, int R, int total, int Hl, const float* __restrict__ s_init,
                const float* __restrict__ alpha, const float* __restrict__ beta,
                __nv_bfloat16* __restrict__ o, float* __restrict__ s_out, int* status,
                uint64_t wait_ns, int hold_first) {
@@ -344,7 +358,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   const int tid = threadIdx.x & (kGroup - 1);  // within the group
   const int grp = tid >> 7;   // warpgroup of the group
   const int c = tid & 127;    // TMEM lane: value column c (and key column c of W)
-  const int h = blockIdx.x, r = blockIdx.y;
+  int4* const ring = reinterpret_cast<int4*>(sm + kOffRing);
   if (threadIdx.x == 0) {
     for (int b = 0; b < 9; ++b) mbar_init(bar_k + b, 1);
     mbar_init(ready, kGroup / 32);
@@ -358,6 +372,74 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     tma_prefetch_desc(&tmV);
   }
   pdl_begin();
+  // This CTA's items, (request, head): request by request in order of decreasing
+  // length, dealt out back and forth (0 .. n-1, n-1 .. 0, ...). `walk` steps
+  // through the chunks of the items that have any; one thread keeps it, in shared
+  // memory (registers are short), with the next item's prefix already read.
+  // R and Hl are at most 65,535, so items and the grid fit 32 bits
+  const unsigned items = unsigned(R) * unsigned(Hl);
+  auto item_at = [&](int u) {
+    return unsigned(u) * gridDim.x + ((u & 1) ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+  };
+  // the item's request and prefix ({-1, 0, 0} past the last item; an empty prefix
+  // for a request the layout does not hold)
+  auto read_item = [&](int u) {
+    const unsigned it = item_at(u);
+    if (it >= items) return make_int3(-1, 0, 0);
+    const int r = MANY ? req_order[it / unsigned(Hl)] : int(it / unsigned(Hl));
+    int a = -1, b = -1;
+    if (r >= 0 && r < R) {
+      a = prefix_offset[r];
+      b = prefix_offset[r + 1];
+    }
+    return make_int3(r, a, b);
+  };
+  struct Walk {
+    int4 cur;   // the chunk to hand out next
+    int3 next;  // the prefix of item u
+    int u;
+  };
+  Walk& walk = *reinterpret_cast<Walk*>(sm + kOffWalk);
+  auto valid = [&](const int3& x) {
+    return x.x >= 0 && x.x < R && x.y >= 0 && x.y <= x.z && x.z <= total;
+  };
+  auto start = [&](int u, int3 x) {  // item u's first chunk; false: it has no tokens
+    if (!valid(x)) {
+      flag(status, JET_ERR_DEVICE);
+      return false;
+    }
+    const int h = int(item_at(u) % unsigned(Hl));
+    walk.cur = make_int4(x.y, x.z, h, x.x * Hl + h);
+    return x.y < x.z;
+  };
+  auto take = [&] {  // the next item that has tokens, or the empty chunk
+    walk.cur = make_int4(0, 0, 0, 0);
+    while (item_at(walk.u) < items) {
+      const int u = walk.u;
+      const int3 x = walk.next;
+      walk.next = read_item(++walk.u);
+      if (start(u, x)) return;
+    }
+  };
+  auto hand_out = [&](int j) {
+    ring[j & (kRing - 1)] = walk.cur;
+    if (walk.cur.x + kC < walk.cur.y)
+      walk.cur.x += kC;
+    else if (walk.cur.x < walk.cur.y)
+      take();
+  };
+  if (MANY && warp == 0) {
+    const int3 x = read_item(lane & 1);  // the first two items at once
+    const int3 x1 = make_int3(__shfl_sync(0xffffffffu, x.x, 1), __shfl_sync(0xffffffffu, x.y, 1),
+                              __shfl_sync(0xffffffffu, x.z, 1));
+    if (lane == 0) {
+      walk.u = 1;
+      walk.next = x1;
+      if (!start(0, x)) take();
+      for (int j = 0; j < 3; ++j) hand_out(j);
+    }
+    __syncwarp();
+  }
   if (warp == 0) {
     tmem_alloc(tslot, 512);
     tmem_relinquish();
@@ -367,17 +449,25 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   tc_fence_after();
   const uint32_t tmem = *tslot;
   const uint32_t lane_off = uint32_t(32 * (warp & 3)) << 16;
-  int p0 = 0, p1 = 0;
-  if (r < R) {
-    p0 = prefix_offset[r];
-    p1 = prefix_offset[r + 1];
+  // chunk j of this CTA's sequence; the walk hands out chunk j + 3 during the solve of
+  // chunk j, which is at most two chunks ahead of the state group
+  // (without MANY: all of it from the item's prefix)
+  int3 only{};
+  if (!MANY) {
+    only = read_item(0);
+    if (!valid(only)) {
+      if (threadIdx.x == 0) flag(status, JET_ERR_DEVICE);
+      only.y = only.z = 0;
+    }
   }
-  if (r >= R || p0 < 0 || p1 < p0 || p1 > total) {
-    if (threadIdx.x == 0) flag(status, JET_ERR_DEVICE);
-    p1 = p0 = 0;
-  }
-  const int nch = (p1 - p0 + kC - 1) / kC;
-  const size_t head = (size_t(r) * Hl + h) * kD;  // row 0 of this (request, head)'s state
+  auto chunk = [&](int j) {
+    if (MANY) return ring[j & (kRing - 1)];
+    return make_int4(only.y + j * kC, only.z, int(blockIdx.x % unsigned(Hl)), int(blockIdx.x));
+  };
+  auto has = [&](int j) {
+    const int4 x = chunk(j);
+    return x.x < x.y;
+  };
   const uint64_t pol = policy_evict_first();
 
   // TMA copies of chunk j's K and Q (into the buffers of its parity) and V. The
@@ -391,9 +481,10 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     par = (par & ~(1u << bit)) | (uint32_t(phase & 1) << bit);
   };
   auto load = [&](const CUtensorMap* map, uint64_t* bar, uint32_t off, uint32_t slice, int j) {
+    const int4 x = chunk(j);
     mbar_arrive_expect_tx(bar, 2 * 8192);
     for (int sl = 0; sl < 2; ++sl)
-      tma_load_3d(sm + off + sl * slice, map, bar, sl * 64, h, p0 + j * kC, pol);
+      tma_load_3d(sm + off + sl * slice, map, bar, sl * 64, x.z, x.x, pol);
   };
   auto load_k = [&](int j) {
     load(&tmK, bar_k + (j & 1), kOffKQ + (j & 1) * kKQBuf, kKQSlice, j);
@@ -426,11 +517,11 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 
   if (role == 0) {
     // ================================================================ solve
-    if (tid == 0 && nch > 0 && !hold_first) {
+    if (tid == 0 && has(0) && !hold_first) {
       load_k(0);
       load_q(0);
       load_v(0);
-      if (nch > 1) {
+      if (has(1)) {
         load_k(1);
         load_q(1);
       }
@@ -441,12 +532,13 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     const int gt = tid - (kGroup - kC);
     float ga = 1.f, go = 1.f, gb = 0.f;  // this token's, and a of the other warp's
     auto read_gates = [&](int j) {
-      const int t = p0 + j * kC + gt, u = p0 + j * kC + (gt ^ 32);
-      ga = t < p1 ? alpha[size_t(t) * Hl + h] : 1.f;
-      gb = t < p1 ? beta[size_t(t) * Hl + h] : 0.f;
-      go = u < p1 ? alpha[size_t(u) * Hl + h] : 1.f;
+      const int4 x = chunk(j);
+      const int t = x.x + gt, u = x.x + (gt ^ 32);
+      ga = t < x.y ? alpha[size_t(t) * Hl + x.z] : 1.f;
+      gb = t < x.y ? beta[size_t(t) * Hl + x.z] : 0.f;
+      go = u < x.y ? alpha[size_t(u) * Hl + x.z] : 1.f;
     };
-    if (gt >= 0 && nch > 0) {
+    if (gt >= 0) {
       read_gates(0);
       decays(vec, gt, lane, ga, go, gb);
       read_gates(1);
@@ -468,10 +560,10 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       return true;
     };
     bool issued = true;  // this thread's loads and MMAs went out
-    if (warp == 0 && nch > 0 && elect_one()) issued = issue_gm(0);
+    if (warp == 0 && has(0) && elect_one()) issued = issue_gm(0);
     __syncwarp();
-    for (int j = 0; j < nch; ++j) {
-      const bool last = j + 1 == nch;
+    for (int j = 0; has(j); ++j) {
+      const bool last = !has(j + 1);  // of the CTA's sequence
       const int odd = j & 1;
       uint8_t* const kt = sm + kOffKQ + odd * kKQBuf;  // this chunk's K (dk-slices kKQSlice apart)
       uint8_t* const mt = sm + kOffM + odd * kMBuf;    // this chunk's M o G
@@ -539,6 +631,8 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         // previous chunk's X has read those
         if (tid < 64 + 6 * 16)
           invert_diagonal(Am, Tm, tid);
+        else if (MANY && tid == kWalker)
+          hand_out(j + 3);
         else if (gt >= 0 && !last) {
           decays(vec + (j + 1) % 3 * kVecFloats, gt, lane, ga, go, gb);
           read_gates(j + 2);
@@ -622,9 +716,10 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         ok = group_and(1, okk);
         if (!ok) break;
         if (lane == 0) mbar_arrive(ready);
+        if (MANY && tid == kWalker) hand_out(j + 3);
         // neither V nor Q is read any more
         if (tid == 0 && !last) load_v(j + 1);
-        if (tid == 0 && j + 2 < nch) load_q(j + 2);
+        if (tid == 0 && has(j + 2)) load_q(j + 2);
         __syncwarp();
         if (warp == 0 && !last && elect_one()) issued = issue_gm(j + 1);
         __syncwarp();
@@ -633,14 +728,33 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     ok = group_and(1, ok && issued);
   } else {
     // ================================================================ state
-    // the initial state: into TMEM (lane c holds S0^T[c][.] = S0[.][c]; this
-    // warpgroup's 64 columns) and as the bf16 hi/lo operand of the first X
-    for (int i0 = 64 * grp; i0 < 64 * grp + 64; i0 += 32) {
-      float v[32];
+    // items without tokens: the state is the initial one (zeros without one); a warp
+    // looks at 32 items at a time
+    for (int u0 = 32 * (warp & 7); item_at(u0) < items; u0 += 32 * (kGroup / 32)) {
+      const int3 x = read_item(u0 + lane);
+      const bool empty = valid(x) && x.y == x.z;
+      for (unsigned m = __ballot_sync(0xffffffffu, empty); m != 0; m &= m - 1) {
+        const int src = __ffs(m) - 1;
+        const int r = __shfl_sync(0xffffffffu, x.x, src);
+        const size_t head = (size_t(r) * Hl + size_t(item_at(u0 + src) % unsigned(Hl))) * kD * kD;
+        for (int i = lane; i < kD * kD; i += 32) s_out[head + i] = s_init ? s_init[head + i] : 0.f;
+      }
+    }
+    // an item's initial state, 32 of this warpgroup's 64 columns at a time: lane c
+    // holds S0^T[c][.] = S0[.][c]
+    auto read_init = [&](const int4& x, int i0, float (&v)[32]) {
+      const float* s0 = s_init + (size_t(x.w) * kD + i0) * kD + c;
 #pragma unroll
-      for (int i = 0; i < 32; ++i) v[i] = s_init ? s_init[(head + i0 + i) * kD + c] : 0.f;
-      tmem_st_32cols(tmem + lane_off + kColSt + i0, v);
-      put32_tmem(tmem + lane_off + kColS0h + (i0 >> 1), tmem + lane_off + kColS0l + (i0 >> 1), v);
+      for (int i = 0; i < 32; ++i) v[i] = s_init ? s0[i * kD] : 0.f;
+    };
+    // the first item's: into TMEM and as the bf16 hi/lo operand of the first X
+    if (has(0)) {
+      for (int i0 = 64 * grp; i0 < 64 * grp + 64; i0 += 32) {
+        float v[32];
+        read_init(chunk(0), i0, v);
+        tmem_st_32cols(tmem + lane_off + kColSt + i0, v);
+        put32_tmem(tmem + lane_off + kColS0h + (i0 >> 1), tmem + lane_off + kColS0l + (i0 >> 1), v);
+      }
     }
     tmem_wait_st();
     tc_fence_before();
@@ -654,16 +768,17 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 #pragma unroll
       for (int i = 0; i < 32; ++i) ost[(32 * grp + i) * kD + c] = __float2bfloat16_rn(ov[i] * rs);
       group_sync(2);
-      const int c0 = p0 + j * kC, n = min(kC, p1 - c0);
-      __nv_bfloat16* const od = o + (size_t(c0 + (tid >> 4)) * Hl + h) * kD + 8 * (tid & 15);
+      const int4 x = chunk(j);
+      const int n = min(kC, x.y - x.x);
+      __nv_bfloat16* const od = o + (size_t(x.x + (tid >> 4)) * Hl + x.z) * kD + 8 * (tid & 15);
 #pragma unroll
       for (int i = 0; i < kC * (kD / 8) / kGroup; ++i)
         if ((tid >> 4) + 16 * i < n)
           *reinterpret_cast<uint4*>(od + size_t(16 * i) * Hl * kD) =
               reinterpret_cast<const uint4*>(ost)[tid + kGroup * i];
     };
-    for (int j = 0; j < nch; ++j) {
-      const bool last = j + 1 == nch;
+    bool pending = false;  // the previous chunk's outputs are still in ov
+    for (int j = 0; has(j); ++j) {
       const int odd = j & 1;
       uint8_t* const kt = sm + kOffKQ + odd * kKQBuf;
       uint8_t* const mt = sm + kOffM + odd * kMBuf;
@@ -692,8 +807,8 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       ok = group_and(2, okk);
       if (!ok) break;
       if (DELTA && tid == 0) {  // this chunk's Q and V are no longer read
-        if (j + 2 < nch) load_q(j + 2);
-        if (!last) load_v(j + 1);
+        if (has(j + 2)) load_q(j + 2);
+        if (has(j + 1)) load_v(j + 1);
       }
       // ---- X = S0^T [-W | g Q] (delta rule) or O^T = S0^T (g Q) (gated linear
       // attention): three hi/lo passes; A (the state, K = dk) from TMEM, 8 packed
@@ -720,7 +835,7 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       // while X runs: the previous chunk's outputs, and this warpgroup's 64 state
       // columns scaled by g_{C-1} for the last MMA to accumulate onto (X reads the
       // hi/lo copy, not these)
-      if (j > 0) write_out(j - 1);
+      if (pending) write_out(j - 1);
       {
         const float g = vec[(j % 3) * kVecFloats + 320];
         float s0[32];
@@ -796,28 +911,47 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       if (!ok) break;
       tc_fence_after();
       // this chunk's K is no longer read: the chunk after next may land there
-      if (tid == 0 && j + 2 < nch) load_k(j + 2);
+      if (tid == 0 && has(j + 2)) load_k(j + 2);
       // ---- the outputs (tokens 32 grp ..) into registers, and this warpgroup's 64
-      // columns of the new state as the next chunk's operand (after the last
-      // chunk, the result)
+      // columns of the new state as the next chunk's operand
       tmem_ld_32cols(tmem + lane_off + kColO + 32 * grp, ov);
+      {
+        const int4 x = chunk(j);
+        pending = x.x + kC < x.y;
+      }
+      if (pending) {
 #pragma unroll
-      for (int hf = 0; hf < 2; ++hf) {
-        float s0[32];
-        tmem_ld_32cols(scol + 32 * hf, s0);
-        tmem_wait_ld();
-        if (last) {
-          const size_t row0 = head + 64 * grp + 32 * hf;
-#pragma unroll
-          for (int i = 0; i < 32; ++i) s_out[(row0 + i) * kD + c] = s0[i];
-        } else {
+        for (int hf = 0; hf < 2; ++hf) {
+          float s0[32];
+          tmem_ld_32cols(scol + 32 * hf, s0);
+          tmem_wait_ld();
           // packed columns 32 grp + 16 hf ..
           put32_tmem(tmem + lane_off + kColS0h + 32 * grp + 16 * hf,
                      tmem + lane_off + kColS0l + 32 * grp + 16 * hf, s0);
         }
+      } else {
+        // an item's last chunk: outputs and state leave, and the next item's initial
+        // state takes the state's place
+        tmem_wait_ld();
+        write_out(j);
+        const int4 x = chunk(j), nx = chunk(j + 1);
+#pragma unroll 1
+        for (int hf = 0; hf < 2; ++hf) {
+          float s0[32];
+          tmem_ld_32cols(scol + 32 * hf, s0);
+          tmem_wait_ld();
+          float* const so = s_out + (size_t(x.w) * kD + 64 * grp + 32 * hf) * kD + c;
+#pragma unroll
+          for (int i = 0; i < 32; ++i) so[i * kD] = s0[i];
+          if (nx.x < nx.y) {
+            read_init(nx, 64 * grp + 32 * hf, s0);
+            tmem_st_32cols(scol + 32 * hf, s0);
+            put32_tmem(tmem + lane_off + kColS0h + 32 * grp + 16 * hf,
+                       tmem + lane_off + kColS0l + 32 * grp + 16 * hf, s0);
+          }
+        }
       }
     }
-    if (ok && nch > 0) write_out(nch - 1);
   }
   if (!ok) {
     // a wait ran out: let the copies and tensor-core work already issued
@@ -833,10 +967,6 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       mma_commit(drain + role);
       mbar_wait(drain + role, 0, kDrainNs, nullptr);
     }
-  } else if (p1 == p0 && r < R && s_out != nullptr && role == 1) {
-    // no prefix tokens: the state is the initial one (zeros without one)
-    for (int i = 64 * grp; i < 64 * grp + 64; ++i)
-      s_out[(head + i) * kD + c] = s_init ? s_init[(head + i) * kD + c] : 0.f;
   }
   tc_fence_before();
   __syncthreads();
@@ -873,6 +1003,14 @@ bool encode_tokens(CUtensorMap* map, const void* base, int tokens, int Hl) {
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
+    return 1;
+  return n;
+}
+
 }  // namespace
 
 bool scan_tc_supported(const jet_dims& d) {
@@ -889,12 +1027,17 @@ cudaError_t launch_scan_tc(const jet_layout& lay, const jet_dims& d, int rule,
       !encode_tokens(&tmK, k, n.total_prefix, d.Hl) ||
       !encode_tokens(&tmV, v, n.total_prefix, d.Hl))
     return cudaErrorInvalidValue;
-  auto kern = rule == JET_RECUR_GLA ? scan_tc_kernel<false> : scan_tc_kernel<true>;
+  const long long items = (long long)n.R * d.Hl;
+  const int sms = sm_count();  // one CTA per SM
+  const bool gla = rule == JET_RECUR_GLA, many = items > sms;
+  auto kern = gla ? (many ? scan_tc_kernel<false, true> : scan_tc_kernel<false, false>)
+                  : (many ? scan_tc_kernel<true, true> : scan_tc_kernel<true, false>);
   cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemBytes));
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(unsigned(d.Hl), unsigned(n.R)), dim3(kThreads), kSmemBytes, st,
-                    tmQ, tmK, tmV, lay.prefix_offset, n.R, n.total_prefix, d.Hl, s_init, alpha,
+  const unsigned grid = unsigned(many ? sms : items);
+  return launch_pdl(kern, dim3(grid), dim3(kThreads), kSmemBytes, st, tmQ, tmK, tmV,
+                    lay.prefix_offset, lay.req_order, n.R, n.total_prefix, d.Hl, s_init, alpha,
                     beta, static_cast<__nv_bfloat16*>(o), s_out, status, wait_budget_ns(),
                     test_stall());
 }
