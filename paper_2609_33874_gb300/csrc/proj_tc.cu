@@ -64,6 +64,8 @@ struct ProjArgs {
   int* status;
   int N, O, K, ldo;     // rows, weight rows, reduction length, output row stride
   int Nt, n_tt, units, nkb, stages, splits;
+  int tail_units, tail_group, tail_Nt, tail_n_tt;  // from this unit on: slices from
+                                                   // tail_group on, in narrower tiles
   uint32_t tmem_cols, acc_cols;  // two accumulators of acc_cols columns
   uint64_t wait_ns;  // budget of one bounded wait (jet_set_wait_budget_ns)
   int hold_first;    // test hook (jet_set_test_stall): withhold the first stage's loads
@@ -71,15 +73,27 @@ struct ProjArgs {
 };
 
 // unit u -> (256-row weight slice, K split, token tile); the token tiles of one
-// weight slice are consecutive, so they share it through L2
+// weight slice are consecutive, so they share it through L2. Units of the tail are
+// not split
 struct Unit {
-  int ot, sp, t0, kb0, kb1;
+  int ot, sp, t0, nt, kb0, kb1;
 };
 __device__ __forceinline__ Unit unit_of(const ProjArgs& a, int u) {
   Unit x;
+  if (u >= a.tail_units) {
+    u -= a.tail_units;
+    x.sp = 0;
+    x.ot = a.tail_group + u / a.tail_n_tt;
+    x.nt = a.tail_Nt;
+    x.t0 = u % a.tail_n_tt * x.nt;
+    x.kb0 = 0;
+    x.kb1 = a.nkb;
+    return x;
+  }
   const int tt = u % a.n_tt, rest = u / a.n_tt;
   x.sp = rest % a.splits;
   x.ot = rest / a.splits;
+  x.nt = a.Nt;
   x.t0 = tt * a.Nt;
   x.kb0 = int((long long)x.sp * a.nkb / a.splits);
   x.kb1 = int((long long)(x.sp + 1) * a.nkb / a.splits);
@@ -89,7 +103,7 @@ __device__ __forceinline__ Unit unit_of(const ProjArgs& a, int u) {
 template <int EPI>
 __global__ void __launch_bounds__(kThreads, 1)
 proj_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
-               const ProjArgs a) {
+               const __grid_constant__ CUtensorMap tmXt, const ProjArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
@@ -126,6 +140,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&tmW);
     tma_prefetch_desc(&tmX);
+    if (a.tail_units < a.units) tma_prefetch_desc(&tmXt);
   }
   pdl_begin();
   if (warp == 1) {
@@ -148,7 +163,9 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       for (int u = cid; ok && u < a.units; u += ncl) {
         const Unit x = unit_of(a, u);
         const int o0 = (2 * x.ot + int(rank)) * kBM;
-        const int t0 = x.t0 + int(rank) * (a.Nt / 2);
+        const int t0 = x.t0 + int(rank) * (x.nt / 2);
+        const CUtensorMap* map_x = u < a.tail_units ? &tmX : &tmXt;
+        const uint32_t bytes = a_bytes + uint32_t(x.nt / 2) * 128;
         for (int kb = x.kb0; kb < x.kb1; ++kb) {
           if (!mbar_wait(empty + s, ph ^ 1u, a.wait_ns, abort_flag)) {
             ok = false;
@@ -161,9 +178,9 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
             // both CTAs' bytes complete on the even CTA's barrier, which
             // expects them all; the odd CTA's may land before that arrive
             const uint32_t bar = mapa_shared(full + s, 0);
-            if (rank == 0) mbar_arrive_expect_tx(full + s, 2 * stage_bytes);
+            if (rank == 0) mbar_arrive_expect_tx(full + s, 2 * bytes);
             tma_load_2d_pair(sa, &tmW, bar, kb * kBK, o0, pol_w);
-            tma_load_2d_pair(sa + a_bytes, &tmX, bar, kb * kBK, t0, pol_x);
+            tma_load_2d_pair(sa + a_bytes, map_x, bar, kb * kBK, t0, pol_x);
             issued |= 1u << s;
             issued_par = (issued_par & ~(1u << s)) | (ph << s);
           }
@@ -191,7 +208,6 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
     if (elect_one() && rank == 0) {
-      const uint32_t idesc = idesc_bf16_f32(2 * kBM, a.Nt);
       int s = 0, local = 0;
       uint32_t ph = 0;
       bool ok = true;
@@ -205,6 +221,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + uint32_t(buf) * a.acc_cols;
         const Unit x = unit_of(a, u);
+        const uint32_t idesc = idesc_bf16_f32(2 * kBM, x.nt);
         for (int kb = x.kb0; kb < x.kb1; ++kb) {
           if (!mbar_wait(full + s, ph, a.wait_ns, abort_flag)) {
             ok = false;
@@ -252,7 +269,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       named_bar_sync(1, 128);
       if (*epi_abort) break;
       tc_fence_after();
-      const int ncols = min(a.Nt, a.N - t0);
+      const int ncols = min(x.nt, a.N - t0);
       const int ot = 2 * x.ot + int(rank);  // this CTA's 128-row weight tile
       const uint32_t tl = tmem_base + uint32_t(buf) * a.acc_cols + (uint32_t(32 * q) << 16);
       for (int c0 = 0; c0 < ncols; c0 += 32) {
@@ -588,6 +605,7 @@ cudaError_t launch_reduce(const ProjArgs& a, float* part, int N, int O, void* ou
 
 struct Tiling {
   int n_tt, Nt, otiles, groups, nkb, splits;  // groups: 256-row weight slices
+  int tail_group, tail_n_tt, tail_Nt;  // slices from tail_group on in narrower tiles
 };
 
 // Token tiles of at most 256 rows (a multiple of 16: each CTA of a pair holds
@@ -602,26 +620,49 @@ struct Tiling {
 // D 4,096 and Dff 12,288 took 525 us of 178 rows, now 513; 643 of 355, now 634; 715
 // of 444, now 691; 851 of 555, now 808; 1,802 of 2,800, now 1,688. Splits over more
 // than one round gain up to 1 % there, but 355 rows take 1 - 2 % more.
+// Where the weight slices past the full rounds would leave most pairs idle, they are
+// a tail in narrower token tiles that all pairs share (the gate and up projection of
+// 24,576 features: 76 slices, then 20 in three tiles each): the stack takes 496 us of
+// 178 rows without it, 481 with; 618 of 355, now 601; 685 of 444, now 674.
 constexpr int kPlanSMs = 152;
 Tiling tiling(int N, int O, int K, bool split) {
   const int pairs = kPlanSMs / 2, least = (N + kMaxNt - 1) / kMaxNt;
+  auto tiles = [&](int c, int& nt, int& n_tt) {  // c tiles, or fewer once rounded
+    nt = ((N + c - 1) / c + 15) / 16 * 16;
+    n_tt = (N + nt - 1) / nt;
+  };
+  auto rounds = [&](long long units) { return (units + pairs - 1) / pairs; };
   Tiling best{};
   long long best_cost = -1;
   for (int c = least; c <= 2 * least + 2; ++c) {
     Tiling t{};
-    t.Nt = ((N + c - 1) / c + 15) / 16 * 16;
-    t.n_tt = (N + t.Nt - 1) / t.Nt;
+    tiles(c, t.Nt, t.n_tt);
     t.otiles = (O + kBM - 1) / kBM;
     t.groups = (t.otiles + 1) / 2;
     t.nkb = (K + kBK - 1) / kBK;
+    t.tail_group = t.groups;
     const int units = t.groups * t.n_tt;
     t.splits = 1;
     while (split && units * (t.splits + 1) <= pairs && t.nkb / (t.splits + 1) >= 8) ++t.splits;
-    const long long rounds = (units * t.splits + pairs - 1) / pairs;
-    const long long cost = rounds * ((t.nkb + t.splits - 1) / t.splits) * (t.Nt + 80);
+    const long long per_kb = (t.nkb + t.splits - 1) / t.splits;
+    long long cost = rounds((long long)units * t.splits) * per_kb * (t.Nt + 80);
     if (best_cost < 0 || cost < best_cost) {
       best = t;
       best_cost = cost;
+    }
+    // the same, with the slices past its full rounds in narrower tiles
+    const int full = units / pairs, head = full * pairs / t.n_tt;
+    if (t.splits > 1 || full == 0 || head == t.groups) continue;
+    for (int ct = c + 1; ct <= 4 * c; ++ct) {
+      Tiling u = t;
+      tiles(ct, u.tail_Nt, u.tail_n_tt);
+      u.tail_group = head;
+      cost = (full * (t.Nt + 80) +
+              rounds((long long)(t.groups - head) * u.tail_n_tt) * (u.tail_Nt + 80)) * t.nkb;
+      if (cost * 100 < best_cost * 97) {
+        best = u;
+        best_cost = cost;
+      }
     }
   }
   return best;
@@ -649,7 +690,11 @@ cudaError_t launch_epi(const void* x, int N, int K, int ldx, const void* w, int 
           reinterpret_cast<uintptr_t>(res) % 16 == 0;
   a.Nt = Nt;
   a.n_tt = n_tt;
-  a.units = tl.groups * n_tt * a.splits;
+  a.tail_units = tl.tail_group * n_tt * a.splits;
+  a.tail_group = tl.tail_group;
+  a.tail_Nt = tl.tail_Nt;
+  a.tail_n_tt = tl.tail_n_tt;
+  a.units = a.tail_units + (tl.groups - tl.tail_group) * tl.tail_n_tt;
   a.nkb = (K + kBK - 1) / kBK;
   a.acc_cols = Nt <= 128 ? 128 : 256;
   a.tmem_cols = 2 * a.acc_cols;
@@ -657,14 +702,16 @@ cudaError_t launch_epi(const void* x, int N, int K, int ldx, const void* w, int 
   const int stage_bytes = kBM * 128 + b_rows * 128;
   a.stages = std::min(8, (kSmemLimit - 1024 - kFixedSmem) / stage_bytes);
   const size_t smem = 1024 + size_t(a.stages) * stage_bytes + kFixedSmem;
-  CUtensorMap tmW, tmX;
+  CUtensorMap tmW, tmX, tmXt;
   if (!encode_rows(&tmW, w, O, K, K, kBM) || !encode_rows(&tmX, x, N, K, ldx, b_rows))
     return cudaErrorInvalidValue;
+  tmXt = tmX;
+  if (tl.tail_Nt && !encode_rows(&tmXt, x, N, K, ldx, tl.tail_Nt / 2)) return cudaErrorInvalidValue;
   auto kern = a.splits > 1 ? proj_tc_kernel<kPartial> : proj_tc_kernel<EPI>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
   const int clusters = std::max(1, std::min(a.units, max_pairs(kern, smem)));
-  e = launch_pdl_pairs(kern, dim3(unsigned(2 * clusters)), dim3(kThreads), smem, st, tmW, tmX, a);
+  e = launch_pdl_pairs(kern, dim3(unsigned(2 * clusters)), dim3(kThreads), smem, st, tmW, tmX, tmXt, a);
   if (e != cudaSuccess) return e;
   if (splits_out) {
     // the caller reduces the partials itself

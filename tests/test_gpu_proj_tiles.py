@@ -1,6 +1,7 @@
 """The stack's projections at the edges of their tilings against the oracle: a width
 that ends inside a 32-feature piece, rows that take more token tiles than the fewest,
-an unsplit residual over several rounds of tiles, and split K with its reduces."""
+an unsplit residual over several rounds of tiles, split K with its reduces, and a last
+round in narrower tiles."""
 import dataclasses
 
 import numpy as np
@@ -18,6 +19,7 @@ CASES = [
     (13, 5, 5, 272, 64, 2, 160),
     (60, 4, 4, 512, 1088, 4, 64),
     (3, 3, 4, 1536, 2048, 8, 128),
+    (8, 2, 3, 128, 9984, 2, 32),
 ]
 
 
