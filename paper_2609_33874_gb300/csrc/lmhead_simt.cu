@@ -15,10 +15,12 @@
 // (four elements each) instead of the tile, so that a row's float4 is one
 // broadcast and a weight float4 is used MR times. The warps' partial sums are
 // added at the end (eight chains of D / 8 terms: shorter than one of D).
-// 7 rows x 512 x 8192 (16.8 MB of weights): 11.2 us; a 32-row tile filled by
-// 4-byte loads, one K slice at a time, took 73.6 us.
+// With few tiles two CTAs split a tile's K slices. 7 rows x 512 x 8192 (16.8 MB of
+// weights): 9.9 us, 11.2 with one CTA a tile; a 32-row tile filled by 4-byte loads,
+// one K slice at a time, took 73.6 us.
 #include "jet_device.cuh"
 #include "jet_internal.h"
+#include "sm100_ptx.cuh"
 
 namespace jet {
 namespace {
@@ -52,7 +54,9 @@ __device__ __forceinline__ void copy16(float* dst, const float* src, bool ok) {
 // warp reads at one chunk fall in different banks
 __device__ __forceinline__ int chunk_at(int r, int c) { return r * kBK + ((c ^ (r & 7)) << 2); }
 
-template <int MR>
+// PAIR: the two CTAs of a cluster take half of the K slices each, and the even one
+// adds the odd one's sums to its own.
+template <int MR, bool PAIR>
 __global__ void __launch_bounds__(kThreads)
 lmhead_simt_kernel(const int32_t* __restrict__ target_ids, const int32_t* __restrict__ row_tgt_offset,
                    const int32_t* __restrict__ row_tgt_index, int N, int T_, int V, int D,
@@ -60,26 +64,30 @@ lmhead_simt_kernel(const int32_t* __restrict__ target_ids, const int32_t* __rest
                    float2* __restrict__ part, float* __restrict__ z_tgt, int* status) {
   pdl_begin();
   extern __shared__ __align__(16) float ring[];
-  const int row0 = blockIdx.x * MR;
+  const int row0 = int(PAIR ? blockIdx.x >> 1 : blockIdx.x) * MR;
+  const bool odd = PAIR && (blockIdx.x & 1);
   const int vt = blockIdx.y;
   const int v0 = vt * kBV;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int nkb = (D + kBK - 1) / kBK;
+  // this CTA's K slices [k0, k0 + nkb)
+  const int all = (D + kBK - 1) / kBK;
+  const int k0 = odd ? all / 2 : 0;
+  const int nkb = !PAIR ? all : odd ? all - all / 2 : all / 2;
 
-  // K slice kb into its stage: the rows past N and V and the elements past D
+  // K slice k0 + kb into its stage: the rows past N and V and the elements past D
   // (a multiple of 8) are zeros
   auto load = [&](int kb) {
     float* st = ring + (kb % kStages) * stage_floats<MR>();
 #pragma unroll
     for (int i = 0; i < kBV * 8 / kThreads; ++i) {
       const int e = tid + i * kThreads, r = e >> 3, c = e & 7;
-      const int kx = kb * kBK + 4 * c;
+      const int kx = (k0 + kb) * kBK + 4 * c;
       const bool ok = v0 + r < V && kx < D;
       copy16(st + chunk_at(r, c), w_lm + (ok ? size_t(v0 + r) * D + kx : 0), ok);
     }
     if (tid < MR * 8) {
       const int r = tid >> 3, c = tid & 7;
-      const int kx = kb * kBK + 4 * c;
+      const int kx = (k0 + kb) * kBK + 4 * c;
       const bool ok = row0 + r < N && kx < D;
       copy16(st + kBV * kBK + r * kBK + 4 * c, hidden + (ok ? size_t(row0 + r) * D + kx : 0), ok);
     }
@@ -144,13 +152,24 @@ lmhead_simt_kernel(const int32_t* __restrict__ target_ids, const int32_t* __rest
 #pragma unroll
     for (int b = 0; b < 4; ++b) red[(warp * MR + a) * kBV + lane + 32 * b] = acc[b][a];
   __syncthreads();
+  if (PAIR) {
+    if (odd) {
+      for (int e = tid; e < MR * kBV; e += kThreads) {
+        float z = red[e];
+#pragma unroll
+        for (int w = 1; w < kWarps; ++w) z += red[w * MR * kBV + e];
+        red[e] = z;  // read and written by this thread alone
+      }
+    }
+    sm100::cluster_sync();
+  }
 
   // epilogue: warp w takes rows w, w + 8 ..: base-2 (max, sum) over the tile's
   // vocabulary, target gather
 #pragma unroll
   for (int i = 0; i < RW; ++i) {
     const int a = warp + kWarps * i, n = row0 + a;
-    if (n >= N) break;
+    if (n >= N || odd) break;
     constexpr float kLog2e = 1.4426950408889634f;
     float z[4], mx = -INFINITY;
 #pragma unroll
@@ -158,6 +177,7 @@ lmhead_simt_kernel(const int32_t* __restrict__ target_ids, const int32_t* __rest
       z[b] = 0.f;
 #pragma unroll
       for (int w = 0; w < kWarps; ++w) z[b] += red[(w * MR + a) * kBV + lane + 32 * b];
+      if (PAIR) z[b] += sm100::ld_shared_remote(red + a * kBV + lane + 32 * b, 1);
       if (v0 + lane + 32 * b < V) mx = fmaxf(mx, z[b] * kLog2e);
     }
     mx = warp_max(mx);
@@ -186,6 +206,7 @@ lmhead_simt_kernel(const int32_t* __restrict__ target_ids, const int32_t* __rest
       }
     }
   }
+  if (PAIR) sm100::cluster_sync();  // the odd CTA's sums stay until they are read
 }
 
 template <int MR>
@@ -197,14 +218,24 @@ cudaError_t launch_mr(const jet_layout& lay, const jet_dims& d, const ScorePlan&
   float2* part = reinterpret_cast<float2*>(base + plan.part_off);
   float* z_tgt = reinterpret_cast<float*>(base + plan.ztgt_off);
   const size_t smem = smem_bytes<MR>();
-  const cudaError_t e = cudaFuncSetAttribute(
-      lmhead_simt_kernel<MR>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  // pairs while both CTAs of every tile find an SM (152 of them) of their own: a
+  // one-request step of 7 rows and 8,192 entries takes 36.8 us of D 1,024 without
+  // them, 28.7 with, 67.6 and 45.8 of D 2,560, 23.4 both ways of D 512 and below
+  // (its launches); past that the halves would queue
+  const long long row_tiles = (n.N + MR - 1) / MR;
+  const bool pair = 2 * row_tiles * plan.vtiles <= 152;
+  const auto kern = pair ? lmhead_simt_kernel<MR, true> : lmhead_simt_kernel<MR, false>;
+  const cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
-  dim3 grid(unsigned((n.N + MR - 1) / MR), unsigned(plan.vtiles));
-  return launch_pdl(lmhead_simt_kernel<MR>, grid, dim3(kThreads), smem, st, lay.target_ids,
-                    lay.row_tgt_offset, lay.row_tgt_index, n.N, n.T, n.V, d.D,
-                    static_cast<const float*>(hidden), static_cast<const float*>(w_lm), part,
-                    z_tgt, status);
+  const dim3 grid(unsigned(pair ? 2 * row_tiles : row_tiles), unsigned(plan.vtiles));
+  auto launch = [&](auto how) {
+    return how(kern, grid, dim3(kThreads), smem, st, lay.target_ids, lay.row_tgt_offset,
+               lay.row_tgt_index, n.N, n.T, n.V, d.D, static_cast<const float*>(hidden),
+               static_cast<const float*>(w_lm), part, z_tgt, status);
+  };
+  return pair ? launch([](auto... x) { return launch_pdl_pairs(x...); })
+              : launch([](auto... x) { return launch_pdl(x...); });
 }
 
 }  // namespace

@@ -398,6 +398,13 @@ __device__ __forceinline__ uint32_t mapa_shared(const void* p, uint32_t rank) {
   return r;
 }
 
+// a float of CTA `rank`'s shared memory, at the same place as p in this CTA's
+__device__ __forceinline__ float ld_shared_remote(const float* p, uint32_t rank) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(mapa_shared(p, rank)) : "memory");
+  return v;
+}
+
 // arrive on an mbarrier of another CTA of the cluster (its mapa address)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)

@@ -1,7 +1,7 @@
 """The float32 LM head's tiles on the GPU against the oracle: rows around the
 8- and 16-row tiles, vocabularies around the 128-entry tile, hidden sizes
 around the 32-element K slice and its ring of stages, a row with more targets
-than a warp has lanes."""
+than a warp has lanes, tiles on one CTA and on two."""
 import dataclasses
 
 import numpy as np
@@ -21,6 +21,8 @@ CASES = [
     ([9], 129, 200),              # 9 rows: the large tile, mostly empty
     ([8, 9], 300, 192),           # 16 rows, as many K slices as stages
     ([12, 7], 1000, 520),         # 18 rows: two row tiles
+    ([8, 1], 9900, 72),           # too many tiles for two CTAs a tile, 8 rows
+    ([12, 7], 5000, 40),          # the same with two row tiles
 ]
 
 
