@@ -48,6 +48,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "jet_device.cuh"
@@ -658,8 +659,8 @@ namespace {
 // clusters of two CTAs of `kern` that can be resident at once; asked once per kernel
 template <typename K>
 int max_pairs(K kern, size_t smem) {
-  static int cached = 0;
-  if (cached > 0) return cached;
+  static std::atomic<int> cached{0};  // any thread may ask first
+  if (const int c = cached.load(std::memory_order_relaxed)) return c;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(2);
   cfg.blockDim = dim3(kThreads);
@@ -676,7 +677,7 @@ int max_pairs(K kern, size_t smem) {
     cudaGetLastError();
     return std::max(1, sm_count() / 2);
   }
-  cached = n;
+  cached.store(n, std::memory_order_relaxed);
   return n;
 }
 

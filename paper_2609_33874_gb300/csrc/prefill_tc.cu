@@ -34,6 +34,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "jet_device.cuh"
@@ -714,8 +715,8 @@ bool encode_3d(CUtensorMap* map, const void* base, int rows, int heads, int DH, 
 // schedule deals the items to that many pairs); asked once per kernel
 template <typename K>
 int max_pairs(K kern, size_t smem) {
-  static int cached = 0;
-  if (cached > 0) return cached;
+  static std::atomic<int> cached{0};  // any thread may ask first
+  if (const int c = cached.load(std::memory_order_relaxed)) return c;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(2);
   cfg.blockDim = dim3(kThreads);
@@ -732,7 +733,7 @@ int max_pairs(K kern, size_t smem) {
     cudaGetLastError();
     return 1;
   }
-  cached = n;
+  cached.store(n, std::memory_order_relaxed);
   return n;
 }
 

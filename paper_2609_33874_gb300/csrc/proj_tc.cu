@@ -33,6 +33,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "jet_device.cuh"
@@ -572,8 +573,8 @@ int sm_count() {
 // the SM pairs the GPCs offer); asked once per kernel
 template <typename K>
 int max_pairs(K kern, size_t smem) {
-  static int cached = 0;
-  if (cached > 0) return cached;
+  static std::atomic<int> cached{0};  // any thread may ask first
+  if (const int c = cached.load(std::memory_order_relaxed)) return c;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(2);
   cfg.blockDim = dim3(kThreads);
@@ -588,7 +589,7 @@ int max_pairs(K kern, size_t smem) {
   int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1)
     n = std::max(1, sm_count() / 2);
-  cached = n;
+  cached.store(n, std::memory_order_relaxed);
   return n;
 }
 
