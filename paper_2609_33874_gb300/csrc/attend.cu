@@ -315,8 +315,8 @@ AttnPlan attn_plan(const jet_sizes& n, const jet_dims& d) {
     int least = kMinChunkTc;
     // a few long prefixes leave most SMs idle at that length: then about
     // kFewItems chunks in all, of at least kLeastChunk keys (one 6,000-key request
-    // with two kv heads: 320 keys 20 us, 640 keys 23 us, 128 keys 23 us; 32
-    // groups of 512 keys: unsplit 17.3 us, halves 18.1 us with the combine)
+    // with two kv heads: 320 keys 17.5 us, 640 keys 19.8 us, 128 keys 21.3 us;
+    // 32 groups of 512 keys: unsplit 15.0 us, halves 16.9 us with the combine)
     if (groups <= kFewGroups) {
       const long long even = (long long)(double(groups) * avg_tiles / kFewItems + 0.999) * 64;
       least = int(std::max<long long>(kLeastChunk, std::min<long long>(kMinChunkTc, even)));

@@ -70,8 +70,8 @@ __device__ __forceinline__ void ms_combine2(float& m, float& s, float m2, float 
 // A warp combines the base-2 partials (m, l, O) of row n, head h over its prefix
 // chunks: l and acc (elements lane + 32 i of the head) relative to m, the largest
 // of their maxima. The (m, l) of 32 chunks are read one a lane and the chunks'
-// outputs four at a time, the first four beside the (m, l): up to four chunks
-// cost one memory latency (64 requests of 100 - 2,000 keys: the whole call 47.9 ->
+// outputs four at a time, with `ahead` the first four beside the (m, l): up to four
+// chunks then cost one memory latency (64 requests of 100 - 2,000 keys: the whole call 47.9 ->
 // 46.0 us; eight at a time 48.1 us; one 6,000-key request in 19 chunks 18.9 ->
 // 18.5 us).
 template <int DH>
