@@ -334,9 +334,19 @@ AttnPlan attn_plan(const jet_sizes& n, const jet_dims& d) {
   p.splits = (n.max_prefix + chunk - 1) / chunk;
   const size_t vecs = size_t(p.splits) * n.N * d.Hq;
   p.bytes = vecs * d.d * sizeof(float) + vecs * sizeof(float2);
-  // tensor-core path: a work list of (request, kv head, query block, chunk)
-  // items plus two counters, 16-byte aligned, after the partials
-  if (tc) p.bytes += 32 + 16 * size_t(n.R) * d.Hkv * p.qgroups * p.splits;
+  // Items dealt out back and forth in the order of the requests' lengths balance well
+  // when that is the order of the items' own lengths: unsplit requests, or lengths
+  // within a quarter of their mean's. Long chunks (16 key tiles or more) of uneven
+  // requests do not come in that order, and with at most 2.5 groups an SM a CTA has
+  // too few of them to even out; then a longest-first list and a shared counter pay
+  // for their launch (requests of 2,048 - 8,192 keys, two kv heads: 128 with the list
+  // 240 us, dealt 245; 90 181 and 188; 256 unsplit 438 and 426; 64 of 4,096 111 and
+  // 106; 400 groups of 300 - 4,000 keys 175 and 171).
+  p.sorted = tc && p.splits > 1 && chunk >= 16 * 64 && 2 * groups <= 5 * kPlanSMs &&
+             4LL * n.max_prefix * n.R > 5LL * n.total_prefix;
+  // the work list: (request, kv head, query block, chunk) items plus two counters,
+  // 16-byte aligned, after the partials
+  if (p.sorted) p.bytes += 32 + 16 * size_t(n.R) * d.Hkv * p.qgroups * p.splits;
   return p;
 }
 

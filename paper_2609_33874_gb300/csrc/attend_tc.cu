@@ -341,14 +341,21 @@ __device__ __forceinline__ LaneReq lane_req(const AttArgs& a, int base, int lane
 // length (req_order); within a request kv head, query block and chunk, the
 // chunk fastest - counting only items that have keys and vectors. One warp
 // scans the requests' item counts 32 at a time; false past the last item.
-// The geometry comes with it; `q` holds the requests when `held` (up to 32: read
-// once per CTA).
-__device__ __forceinline__ bool nth_item(const AttArgs& a, int k, int lane, LaneReq& q, bool& held,
+// The geometry comes with it. A CTA asks for growing k, so the scan goes on from
+// the window of the last item, `w` (from the first one at every item, 512 requests
+// of 1,024 keys took 235 us instead of 197, 300 of 512 90 instead of 75).
+struct ItemWindow {
+  LaneReq q;   // its requests, when held
+  bool held;
+  int base, before;  // its first request in the order; the items before it
+};
+__device__ __forceinline__ bool nth_item(const AttArgs& a, int k, int lane, ItemWindow& w,
                                          int4* out, ItemGeo* geo) {
-  int before = 0;
-  for (int base = 0; base < a.R; base += 32) {
-    if (!held) q = lane_req(a, base, lane);
-    held = a.R <= 32;
+  LaneReq& q = w.q;
+  for (; w.base < a.R; w.base += 32) {
+    if (!w.held) q = lane_req(a, w.base, lane);
+    w.held = true;
+    const int before = w.before;
     int cnt = 0, nq = 0, sp = 0;
     if (q.r >= 0) {
       int per = 0;
@@ -377,7 +384,8 @@ __device__ __forceinline__ bool nth_item(const AttArgs& a, int k, int lane, Lane
                          __shfl_sync(0xffffffffu, q.P, src));
       return true;
     }
-    before += total;
+    w.before += total;
+    w.held = false;
   }
   return false;
 }
@@ -479,8 +487,7 @@ attend_prefix_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
   if (warp == kSchedWarp) {
     // ---------------------------------------------------------------- scheduler
     const int count = a.sorted ? *a.item_count : 0;
-    LaneReq reqs{};
-    bool held = false;
+    ItemWindow window{};
     for (int u = 0;; ++u) {
       const int slot = u & 1;
       bool okw = true;
@@ -521,7 +528,7 @@ attend_prefix_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
         const int k = u * n + ((u & 1) ? n - 1 - int(blockIdx.x) : int(blockIdx.x));
         int4 cand;
         ItemGeo ce;
-        if (k < a.n_all && nth_item(a, k, lane, reqs, held, &cand, &ce)) {
+        if (k < a.n_all && nth_item(a, k, lane, window, &cand, &ce)) {
           if (ce.ok) {
             it = cand;
             e = ce;
@@ -1110,10 +1117,7 @@ cudaError_t launch_dh(const jet_layout& lay, const jet_dims& d, const AttnPlan& 
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
     return cudaErrorInvalidValue;
   const int grid = int(std::max<long long>(1, std::min<long long>(sms, a.n_all)));
-  // longest-first dynamic order pays for its extra launch only when items are
-  // long and uneven (chunks of 16 key tiles or more); shorter items are dealt out
-  // back and forth, which needs no counter (and no launch to reset one)
-  a.sorted = plan.chunk >= 16 * kBN;
+  a.sorted = plan.sorted;
   cudaError_t e = cudaSuccess;
   if (a.sorted)
     e = launch_pdl(attend_items_kernel, dim3(1), dim3(1024), 0, st, a, plan.qgroups, plan.splits);

@@ -27,6 +27,7 @@ struct AttnPlan {
   int splits;    // prefix chunks per (request, key/value head)
   int chunk;     // prefix keys per chunk (multiple of 32)
   int qgroups;   // query-vector groups per (request, key/value head)
+  bool sorted;   // tensor-core path: items from a longest-first work list
   size_t bytes;  // workspace bytes
 };
 AttnPlan attn_plan(const jet_sizes& n, const jet_dims& d);

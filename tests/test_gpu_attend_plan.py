@@ -2,7 +2,8 @@
 prefixes cut into many chunks, a prefix just past the shortest chunk, more items
 than CTAs of uneven length (several a CTA, dealt back and forth), and more than 32
 requests of one to many chunks (the combine meets rows that are already written
-and chunks that a request does not have)."""
+and chunks that a request does not have), long uneven chunks from the longest-first
+list, and a deal that passes over windows of 32 requests."""
 import dataclasses
 
 import numpy as np
@@ -19,6 +20,8 @@ CASES = [
     ([2049, 100, 700], dict(Hq=32, Hkv=8, d=128)),
     ([1 + 37 * i % 900 for i in range(90)], dict(Hq=24, Hkv=4, d=64)),
     ([4000] + [50 + 61 * i for i in range(32)], dict(Hq=32, Hkv=8, d=128)),
+    ([600 + 230 * i for i in range(20)], dict(Hq=8, Hkv=8, d=64)),
+    ([60 + 7 * (i % 3) for i in range(300)], dict(Hq=4, Hkv=4, d=64)),
 ]
 
 
