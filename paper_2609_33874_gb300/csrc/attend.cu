@@ -62,7 +62,9 @@ attend_prefix_kernel(const int32_t* __restrict__ prefix_offset, const int32_t* _
   if (r >= R) return;
   const int n0 = row_offset[r], nr = row_offset[r + 1] - n0;
   const int p0 = prefix_offset[r], P = prefix_offset[r + 1] - p0;
-  if (n0 < 0 || nr < 1 || n0 + nr > N || p0 < 0 || P < 0 || p0 + P > total_prefix) {
+  // (a request longer than the plan's chunks or vector groups is left out too)
+  if (n0 < 0 || nr < 1 || n0 + nr > N || p0 < 0 || P < 0 || p0 + P > total_prefix ||
+      P > chunk * int(gridDim.x) || nr * g > kQV * int(gridDim.y)) {
     if (threadIdx.x == 0) flag(status, JET_ERR_DEVICE);
     return;
   }

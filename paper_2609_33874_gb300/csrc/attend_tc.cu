@@ -39,6 +39,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "attend_items.h"
 #include "jet_device.cuh"
 #include "jet_internal.h"
 #include "sm100_ptx.cuh"
@@ -49,7 +50,7 @@ namespace {
 using namespace sm100;
 
 constexpr int kBV = 128;      // query vectors per CTA (MMA M, TMEM lanes)
-constexpr int kBN = 64;       // keys per tile
+constexpr int kBN = kItemTile;  // keys per tile
 constexpr int kStages = 2;
 constexpr int kThreads = 224;
 constexpr int kSchedWarp = 6;  // the work-item scheduler
@@ -72,7 +73,7 @@ struct Geo {
   static constexpr uint32_t kPCol = 2 * kBN + DH;           // P buffer b at kPCol + 32 b
 };
 
-struct AttArgs {
+struct AttArgs : ItemPlan {
   const int32_t* prefix_offset;
   const int32_t* row_offset;
   const int32_t* req_order;
@@ -86,13 +87,10 @@ struct AttArgs {
   int4* items;       // work list (attend_items_kernel)
   int* item_count;
   int* item_next;    // next item to take (dynamic schedule)
-  int R, N, C, total_prefix, Hq, Hkv, chunk;
-  int g, rb;         // query heads per kv head; rows per query block (128 / g)
+  int C, Hq;
   int sorted;        // 1: take items from the longest-first work list; 0: a static deal of
                      // the items in the order of nth_item
-  int splits;        // chunks per request (the plan's)
   long long n_all;   // upper bound of the items: (request, kv head, block, chunk) slots
-  int has_cand;      // the batch has fed candidate tokens (F > 0)
   int prefill;       // 1: causal self-attention over the prefixes (rows = prefix positions)
   float scale_log2;  // log2(e) / sqrt(d)
   uint64_t wait_ns;  // budget of one bounded wait (jet_set_wait_budget_ns)
@@ -133,98 +131,40 @@ __device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int32_t 
                : "memory");
 }
 
-// A request's P prefix keys in chunks of nearly equal length: at most
-// ceil(P / chunk) chunks of a whole number of 64-key tiles each, none empty
-// (the last also takes the candidates' own keys).
-__device__ __forceinline__ int req_splits(int P, int chunk, int* tiles_per_split) {
-  const int tiles = (P + kBN - 1) / kBN;
-  const int s0 = max(1, (P + chunk - 1) / chunk);
-  const int per = (tiles + s0 - 1) / s0;
-  *tiles_per_split = per;
-  return (tiles + per - 1) / per;
-}
-
-// Geometry of one work item (request r, key/value head kh, query block qb,
-// prefix chunk split); every role derives it the same way from the item.
-struct ItemGeo {
-  int r, kh, n0, nr, p0, P, row0, vbase, nv, k_begin, k_end, npt, nct, ntiles, splits_r, f_begin;
-  int split;
-  bool ok;
-};
-
-__device__ __forceinline__ ItemGeo item_geo_at(const AttArgs& a, int4 it, int n0, int nr, int p0,
-                                               int P);
-
-__device__ __forceinline__ ItemGeo item_geo(const AttArgs& a, int4 it) {
-  ItemGeo e{};
-  e.r = it.x;
-  e.kh = it.y;
-  const int qb = it.z;
-  e.split = it.w;
-  e.ok = false;
-  if (e.r < 0 || e.r >= a.R || e.kh < 0 || e.kh >= a.Hkv) return e;
-  if (a.prefill) {
-    // prefill: the rows are the request's prefix positions and a block of
-    // them sees the keys up to its last position (per-row causal mask in the
-    // softmax); one chunk per item, the output written directly
-    e.p0 = a.prefix_offset[e.r];
-    e.P = a.prefix_offset[e.r + 1] - e.p0;
-    if (e.p0 < 0 || e.P < 1 || e.p0 + e.P > a.total_prefix || e.split != 0) return e;
-    e.n0 = e.p0;
-    e.nr = e.P;
-    e.row0 = qb * a.rb;
-    if (e.row0 >= e.nr) return e;
-    e.vbase = e.row0 * a.g;
-    e.nv = min(a.rb, e.nr - e.row0) * a.g;
-    e.splits_r = 1;
-    e.k_begin = 0;
-    e.k_end = min(e.P, e.row0 + a.rb);
-    e.npt = (e.k_end + kBN - 1) / kBN;
-    e.nct = 0;
-    e.f_begin = 0;
-    e.ntiles = e.npt;
-    e.ok = true;
-    return e;
+// Of an item of the work list; *fits: its request is one to work on
+__device__ __forceinline__ ItemGeo item_geo(const AttArgs& a, int4 it, bool* fits) {
+  *fits = false;
+  if (!a.prefill) {
+    if (it.x < 0 || it.x >= a.R) return ItemGeo{};
+    const int n0 = a.row_offset[it.x], nr = a.row_offset[it.x + 1] - n0;
+    const int p0 = a.prefix_offset[it.x], P = a.prefix_offset[it.x + 1] - p0;
+    const RequestCut cut = request_cut(a, n0, nr, p0, P);
+    *fits = cut.nq > 0;
+    return item_geo_at(a, it.x, it.y, it.z, it.w, n0, nr, p0, P, cut);
   }
-  const int n0 = a.row_offset[e.r], p0 = a.prefix_offset[e.r];
-  return item_geo_at(a, it, n0, a.row_offset[e.r + 1] - n0, p0, a.prefix_offset[e.r + 1] - p0);
-}
-
-// The same of a scoring item whose request's rows [n0, n0 + nr) and prefix
-// [p0, p0 + P) are at hand.
-__device__ __forceinline__ ItemGeo item_geo_at(const AttArgs& a, int4 it, int n0, int nr, int p0,
-                                               int P) {
+  // prefill: the rows are the request's prefix positions and a block of
+  // them sees the keys up to its last position (per-row causal mask in the
+  // softmax); one chunk per item, the output written directly
   ItemGeo e{};
   e.r = it.x;
   e.kh = it.y;
   const int qb = it.z;
   e.split = it.w;
-  e.ok = false;
   if (e.r < 0 || e.r >= a.R || e.kh < 0 || e.kh >= a.Hkv) return e;
-  e.n0 = n0;
-  e.nr = nr;
-  e.p0 = p0;
-  e.P = P;
-  if (e.n0 < 0 || e.nr < 1 || e.n0 + e.nr > a.N || e.p0 < 0 || e.P < 1 ||
-      e.p0 + e.P > a.total_prefix)
-    return e;
+  e.p0 = a.prefix_offset[e.r];
+  e.P = a.prefix_offset[e.r + 1] - e.p0;
+  *fits = request_cut(a, e.p0, e.P, e.p0, e.P).nq > 0;
+  if (!*fits || e.split != 0) return e;
+  e.n0 = e.p0;
+  e.nr = e.P;
   e.row0 = qb * a.rb;
   if (e.row0 >= e.nr) return e;
   e.vbase = e.row0 * a.g;
   e.nv = min(a.rb, e.nr - e.row0) * a.g;
-  int per = 0;
-  e.splits_r = req_splits(e.P, a.chunk, &per);
-  if (e.split >= e.splits_r) return e;
-  e.k_begin = e.split * per * kBN;
-  e.k_end = min(e.P, e.k_begin + per * kBN);
-  e.npt = (e.k_end - e.k_begin + kBN - 1) / kBN;
-  // the request's last chunk also takes its candidates' own keys: the F_r fed
-  // tokens, as extra 64-key tiles masked per row to the row's candidate and
-  // position (Sec. 4.1: a candidate attends to its own earlier tokens only)
-  e.f_begin = e.n0 - e.r;  // fed-token index of the request's first fed row
-  const int F_r = e.nr - 1;
-  e.nct = (e.split == e.splits_r - 1 && a.has_cand && F_r > 0) ? (F_r + kBN - 1) / kBN : 0;
-  e.ntiles = e.npt + e.nct;
+  e.splits_r = 1;
+  e.k_end = min(e.P, e.row0 + a.rb);
+  e.npt = (e.k_end + kBN - 1) / kBN;
+  e.ntiles = e.npt;
   e.ok = true;
   return e;
 }
@@ -255,7 +195,9 @@ attend_items_kernel(const AttArgs a, int qgroups, int splits) {
   __syncthreads();
   const long long n_all = (long long)a.R * a.Hkv * qgroups * splits;
   for (long long idx = threadIdx.x; idx < n_all; idx += blockDim.x) {
-    const ItemGeo e = item_geo(a, item_of(a, idx, splits));
+    bool fits;
+    const ItemGeo e = item_geo(a, item_of(a, idx, splits), &fits);
+    if (!fits) flag(a.status, JET_ERR_DEVICE);  // the request is left out
     const int b = e.ok ? min(e.ntiles, kBuckets - 1) : 0;
     if (idx < kItemCache) bucket[idx] = uint8_t(b);
     if (b > 0) atomicAdd(&hist[b], 1);
@@ -289,7 +231,8 @@ attend_items_kernel(const AttArgs a, int qgroups, int splits) {
     if (idx < kItemCache) {
       b = bucket[idx];
     } else {
-      const ItemGeo e = item_geo(a, it);
+      bool fits;
+      const ItemGeo e = item_geo(a, it, &fits);
       b = e.ok ? min(e.ntiles, kBuckets - 1) : 0;
     }
     if (b > 0) a.items[atomicAdd(&cursor[b], 1)] = it;
@@ -297,14 +240,15 @@ attend_items_kernel(const AttArgs a, int qgroups, int splits) {
 }
 
 // The offsets of the requests a lane stands for: its request in the order, its
-// rows [n0, n0 + nr) and its prefix [p0, p0 + P).
+// rows [n0, n0 + nr), its prefix [p0, p0 + P) and how it is cut.
 struct LaneReq {
   int r, n0, nr, p0, P;
+  RequestCut cut;
 };
 
 // The requests [base, base + 32) of the order, one a lane.
 __device__ __forceinline__ LaneReq lane_req(const AttArgs& a, int base, int lane) {
-  LaneReq q{-1, 0, 0, 0, 0};
+  LaneReq q{-1, 0, 0, 0, 0, {}};
   const int ri = base + lane;
   if (a.R <= 32) {
     // all offsets beside the order, then one lane from another: one memory
@@ -323,7 +267,7 @@ __device__ __forceinline__ LaneReq lane_req(const AttArgs& a, int base, int lane
     q.P = __shfl_sync(0xffffffffu, p1 - p0, src);
     q.n0 = __shfl_sync(0xffffffffu, n0, src);
     q.nr = __shfl_sync(0xffffffffu, n1 - n0, src);
-    if (!in) q = LaneReq{-1, 0, 0, 0, 0};
+    if (!in) q = LaneReq{-1, 0, 0, 0, 0, {}};
   } else if (ri < a.R) {
     const int r = a.req_order[ri];
     if (r >= 0 && r < a.R) {
@@ -339,7 +283,8 @@ __device__ __forceinline__ LaneReq lane_req(const AttArgs& a, int base, int lane
 
 // The k-th work item of the unsorted order - requests by decreasing prefix
 // length (req_order); within a request kv head, query block and chunk, the
-// chunk fastest - counting only items that have keys and vectors. One warp
+// chunk fastest - counting only items that have keys and vectors, and only
+// requests that fit the plan (at most n_all items in all, then). One warp
 // scans the requests' item counts 32 at a time; false past the last item.
 // The geometry comes with it. A CTA asks for growing k, so the scan goes on from
 // the window of the last item, `w` (from the first one at every item, 512 requests
@@ -353,16 +298,15 @@ __device__ __forceinline__ bool nth_item(const AttArgs& a, int k, int lane, Item
                                          int4* out, ItemGeo* geo) {
   LaneReq& q = w.q;
   for (; w.base < a.R; w.base += 32) {
-    if (!w.held) q = lane_req(a, w.base, lane);
-    w.held = true;
-    const int before = w.before;
-    int cnt = 0, nq = 0, sp = 0;
-    if (q.r >= 0) {
-      int per = 0;
-      sp = q.P >= 1 ? req_splits(q.P, a.chunk, &per) : 0;
-      nq = q.nr >= 1 ? (q.nr + a.rb - 1) / a.rb : 0;
-      cnt = a.Hkv * nq * sp;
+    if (!w.held) {
+      q = lane_req(a, w.base, lane);
+      if (q.r >= 0) q.cut = request_cut(a, q.n0, q.nr, q.p0, q.P);
+      // a request that the layout or the plan does not hold is left out
+      if (q.cut.nq == 0 && w.base + lane < a.R) flag(a.status, JET_ERR_DEVICE);
+      w.held = true;
     }
+    const int before = w.before;
+    const int cnt = a.Hkv * q.cut.nq * q.cut.sp;
     int inc = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -375,13 +319,15 @@ __device__ __forceinline__ bool nth_item(const AttArgs& a, int k, int lane, Item
       const int src = __ffs(hit) - 1;
       const int kk = k - before - __shfl_sync(0xffffffffu, inc - cnt, src);
       const int r = __shfl_sync(0xffffffffu, q.r, src);
-      nq = __shfl_sync(0xffffffffu, nq, src);
-      sp = __shfl_sync(0xffffffffu, sp, src);
+      const RequestCut cut{__shfl_sync(0xffffffffu, q.cut.nq, src),
+                           __shfl_sync(0xffffffffu, q.cut.sp, src),
+                           __shfl_sync(0xffffffffu, q.cut.per, src)};
+      const int nq = cut.nq, sp = cut.sp;
       const int split = kk % sp, rest = kk / sp;
       *out = make_int4(r, rest / nq, rest % nq, split);
-      *geo = item_geo_at(a, *out, __shfl_sync(0xffffffffu, q.n0, src),
+      *geo = item_geo_at(a, r, rest / nq, rest % nq, split, __shfl_sync(0xffffffffu, q.n0, src),
                          __shfl_sync(0xffffffffu, q.nr, src), __shfl_sync(0xffffffffu, q.p0, src),
-                         __shfl_sync(0xffffffffu, q.P, src));
+                         __shfl_sync(0xffffffffu, q.P, src), cut);
       return true;
     }
     w.before += total;
@@ -399,8 +345,7 @@ struct __align__(16) RingItem {
 static_assert(sizeof(RingItem) % 16 == 0, "ring entries keep 16-byte alignment");
 
 // One persistent CTA per SM. The scheduler warp claims the work items one
-// ahead of the others,
-// computes their geometry once and starts their query block on its way into
+// ahead of the others, computes their geometry once and starts their query block on its way into
 // L2; the other roles take the items from a two-slot ring and release a slot
 // when they are done with its item. All barrier phases run on counters that
 // continue across items, so the next item's query block and first K/V tiles
@@ -509,7 +454,8 @@ attend_prefix_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
             const int idx = first ? int(blockIdx.x) : int(gridDim.x) + atomicAdd(a.item_next, 1);
             if (idx >= count) break;
             const int4 cand = a.items[idx];
-            const ItemGeo ce = item_geo(a, cand);
+            bool fits;
+            const ItemGeo ce = item_geo(a, cand, &fits);
             if (ce.ok) {
               it = cand;
               e = ce;
@@ -1111,6 +1057,7 @@ cudaError_t launch_dh(const jet_layout& lay, const jet_dims& d, const AttnPlan& 
   a.item_count = a.item_next + 1;
   a.items = reinterpret_cast<int4*>(ctrl + 16);
   a.splits = plan.splits;
+  a.qgroups = plan.qgroups;
   a.n_all = (long long)n.R * d.Hkv * plan.qgroups * plan.splits;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -1181,6 +1128,7 @@ cudaError_t launch_prefill_dh(const jet_layout& lay, const jet_dims& d, const vo
   a.item_count = a.item_next + 1;
   a.items = reinterpret_cast<int4*>(ctrl + 16);
   a.splits = 1;
+  a.qgroups = qgroups;
   a.n_all = (long long)n.R * d.Hkv * qgroups;
   a.sorted = 1;
   cudaError_t e =

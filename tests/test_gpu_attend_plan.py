@@ -10,7 +10,8 @@ import numpy as np
 import pytest
 
 import jet_synth
-from gpu_common import TOL_ATTN_BF16, check_attention, oracle_layout, run_problem
+from gpu_common import (TOL_ATTN_BF16, TOL_ATTN_F32, build_step, check_attention, oracle_layout,
+                        run_problem)
 
 pytestmark = pytest.mark.gpu
 
@@ -36,3 +37,47 @@ def test_attention_plan(jet, case):
     got, _ = run_problem(jet, p)
     rows = list(range(p.N)) if p.N <= 60 else sorted(rng.choice(p.N, 60, replace=False).tolist())
     check_attention(oracle_layout(p), p, got["o"], rows, TOL_ATTN_BF16)
+
+
+LONG = [600 + 230 * i for i in range(20)]
+LONGER = [100] + LONG[1:10] + [LONG[10] - 1030] + LONG[11:19] + [LONG[19] + 1530]
+OTHER_WORDS = [
+    # prefixes of the sizes and of the words (as many keys), the request past the plan
+    ("bf16", [128, 100], [150, 78], 0, dict(Hq=8, Hkv=2, d=64)),            # one chunk
+    ("bf16", [500, 460, 300], [300, 360, 600], 2, dict(Hq=16, Hkv=2, d=128)),  # split chunks
+    ("bf16", LONG, LONGER, 19, dict(Hq=8, Hkv=8, d=64)),                    # the work list
+    ("f32", [128, 100], [150, 78], 0, dict(Hq=8, Hkv=2, d=64)),
+]
+
+
+@pytest.mark.parametrize("case", range(len(OTHER_WORDS)))
+def test_words_of_another_batch_stay_in_the_workspace(jet, case):
+    # a layout whose words hold a longer prefix than the sizes that the workspace was
+    # planned for: that request is left out and reported, nothing is written past the
+    # plan's bytes, and the other requests get their answers
+    import torch
+    dtype, planned, worded, long, over = OTHER_WORDS[case]
+    w = dataclasses.replace(jet_synth.WORKLOADS["tiny"], dtype=dtype, **over)
+    R = len(planned)
+
+    def problem(pl):
+        return jet_synth.custom_problem(w, pl, [2] * R, [3] * (2 * R), [1] * (6 * R), seed=180 + case)
+
+    step, _, _ = build_step(jet, problem(planned))
+    p = problem(worded)
+    x = {n: jet_synth.torch_tensor(p, n, device="cuda")
+         for n in ("q", "k_pre", "v_pre", "k_cand", "v_cand")}
+    words = jet.jet_layout_build(p.prefix_len, p.n_cand, p.cand_len, p.target_ids, w.V).words
+    step.layout.words.copy_(torch.from_numpy(words.copy()).to(step.layout.words.device))
+    need = jet.jet_workspace_bytes(step.host_layout.sizes, step.dims)
+    ws = torch.full((need + (8 << 20),), 0x5A, dtype=torch.uint8, device="cuda")
+    jet.jet_prefix_attend(step.layout, step.dims, x["q"], x["k_pre"], x["v_pre"], x["k_cand"],
+                          x["v_cand"], step.o, ws, ws_bytes=need)
+    torch.cuda.synchronize()
+    assert jet.jet_device_status() == 10  # JET_ERR_DEVICE
+    assert bool((ws[need:] == 0x5A).all())
+    lay = oracle_layout(p)
+    rows = [n for n in range(p.N) if lay["row_req"][n] != long]
+    rows = rows[:30] + rows[-10:]
+    check_attention(lay, p, step.o.float().cpu().numpy(), sorted(set(rows)),
+                    TOL_ATTN_BF16 if dtype == "bf16" else TOL_ATTN_F32)
