@@ -91,8 +91,9 @@ struct TcArgs {
   int* status;
   int N, T, V, D;
   int Nt, n_tt, units, nkb, stages, vtiles;
-  int tile_blk, tile_more;  // 16-row blocks of a token tile; tiles that have one more
-                            // (not mxfp8: its tiles have Nt rows)
+  // token tiles of blk-row blocks: tile_blk of them each and one more in the first
+  // tile_more tiles; whether their order rotates (mxfp8: tiles of Nt rows)
+  int blk, tile_blk, tile_more, rotate;
   uint32_t tt_inv, worker_inv;  // for div_rem by n_tt and by the number of workers
   uint32_t tmem_cols;
   uint32_t buf_cols;     // columns of one accumulator
@@ -133,13 +134,16 @@ __device__ __forceinline__ Unit unit_of(const TcArgs& a, int u, int workers) {
     x.cols = a.Nt;
     return x;
   }
-  if (a.n_tt == 1) return Unit{u, 0, 0, 16 * a.tile_blk};
+  if (a.n_tt == 1) return Unit{u, 0, 0, a.blk * a.tile_blk};
   const int2 at = div_rem(unsigned(u), unsigned(a.n_tt), a.tt_inv);
-  const int rot = div_rem(unsigned(u - at.y), unsigned(workers), a.worker_inv).x;
   x.vg = at.x;
-  x.tt = div_rem(unsigned(at.y + rot), unsigned(a.n_tt), a.tt_inv).y;
-  x.t0 = 16 * (x.tt * a.tile_blk + min(x.tt, a.tile_more));
-  x.cols = 16 * (a.tile_blk + (x.tt < a.tile_more ? 1 : 0));
+  x.tt = at.y;
+  if (a.rotate) {
+    const int rot = div_rem(unsigned(u - at.y), unsigned(workers), a.worker_inv).x;
+    x.tt = div_rem(unsigned(at.y + rot), unsigned(a.n_tt), a.tt_inv).y;
+  }
+  x.t0 = a.blk * (x.tt * a.tile_blk + min(x.tt, a.tile_more));
+  x.cols = a.blk * (a.tile_blk + (x.tt < a.tile_more ? 1 : 0));
   return x;
 }
 
@@ -699,6 +703,17 @@ int max_pairs(K kern, size_t smem) {
   return n;
 }
 
+// K slices of a row of `esize`-byte elements
+int k_slices(const jet_dims& d, int esize) { return (d.D * esize + kBKBytes - 1) / kBKBytes; }
+
+// Rows past one token tile go to CTA pairs from this many K slices on (D 1,024 in
+// bf16, 2,048 in e4m3). With fewer, a unit's epilogue (31 exponentials a column of
+// 32 vocabulary rows) takes longer than its products, and a pair, whose next unit
+// waits for two epilogues, is no faster or slower: 542 rows x 512 x 32,000 34.0 us on
+// pairs, 33.4 on single CTAs, e4m3 with D 1,024 41.8 and 41.0; at the line 37.2 and
+// 38.6 (bf16, D 1,024), 46.7 and 47.7 (e4m3, D 2,048).
+constexpr int kPairSlices = 16;
+
 // one launch of the LM head on bf16 operands, or e4m3 hidden codes with e4m3
 // or block-scaled 4-bit weights, per-row weight scales and per-token hidden scales
 template <int FMT, bool PAIR>
@@ -718,6 +733,16 @@ cudaError_t launch_head(const jet_layout& lay, const jet_dims& d, const ScorePla
   }
   const int esize = F8 ? 1 : 2;
   TcArgs a{};
+  a.blk = 16;
+  a.rotate = 1;
+  if (!PAIR && !W4 && !MX && n_tt > 1 && k_slices(d, esize) < kPairSlices) {
+    // the epilogue sets the pace, and takes 32 rows at a time: tiles of 32-row
+    // blocks, in order (2,190 rows x 512 x 151,936: 429 us with 16-row blocks that
+    // rotate, 427 with 32-row ones, 418 in order)
+    a.blk = 32;
+    a.rotate = 0;
+    Nt = (n.N + 32 * n_tt - 1) / (32 * n_tt) * 32;
+  }
   a.wait_ns = wait_budget_ns();
   a.hold_first = test_stall();
   a.target_ids = lay.target_ids;
@@ -737,12 +762,12 @@ cudaError_t launch_head(const jet_layout& lay, const jet_dims& d, const ScorePla
   a.Nt = Nt;
   a.n_tt = n_tt;
   // mxfp8 lays the hidden states' scale factors out by tiles of Nt rows
-  const int nblk = (n.N + 15) / 16;
+  const int nblk = (n.N + a.blk - 1) / a.blk;
   a.tile_blk = nblk / n_tt;
   a.tile_more = nblk % n_tt;
   a.units = (PAIR ? (plan.vtiles + 1) / 2 : plan.vtiles) * n_tt;
   a.vtiles = plan.vtiles;
-  a.nkb = (d.D * esize + kBKBytes - 1) / kBKBytes;
+  a.nkb = k_slices(d, esize);
   const int b_rows = PAIR ? Nt / 2 : Nt;  // token-tile rows one CTA loads
   const int a_bytes = kBM * kBKBytes, b_bytes = b_rows * kBKBytes;
   const int stage_bytes = a_bytes + b_bytes + (W4 ? 1024 : MX ? 2048 : 0);
@@ -804,14 +829,15 @@ cudaError_t launch_head(const jet_layout& lay, const jet_dims& d, const ScorePla
   return launch_pdl(kern, dim3(grid), dim3(kThreads), smem, st, tmW, tmH, a);
 }
 
-// More than one token tile: on CTA pairs (tcgen05 cta_group::2, 256 vocabulary
-// rows), which halves the hidden-state bytes each SM takes in: 2,405 rows x 2048
-// x 151,936 in the whole step 1,492 -> 1,370 us, 355 rows x 4096 353 -> 326 us.
-// e4m3: 355 rows x 4096 195 -> 179 us, 300 rows x 5120 215 -> 190 us.
-// With a single tile the weights' stream from HBM sets the pace (93 % of the
-// copy rate on single CTAs). A limit of one SM (jet_dims.max_sms) leaves no pair.
-bool use_pairs(const jet_layout& lay, const jet_dims& d) {
-  return lay.n.N > kMaxNt && d.max_sms != 1;
+// More than one token tile and K slices enough (kPairSlices): on CTA pairs
+// (tcgen05 cta_group::2, 256 vocabulary rows), which halves the hidden-state bytes
+// each SM takes in: 2,405 rows x 2048 x 151,936 in the whole step 1,492 -> 1,370 us,
+// 355 rows x 4096 353 -> 326 us. e4m3: 355 rows x 4096 195 -> 179 us, 300 rows x
+// 5120 215 -> 190 us. With a single tile the weights' stream from HBM sets the pace
+// (93 % of the copy rate on single CTAs). A limit of one SM (jet_dims.max_sms)
+// leaves no pair.
+bool use_pairs(const jet_layout& lay, const jet_dims& d, int esize) {
+  return lay.n.N > kMaxNt && d.max_sms != 1 && k_slices(d, esize) >= kPairSlices;
 }
 
 }  // namespace
@@ -819,7 +845,7 @@ bool use_pairs(const jet_layout& lay, const jet_dims& d) {
 cudaError_t launch_lmhead_tc(const jet_layout& lay, const jet_dims& d, const ScorePlan& plan,
                              const void* hidden, const void* w_lm, void* ws, int* status,
                              cudaStream_t st) {
-  if (use_pairs(lay, d))
+  if (use_pairs(lay, d, 2))
     return launch_head<kFmtBf16, true>(lay, d, plan, hidden, nullptr, w_lm, nullptr, ws, status,
                                        st);
   return launch_head<kFmtBf16, false>(lay, d, plan, hidden, nullptr, w_lm, nullptr, ws, status,
@@ -829,7 +855,7 @@ cudaError_t launch_lmhead_tc(const jet_layout& lay, const jet_dims& d, const Sco
 cudaError_t launch_lmhead_e4m3(const jet_layout& lay, const jet_dims& d, const ScorePlan& plan,
                                const uint8_t* h_q, const float* h_scale, const uint8_t* w_q,
                                const float* w_scale, void* ws, int* status, cudaStream_t st) {
-  if (use_pairs(lay, d))
+  if (use_pairs(lay, d, 1))
     return launch_head<kFmtE4m3, true>(lay, d, plan, h_q, h_scale, w_q, w_scale, ws, status, st);
   return launch_head<kFmtE4m3, false>(lay, d, plan, h_q, h_scale, w_q, w_scale, ws, status, st);
 }

@@ -1,7 +1,7 @@
-"""The LM head on CTA pairs (more than 256 rows) against the oracle: rows just
-past one token tile and at uneven shares of 16-row blocks, odd numbers of
-vocabulary tiles, and limits on the SMs it may use (one SM leaves no pair),
-which must not change a result."""
+"""The LM head of more than 256 rows against the oracle, on CTA pairs (from 16 K
+slices on) and on single CTAs: rows just past one token tile and at uneven shares of
+16- and 32-row blocks, odd numbers of vocabulary tiles, and limits on the SMs it may
+use (one SM leaves no pair), which must not change a result."""
 import dataclasses
 
 import numpy as np
@@ -13,8 +13,12 @@ from gpu_common import TOL_LOGPROB, dims_for, oracle_layout
 
 pytestmark = pytest.mark.gpu
 
-# (rows of the one request - a shared row and one candidate's fed tokens, V, D)
-CASES = [(257, 300, 72), (272, 129, 64), (400, 1000, 200), (513, 640, 136), (529, 127, 64)]
+# (rows of the one request - a shared row and one candidate's fed tokens, V, D): single
+# CTAs, then pairs in both formats, in bf16 alone (15 and 16 K slices are D 960 and 961
+# there, twice that in e4m3), and in neither
+CASES = [(257, 300, 72), (272, 129, 64), (400, 1000, 200), (513, 640, 136), (529, 127, 64),
+         (257, 300, 1928), (272, 129, 2048), (400, 1000, 1992), (513, 640, 1928),
+         (529, 127, 2048), (609, 300, 968), (609, 300, 960)]
 
 
 @pytest.mark.parametrize("case", range(len(CASES)))
