@@ -1059,10 +1059,8 @@ cudaError_t launch_dh(const jet_layout& lay, const jet_dims& d, const AttnPlan& 
   a.splits = plan.splits;
   a.qgroups = plan.qgroups;
   a.n_all = (long long)n.R * d.Hkv * plan.qgroups * plan.splits;
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-    return cudaErrorInvalidValue;
+  const int sms = sm_count();
+  if (sms < 1) return cudaErrorInvalidValue;
   const int grid = int(std::max<long long>(1, std::min<long long>(sms, a.n_all)));
   a.sorted = plan.sorted;
   cudaError_t e = cudaSuccess;
@@ -1138,10 +1136,8 @@ cudaError_t launch_prefill_dh(const jet_layout& lay, const jet_dims& d, const vo
   e = cudaFuncSetAttribute(attend_prefix_tc_kernel<DH>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-    return cudaErrorInvalidValue;
+  const int sms = sm_count();
+  if (sms < 1) return cudaErrorInvalidValue;
   const int grid = int(std::max<long long>(1, std::min<long long>(sms, a.n_all)));
   return launch_pdl(attend_prefix_tc_kernel<DH>, dim3(grid), dim3(kThreads), smem, st, tmQ, tmK,
                     tmV, tmK, tmV, a);

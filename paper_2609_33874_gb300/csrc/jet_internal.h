@@ -53,6 +53,14 @@ int test_stall();
 // Counts one kernel launch of this library (jet_launch_count).
 void note_launch();
 
+// ---- the current device (occupancy.cu) ---------------------------------------------
+// Its SMs; 0 when it cannot be asked.
+int sm_count();
+// The clusters of two CTAs of `kernel` (threads each, smem bytes of dynamic shared
+// memory, which its attribute must already allow) that it holds at once, at least 1.
+// Asked once per device, kernel and smem.
+int resident_pairs(const void* kernel, int threads, size_t smem);
+
 // ---- launches ------------------------------------------------------------------
 // Stream-ordered launch with programmatic stream serialization: the kernel may
 // begin (up to its pdl_begin()) while the previous kernel of the stream ends,

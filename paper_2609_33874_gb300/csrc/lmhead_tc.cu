@@ -48,7 +48,6 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
-#include <atomic>
 #include <mutex>
 
 #include "jet_device.cuh"
@@ -667,42 +666,6 @@ bool encode_w4_codes(CUtensorMap* map, const void* base, int rows, int kd) {
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int sm_count() {
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  return n;
-}
-
-}  // namespace
-
-namespace {
-
-// clusters of two CTAs of `kern` that can be resident at once; asked once per kernel
-template <typename K>
-int max_pairs(K kern, size_t smem) {
-  static std::atomic<int> cached{0};  // any thread may ask first
-  if (const int c = cached.load(std::memory_order_relaxed)) return c;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(2);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cudaLaunchAttribute cl{};
-  cl.id = cudaLaunchAttributeClusterDimension;
-  cl.val.clusterDim.x = 2;
-  cl.val.clusterDim.y = 1;
-  cl.val.clusterDim.z = 1;
-  cfg.attrs = &cl;
-  cfg.numAttrs = 1;
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
-    cudaGetLastError();
-    return std::max(1, sm_count() / 2);
-  }
-  cached.store(n, std::memory_order_relaxed);
-  return n;
-}
-
 // K slices of a row of `esize`-byte elements
 int k_slices(const jet_dims& d, int esize) { return (d.D * esize + kBKBytes - 1) / kBKBytes; }
 
@@ -819,7 +782,7 @@ cudaError_t launch_head(const jet_layout& lay, const jet_dims& d, const ScorePla
   };
   a.tt_inv = inverse(n_tt);
   if (PAIR) {
-    const int pairs = std::max(1, std::min(a.units, std::min(sms / 2, max_pairs(kern, smem))));
+    const int pairs = std::max(1, std::min(a.units, std::min(sms / 2, resident_pairs(reinterpret_cast<const void*>(kern), kThreads, smem))));
     a.worker_inv = inverse(pairs);
     return launch_pdl_pairs(kern, dim3(unsigned(2 * pairs)), dim3(kThreads), smem, st, tmW, tmH,
                             a);

@@ -34,7 +34,6 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
-#include <atomic>
 #include <mutex>
 
 #include "jet_device.cuh"
@@ -711,32 +710,6 @@ bool encode_3d(CUtensorMap* map, const void* base, int rows, int heads, int DH, 
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// clusters of two CTAs of `kern` that can be resident at once (the static
-// schedule deals the items to that many pairs); asked once per kernel
-template <typename K>
-int max_pairs(K kern, size_t smem) {
-  static std::atomic<int> cached{0};  // any thread may ask first
-  if (const int c = cached.load(std::memory_order_relaxed)) return c;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(2);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cudaLaunchAttribute cl{};
-  cl.id = cudaLaunchAttributeClusterDimension;
-  cl.val.clusterDim.x = 2;
-  cl.val.clusterDim.y = 1;
-  cl.val.clusterDim.z = 1;
-  cfg.attrs = &cl;
-  cfg.numAttrs = 1;
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
-    cudaGetLastError();
-    return 1;
-  }
-  cached.store(n, std::memory_order_relaxed);
-  return n;
-}
-
 }  // namespace
 
 template <int DH>
@@ -772,7 +745,9 @@ cudaError_t launch_prefill_pair(const jet_layout& lay, const jet_dims& d, const 
   if (e != cudaSuccess) return e;
   const long long items =
       (long long)n.R * d.Hkv * ((n.max_prefix + 2 * a.rb - 1) / (2 * a.rb));
-  const int pairs = int(std::max<long long>(1, std::min<long long>(max_pairs(kern, smem), items)));
+  // the static schedule deals the items to the pairs that are resident at once
+  const int held = resident_pairs(reinterpret_cast<const void*>(kern), kThreads, smem);
+  const int pairs = int(std::max<long long>(1, std::min<long long>(held, items)));
   return launch_pdl_pairs(kern, dim3(unsigned(2 * pairs)), dim3(kThreads), smem, st, tmQ, tmK,
                           tmV, a);
 }

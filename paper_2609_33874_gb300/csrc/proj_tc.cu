@@ -33,7 +33,6 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
-#include <atomic>
 #include <mutex>
 
 #include "jet_device.cuh"
@@ -562,37 +561,6 @@ bool encode_rows(CUtensorMap* map, const void* base, int rows, int K, int ld, in
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int sm_count() {
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  return n;
-}
-
-// clusters of two CTAs of `kern` that can be resident at once (one CTA per SM:
-// the SM pairs the GPCs offer); asked once per kernel
-template <typename K>
-int max_pairs(K kern, size_t smem) {
-  static std::atomic<int> cached{0};  // any thread may ask first
-  if (const int c = cached.load(std::memory_order_relaxed)) return c;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(2);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cudaLaunchAttribute cl{};
-  cl.id = cudaLaunchAttributeClusterDimension;
-  cl.val.clusterDim.x = 2;
-  cl.val.clusterDim.y = 1;
-  cl.val.clusterDim.z = 1;
-  cfg.attrs = &cl;
-  cfg.numAttrs = 1;
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1)
-    n = std::max(1, sm_count() / 2);
-  cached.store(n, std::memory_order_relaxed);
-  return n;
-}
-
 // the RMSNorm a residual projection's output feeds (h null: none)
 struct Norm {
   const void* g;
@@ -711,7 +679,7 @@ cudaError_t launch_epi(const void* x, int N, int K, int ldx, const void* w, int 
   auto kern = a.splits > 1 ? proj_tc_kernel<kPartial> : proj_tc_kernel<EPI>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
-  const int clusters = std::max(1, std::min(a.units, max_pairs(kern, smem)));
+  const int clusters = std::max(1, std::min(a.units, resident_pairs(reinterpret_cast<const void*>(kern), kThreads, smem)));
   e = launch_pdl_pairs(kern, dim3(unsigned(2 * clusters)), dim3(kThreads), smem, st, tmW, tmX, tmXt, a);
   if (e != cudaSuccess) return e;
   if (splits_out) {

@@ -50,6 +50,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "jet_device.cuh"
@@ -1003,14 +1004,6 @@ bool encode_tokens(CUtensorMap* map, const void* base, int tokens, int Hl) {
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int sm_count() {
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-    return 1;
-  return n;
-}
-
 }  // namespace
 
 bool scan_tc_supported(const jet_dims& d) {
@@ -1028,7 +1021,7 @@ cudaError_t launch_scan_tc(const jet_layout& lay, const jet_dims& d, int rule,
       !encode_tokens(&tmV, v, n.total_prefix, d.Hl))
     return cudaErrorInvalidValue;
   const long long items = (long long)n.R * d.Hl;
-  const int sms = sm_count();  // one CTA per SM
+  const int sms = std::max(1, sm_count());  // one CTA per SM
   const bool gla = rule == JET_RECUR_GLA, many = items > sms;
   auto kern = gla ? (many ? scan_tc_kernel<false, true> : scan_tc_kernel<false, false>)
                   : (many ? scan_tc_kernel<true, true> : scan_tc_kernel<true, false>);
