@@ -23,8 +23,7 @@ namespace {
 constexpr int kQV = 16;       // query vectors per CTA
 constexpr int kKT = 32;       // keys per tile
 constexpr int kThreads = 256;
-constexpr long long kTargetCtas = 608;  // about four CTAs per SM on 152 SMs
-constexpr int kPlanSMs = 152;           // GB300
+constexpr long long kTargetCtas = 4 * kPlanSMs;
 constexpr int kMinChunkTc = 640;        // keys
 constexpr int kFewGroups = 22, kFewItems = 44, kLeastChunk = 192;
 

@@ -967,11 +967,11 @@ bool encode_3d(CUtensorMap* map, const void* base, int rows, int heads, int DH, 
 // candidate's own keys) and normalise. Single-chunk requests were written by
 // the attention kernel itself; it also left every chunk's (m, l) in place, empty
 // for the chunks a request does not have, so that nothing here waits for the
-// layout.
+// layout. `ahead`: the partials are read beside their (m, l), wanted or not.
 template <int DH>
 __global__ void __launch_bounds__(128)
 attend_combine_kernel(const int32_t* __restrict__ row_req, int N, int R, int Hq, int splits,
-                      const float* __restrict__ o_part,
+                      bool ahead, const float* __restrict__ o_part,
                       const float2* __restrict__ ml_part, __nv_bfloat16* __restrict__ o,
                       int* status) {
   pdl_begin();
@@ -982,11 +982,6 @@ attend_combine_kernel(const int32_t* __restrict__ row_req, int N, int R, int Hq,
   const int r = row_req[n];
   // written by the attention kernel itself (l = -1 in the first chunk's place)
   const bool direct = ml_part[size_t(n) * Hq + h].y < 0.f;
-  // partials read beside their (m, l), wanted or not, while the grid is one that
-  // the chip holds at once: then a memory latency is all that counts (one request
-  // of 500 keys 13.5 -> 13.1 us); in a larger grid the rows of short requests are
-  // traffic (64 requests of 100 - 2,000 keys 46.4 -> 48.2 us)
-  const bool ahead = gridDim.x <= 152 * 8;
   if (!ahead && direct) return;
   constexpr int PER = DH / 32;
   float acc[PER];
@@ -1074,9 +1069,12 @@ cudaError_t launch_dh(const jet_layout& lay, const jet_dims& d, const AttnPlan& 
   e = launch_pdl(attend_prefix_tc_kernel<DH>, dim3(grid), dim3(kThreads), smem, st, tmQ, tmK, tmV,
                  tmKc, tmVc, a);
   if (e != cudaSuccess || plan.splits <= 1) return e;
-  const long long warps = (long long)n.N * d.Hq;
-  return launch_pdl(attend_combine_kernel<DH>, dim3(unsigned((warps + 3) / 4)), dim3(128), 0, st,
-                    lay.row_req, n.N, n.R, d.Hq, plan.splits, o_part, ml_part,
+  // ahead while the grid is one that the chip holds at once: then a memory latency is
+  // all that counts (one request of 500 keys 13.5 -> 13.1 us); in a larger grid the
+  // rows of short requests are traffic (64 requests of 100 - 2,000 keys 46.4 -> 48.2 us)
+  const long long blocks = ((long long)n.N * d.Hq + 3) / 4;
+  return launch_pdl(attend_combine_kernel<DH>, dim3(unsigned(blocks)), dim3(128), 0, st,
+                    lay.row_req, n.N, n.R, d.Hq, plan.splits, blocks <= 8LL * sms, o_part, ml_part,
                     static_cast<__nv_bfloat16*>(o), status);
 }
 

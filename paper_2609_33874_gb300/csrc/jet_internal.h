@@ -15,6 +15,9 @@ namespace jet {
 int* device_status_ptr();
 
 // ---- workspace plans -----------------------------------------------------------
+// Plans are functions of the shapes alone, so that the bytes asked for fit the launch
+// on any device: they reckon with a GB300's SMs.
+constexpr int kPlanSMs = 152;
 constexpr int kVocabTile = 128;  // vocabulary entries per LM-head partial
 // 4-bit weights, per (128 vocabulary rows, 128-element K slice): 128 x 64
 // bytes of packed E2M1 codes (in the row-major code region) and a 512-byte

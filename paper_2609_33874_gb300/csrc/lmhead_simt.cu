@@ -218,12 +218,12 @@ cudaError_t launch_mr(const jet_layout& lay, const jet_dims& d, const ScorePlan&
   float2* part = reinterpret_cast<float2*>(base + plan.part_off);
   float* z_tgt = reinterpret_cast<float*>(base + plan.ztgt_off);
   const size_t smem = smem_bytes<MR>();
-  // pairs while both CTAs of every tile find an SM (152 of them) of their own: a
+  // pairs while both CTAs of every tile find an SM of their own: a
   // one-request step of 7 rows and 8,192 entries takes 36.8 us of D 1,024 without
   // them, 28.7 with, 67.6 and 45.8 of D 2,560, 23.4 both ways of D 512 and below
   // (its launches); past that the halves would queue
   const long long row_tiles = (n.N + MR - 1) / MR;
-  const bool pair = 2 * row_tiles * plan.vtiles <= 152;
+  const bool pair = 2 * row_tiles * plan.vtiles <= sm_count();
   const auto kern = pair ? lmhead_simt_kernel<MR, true> : lmhead_simt_kernel<MR, false>;
   const cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));

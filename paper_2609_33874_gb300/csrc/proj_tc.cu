@@ -593,7 +593,6 @@ struct Tiling {
 // a tail in narrower token tiles that all pairs share (the gate and up projection of
 // 24,576 features: 76 slices, then 20 in three tiles each): the stack takes 496 us of
 // 178 rows without it, 481 with; 618 of 355, now 601; 685 of 444, now 674.
-constexpr int kPlanSMs = 152;
 Tiling tiling(int N, int O, int K, bool split) {
   const int pairs = kPlanSMs / 2, least = (N + kMaxNt - 1) / kMaxNt;
   auto tiles = [&](int c, int& nt, int& n_tt) {  // c tiles, or fewer once rounded
