@@ -104,15 +104,18 @@ __device__ __forceinline__ void combine_chunks(bool ahead, int splits, int N, in
   if (ahead) load(0);
   for (int s32 = 0; s32 < splits; s32 += 32) {
     if (s32 > 0) ml = load_ml(s32);
-    if (!(ml.y > 0.f)) ml = make_float2(-INFINITY, 0.f);  // an empty chunk
+    // an empty chunk has l = 0; a NaN l (a NaN score) counts, whatever its maximum,
+    // and so does a chunk whose weight underflows (0 x an infinite output is NaN)
+    const bool held = ml.y != 0.f;
+    if (!held) ml.x = -INFINITY;
     const float mn = fmaxf(m, warp_max(ml.x));
     const float keep = mn == -INFINITY ? 1.f : exp2f(m - mn);
-    const float w = ml.x == -INFINITY ? 0.f : exp2f(ml.x - mn);
+    const float w = held ? exp2f(ml.x - mn) : 0.f;
     l = l * keep + warp_sum(ml.y * w);
     m = mn;
 #pragma unroll
     for (int i = 0; i < PER; ++i) acc[i] *= keep;
-    const unsigned some = __ballot_sync(0xffffffffu, w > 0.f);
+    const unsigned some = __ballot_sync(0xffffffffu, held);
     for (int s0 = s32; s0 < min(s32 + 32, splits); s0 += kGroup) {
       if (!(some >> (s0 & 31) & ((1u << kGroup) - 1))) continue;  // all empty
       if (!ahead || s0 > 0) load(s0);
@@ -120,7 +123,7 @@ __device__ __forceinline__ void combine_chunks(bool ahead, int splits, int N, in
       for (int g = 0; g < kGroup; ++g) {
         const float ws = __shfl_sync(0xffffffffu, w, (s0 + g) & 31);
         // an empty chunk's outputs were not written
-        if (s0 + g < splits && ws > 0.f) {
+        if (some >> ((s0 + g) & 31) & 1u) {
 #pragma unroll
           for (int i = 0; i < PER; ++i) acc[i] = fmaf(ws, v[g][i], acc[i]);
         }

@@ -81,3 +81,44 @@ def test_words_of_another_batch_stay_in_the_workspace(jet, case):
     rows = rows[:30] + rows[-10:]
     check_attention(lay, p, step.o.float().cpu().numpy(), sorted(set(rows)),
                     TOL_ATTN_BF16 if dtype == "bf16" else TOL_ATTN_F32)
+
+
+SPLIT = [
+    ("bf16", 500, dict(Hq=16, Hkv=2, d=128)),   # chunks of 192 keys
+    ("bf16", 6000, dict(Hq=8, Hkv=2, d=64)),
+    ("bf16", 100, dict(Hq=8, Hkv=2, d=256)),    # one chunk, written directly
+    ("f32", 100, dict(Hq=8, Hkv=2, d=64)),      # four chunks
+]
+
+
+@pytest.mark.parametrize("case", range(len(SPLIT)))
+@pytest.mark.parametrize("what", ["nan_key", "inf_value"])
+def test_non_finite_inputs_reach_the_output(jet, case, what):
+    # a NaN key makes the outputs of its kv head's query heads NaN, an infinite value
+    # its column of them non-finite, also where the prefix is split and where the
+    # chunk of that key has no weight left against the others
+    import torch
+    dtype, P, over = SPLIT[case]
+    w = dataclasses.replace(jet_synth.WORKLOADS["tiny"], dtype=dtype, **over)
+    p = jet_synth.custom_problem(w, [P], [2], [3, 2], [1] * 5, seed=190 + case)
+    step, x, w_lm = build_step(jet, p)
+    at, g = P // 3, w.Hq // w.Hkv
+    if what == "nan_key":
+        x["k_pre"][at, 1, 5] = float("nan")
+    else:
+        x["v_pre"][at, 1, 5] = float("inf")
+        # the last key's score is larger by 416, 600 powers of two of weight
+        x["q"][:, :, 0] = 16.0
+        x["k_pre"][:, :, 0] = 0.0
+        x["k_pre"][P - 1, :, 0] = 26.0 * w.d ** 0.5
+    jet.jet_prefix_attend(step.layout, step.dims, x["q"], x["k_pre"], x["v_pre"], x["k_cand"],
+                          x["v_cand"], step.o, step.ws)
+    torch.cuda.synchronize()
+    assert jet.jet_device_status() == 0
+    o = step.o.float().cpu()
+    assert torch.isfinite(o[:, :g]).all()  # the other kv head's
+    if what == "nan_key":
+        assert torch.isnan(o[:, g:]).all()
+    else:
+        assert not torch.isfinite(o[:, g:, 5]).any()
+        assert torch.isfinite(o[:, g:, :5]).all() and torch.isfinite(o[:, g:, 6:]).all()
