@@ -37,6 +37,7 @@
 
 #include "jet_device.cuh"
 #include "jet_internal.h"
+#include "proj_tiling.h"
 #include "sm100_ptx.cuh"
 
 namespace jet {
@@ -44,10 +45,10 @@ namespace {
 
 using namespace sm100;
 
-constexpr int kBM = 128;            // weight rows per CTA (MMA M per CTA, TMEM lanes)
-constexpr int kBK = 64;             // bf16 elements per stage: 128 bytes
+constexpr int kBM = kProjRows;      // weight rows per CTA (MMA M per CTA, TMEM lanes)
+constexpr int kBK = kProjK;         // bf16 elements per stage: 128 bytes
 constexpr int kThreads = 192;
-constexpr int kMaxNt = 256;
+constexpr int kMaxNt = kProjMaxNt;
 constexpr uint64_t kDrainNs = 200000000ull;
 constexpr int kSmemLimit = 232448;
 // gate/up exchange (16 columns x 128 lanes f32) + barriers and flags
@@ -572,68 +573,8 @@ template <int EPI>
 cudaError_t launch_reduce(const ProjArgs& a, float* part, int N, int O, void* out, int ldo,
                           const void* res, cudaStream_t st);
 
-struct Tiling {
-  int n_tt, Nt, otiles, groups, nkb, splits;  // groups: 256-row weight slices
-  int tail_group, tail_n_tt, tail_Nt;  // slices from tail_group on in narrower tiles
-};
-
-// Token tiles of at most 256 rows (a multiple of 16: each CTA of a pair holds
-// half); units of 256 weight rows on CTA pairs; K split while the units still
-// fit the 76 SM pairs once, keeping at least 8 K slices per unit. A function
-// of the shapes only, so that the workspace planned for a call matches the
-// launch.
-// The number of tiles is the one of least cost: rounds of the SM pairs, times K
-// slices a unit, times a slice's time, which goes as Nt + 80 (the weights' share of
-// the bytes an SM takes in; 64 to 110 in place of 80 choose alike but for a few
-// sizes). Always the fewest tiles left the last round half empty: four layers of
-// D 4,096 and Dff 12,288 took 525 us of 178 rows, now 513; 643 of 355, now 634; 715
-// of 444, now 691; 851 of 555, now 808; 1,802 of 2,800, now 1,688. Splits over more
-// than one round gain up to 1 % there, but 355 rows take 1 - 2 % more.
-// Where the weight slices past the full rounds would leave most pairs idle, they are
-// a tail in narrower token tiles that all pairs share (the gate and up projection of
-// 24,576 features: 76 slices, then 20 in three tiles each): the stack takes 496 us of
-// 178 rows without it, 481 with; 618 of 355, now 601; 685 of 444, now 674.
 Tiling tiling(int N, int O, int K, bool split) {
-  const int pairs = kPlanSMs / 2, least = (N + kMaxNt - 1) / kMaxNt;
-  auto tiles = [&](int c, int& nt, int& n_tt) {  // c tiles, or fewer once rounded
-    nt = ((N + c - 1) / c + 15) / 16 * 16;
-    n_tt = (N + nt - 1) / nt;
-  };
-  auto rounds = [&](long long units) { return (units + pairs - 1) / pairs; };
-  Tiling best{};
-  long long best_cost = -1;
-  for (int c = least; c <= 2 * least + 2; ++c) {
-    Tiling t{};
-    tiles(c, t.Nt, t.n_tt);
-    t.otiles = (O + kBM - 1) / kBM;
-    t.groups = (t.otiles + 1) / 2;
-    t.nkb = (K + kBK - 1) / kBK;
-    t.tail_group = t.groups;
-    const int units = t.groups * t.n_tt;
-    t.splits = 1;
-    while (split && units * (t.splits + 1) <= pairs && t.nkb / (t.splits + 1) >= 8) ++t.splits;
-    const long long per_kb = (t.nkb + t.splits - 1) / t.splits;
-    long long cost = rounds((long long)units * t.splits) * per_kb * (t.Nt + 80);
-    if (best_cost < 0 || cost < best_cost) {
-      best = t;
-      best_cost = cost;
-    }
-    // the same, with the slices past its full rounds in narrower tiles
-    const int full = units / pairs, head = full * pairs / t.n_tt;
-    if (t.splits > 1 || full == 0 || head == t.groups) continue;
-    for (int ct = c + 1; ct <= 4 * c; ++ct) {
-      Tiling u = t;
-      tiles(ct, u.tail_Nt, u.tail_n_tt);
-      u.tail_group = head;
-      cost = (full * (t.Nt + 80) +
-              rounds((long long)(t.groups - head) * u.tail_n_tt) * (u.tail_Nt + 80)) * t.nkb;
-      if (cost * 100 < best_cost * 97) {
-        best = u;
-        best_cost = cost;
-      }
-    }
-  }
-  return best;
+  return projection_tiling(N, O, K, split, kPlanSMs / 2);
 }
 
 template <int EPI>
@@ -678,7 +619,8 @@ cudaError_t launch_epi(const void* x, int N, int K, int ldx, const void* w, int 
   auto kern = a.splits > 1 ? proj_tc_kernel<kPartial> : proj_tc_kernel<EPI>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
-  const int clusters = std::max(1, std::min(a.units, resident_pairs(reinterpret_cast<const void*>(kern), kThreads, smem)));
+  const int clusters = std::max(
+      1, std::min(a.units, resident_pairs(reinterpret_cast<const void*>(kern), kThreads, smem)));
   e = launch_pdl_pairs(kern, dim3(unsigned(2 * clusters)), dim3(kThreads), smem, st, tmW, tmX, tmXt, a);
   if (e != cudaSuccess) return e;
   if (splits_out) {
