@@ -37,6 +37,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 
 #include "attend_items.h"
@@ -153,7 +154,8 @@ __device__ __forceinline__ ItemGeo item_geo(const AttArgs& a, int4 it, bool* fit
   if (e.r < 0 || e.r >= a.R || e.kh < 0 || e.kh >= a.Hkv) return e;
   e.p0 = a.prefix_offset[e.r];
   e.P = a.prefix_offset[e.r + 1] - e.p0;
-  *fits = request_cut(a, e.p0, e.P, e.p0, e.P).nq > 0;
+  *fits = e.p0 >= 0 && e.P >= 1 && e.P <= a.total_prefix && e.p0 <= a.total_prefix - e.P &&
+          e.P <= (long long)a.qgroups * a.rb;
   if (!*fits || e.split != 0) return e;
   e.n0 = e.p0;
   e.nr = e.P;
@@ -1154,12 +1156,51 @@ size_t prefill_workspace_bytes(const jet_sizes& n, const jet_dims& d) {
   return 32 + 16 * size_t(n.R) * d.Hkv * qgroups;
 }
 
+namespace {
+
+// Whether SM pairs (prefill_tc.cu) finish the batch before single SMs do. A pair's
+// items are blocks of twice the positions: requests of few positions leave the second
+// half empty, and then twice the CTAs work beside each other on the halves. Rounds of
+// items, each its start and end and then its key tiles, in units of about 1.2 us; the
+// single SMs also launch their work list. The figures are fitted to 879 batches of 1 -
+// 256 requests of 1 - 2,000 positions: 64 requests of 63 (24/4 heads, d 256) 39.7 us
+// on pairs, 34.0 on single SMs; of 42, which fill the pairs' blocks, 23.8 and 25.9;
+// 256 of 64 (8/8 heads, d 128) 104 and 61. The choice is 0.3 % off the faster of the
+// two on average, 14 % at most.
+bool prefill_on_pairs(const jet_sizes& n, const jet_dims& d) {
+  struct Cost {
+    double start, tile, launch;
+  };
+  const Cost single = d.d == 128 ? Cost{4.6, 0.8, 3.0} : Cost{4.4, 0.8, 0.0};
+  const Cost pair = d.d == 128 ? Cost{4.0, 1.0, 0.0} : Cost{4.0, 0.8, 0.0};
+  const int rb = kBV / (d.Hq / d.Hkv);
+  const double P = double(n.total_prefix) / n.R;
+  const bool even = (long long)n.R * n.max_prefix == n.total_prefix;
+  auto time = [&](const Cost& c, int block, int keys_per_tile, int workers) {
+    const double most = (n.max_prefix + block - 1) / block;
+    const double blocks = even ? most : std::min(most, std::max(1.0, P / block + 0.5));
+    const double keys = (P + std::min(P, double(block))) / 2.0;
+    const double tiles = keys > keys_per_tile ? keys / keys_per_tile + 0.5 : 1.0;
+    const double rounds = std::ceil(double(n.R) * d.Hkv * blocks / workers);
+    return rounds * (c.start + c.tile * (tiles - 1.0)) + c.launch;
+  };
+  return time(single, rb, kBN, kPlanSMs) >= time(pair, 2 * rb, 128, kPlanSMs / 2);
+}
+
+}  // namespace
+
 cudaError_t launch_prefill_tc(const jet_layout& lay, const jet_dims& d, const void* q,
                               const void* k, const void* v, void* o, void* ws, int* status,
                               cudaStream_t st) {
   if (d.d == 64) return launch_prefill_dh<64>(lay, d, q, k, v, o, ws, status, st);
-  if (d.d == 128) return launch_prefill_pair<128>(lay, d, q, k, v, o, status, st);
-  if (d.d == 256) return launch_prefill_pair<256>(lay, d, q, k, v, o, status, st);
+  if (d.Hq / d.Hkv > kBV) return cudaErrorInvalidValue;
+  const bool pairs = prefill_on_pairs(lay.n, d);
+  if (d.d == 128)
+    return pairs ? launch_prefill_pair<128>(lay, d, q, k, v, o, status, st)
+                 : launch_prefill_dh<128>(lay, d, q, k, v, o, ws, status, st);
+  if (d.d == 256)
+    return pairs ? launch_prefill_pair<256>(lay, d, q, k, v, o, status, st)
+                 : launch_prefill_dh<256>(lay, d, q, k, v, o, ws, status, st);
   return cudaErrorInvalidValue;
 }
 

@@ -1,7 +1,7 @@
 """Prefill attention on SM pairs (head dimensions 128 and 256) against the
 oracle: prefixes around the 128-key tile and the pair's query block, more items
-than pairs with one or two tiles each (every role runs ahead of the others),
-and a running maximum that keeps growing, so that the output accumulator is
+than pairs of one tile each (every role runs ahead of the others), short prefixes
+that leave a pair's second half empty and run on single SMs, and a running maximum that keeps growing, so that the output accumulator is
 rescaled for some of a warp's vectors and not for others - also in the scoring
 step's attention, which shares that rule."""
 import dataclasses
@@ -21,7 +21,7 @@ CASES = [
     ([256, 41, 42, 43, 84, 85], dict(Hq=24, Hkv=4, d=256)),       # 42-position blocks
     ([255, 257, 384], dict(Hq=2, Hkv=2, d=128)),                  # g = 1: 256-position blocks
     ([3, 130, 2], dict(Hq=128, Hkv=1, d=128)),                    # g = 128: two positions
-    (list(range(1, 120)) * 2, dict(Hq=16, Hkv=4, d=256)),         # 952 items of one tile
+    (list(range(1, 120)) * 2, dict(Hq=16, Hkv=4, d=256)),         # single SMs: half of it empty
 ]
 
 
@@ -47,6 +47,23 @@ def test_prefill_pair_blocks(jet, case):
     rows = range(p.total_prefix) if p.total_prefix <= 600 else \
         sorted(set(rng.integers(0, p.total_prefix, 300).tolist()) | {0, p.total_prefix - 1})
     _check(p, got, list(rows), TOL_ATTN_BF16)
+
+
+SHORT = [
+    ([48] * 240, dict(Hq=16, Hkv=4, d=256)),        # pairs: 960 items of one tile
+    ([60] * 90, dict(Hq=8, Hkv=2, d=128)),          # pairs: 180 items of one tile
+    ([16] * 64, dict(Hq=32, Hkv=8, d=128)),         # half of a pair's block: single SMs
+    ([17, 31, 1] * 40, dict(Hq=16, Hkv=4, d=128)),  # single SMs
+    ([21] * 90, dict(Hq=24, Hkv=4, d=256)),         # single SMs
+]
+
+
+@pytest.mark.parametrize("case", range(len(SHORT)))
+def test_prefill_of_many_short_prefixes(jet, case):
+    pl, over = SHORT[case]
+    p = _problem(pl, over, 200 + case)
+    rows = np.random.default_rng(case).integers(0, p.total_prefix, 300).tolist()
+    _check(p, _prefill(jet, p), sorted(set(rows) | {0, p.total_prefix - 1}), _bar(p))
 
 
 def _grow(p, tensor="k_pre"):
