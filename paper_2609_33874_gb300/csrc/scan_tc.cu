@@ -46,7 +46,8 @@
 // 220 and 147 -> 141 us; 64 x 64 tokens 89 -> 62 and 64 -> 43 us; 24 x 100 - 4,000
 // tokens 671 -> 500 and 416 -> 319 us). Where it was lost before: bank conflicts and
 // address arithmetic in the inverse, one chunk's gates scanned inside its chain,
-// outputs written before the next chunk's X.
+// outputs written before the next chunk's X (of gated linear attention: in the place
+// of its state MMAs; 141 -> 138 us, 3 x 2,000 - 4,000 tokens 234 -> 213).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -694,15 +695,14 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         __syncwarp();
       } else {
         // gated linear attention: U = diag(b) V straight into TMEM
-        if (gt >= 0 && !last) {
-          decays(vec + (j + 1) % 3 * kVecFloats, gt, lane, ga, go, gb);
-          read_gates(j + 2);
-        }
-        okk = mbar_wait(bar_v, j & 1, wait_ns, abort_flag) &&
-              (j == 0 || (mbar_wait(bar_x, (j - 1) & 1, wait_ns, abort_flag) &&
-                          mbar_wait(u_free, (j - 1) & 1, wait_ns, abort_flag)));
+        // (g Q as soon as the previous X has read its own, and the next chunk's
+        // decays after this one is handed over: only U waits for d; with all of it
+        // in the chain 3 x 2,000 - 4,000 tokens took 234 us instead of 225)
+        okk = j == 0 || mbar_wait(bar_x, (j - 1) & 1, wait_ns, abort_flag);
+        if (okk) write_gq(j);
+        okk = okk && mbar_wait(bar_v, j & 1, wait_ns, abort_flag) &&
+              (j == 0 || mbar_wait(u_free, (j - 1) & 1, wait_ns, abort_flag));
         if (okk) {
-          write_gq(j);
           tc_fence_after();
           const uint8_t* vt = sm + kOffV;
           float uv[32];
@@ -717,6 +717,10 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         ok = group_and(1, okk);
         if (!ok) break;
         if (lane == 0) mbar_arrive(ready);
+        if (gt >= 0 && !last) {
+          decays(vec + (j + 1) % 3 * kVecFloats, gt, lane, ga, go, gb);
+          read_gates(j + 2);
+        }
         if (MANY && tid == kWalker) hand_out(j + 3);
         // neither V nor Q is read any more
         if (tid == 0 && !last) load_v(j + 1);
@@ -833,10 +837,10 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         mma_commit(bar_x);
       }
       __syncwarp();
-      // while X runs: the previous chunk's outputs, and this warpgroup's 64 state
-      // columns scaled by g_{C-1} for the last MMA to accumulate onto (X reads the
-      // hi/lo copy, not these)
-      if (pending) write_out(j - 1);
+      // while X runs: the previous chunk's outputs (delta rule), and this warpgroup's
+      // 64 state columns scaled by g_{C-1} for the last MMA to accumulate onto (X
+      // reads the hi/lo copy, not these)
+      if (DELTA && pending) write_out(j - 1);
       {
         const float g = vec[(j % 3) * kVecFloats + 320];
         float s0[32];
@@ -908,6 +912,9 @@ scan_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         mma_commit(bar_so);
       }
       __syncwarp();
+      // gated linear attention's X is half as long and hides the scaling alone: the
+      // outputs leave here (3 x 2,000 - 4,000 tokens 225 -> 213 us)
+      if (!DELTA && pending) write_out(j - 1);
       ok = group_and(2, mbar_wait(bar_so, j & 1, wait_ns, abort_flag));
       if (!ok) break;
       tc_fence_after();
