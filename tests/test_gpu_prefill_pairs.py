@@ -1,9 +1,10 @@
 """Prefill attention on SM pairs (head dimensions 128 and 256) against the
 oracle: prefixes around the 128-key tile and the pair's query block, more items
 than pairs of one tile each (every role runs ahead of the others), short prefixes
-that leave a pair's second half empty and run on single SMs, and a running maximum that keeps growing, so that the output accumulator is
-rescaled for some of a warp's vectors and not for others - also in the scoring
-step's attention, which shares that rule."""
+that leave a pair's second half empty and run on single SMs, and a running maximum
+that keeps growing, so that the output accumulator is rescaled for some of a warp's
+vectors and not for others - also in the scoring step's attention, which shares
+that rule."""
 import dataclasses
 
 import numpy as np

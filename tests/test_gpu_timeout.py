@@ -1,6 +1,6 @@
 """Failure detection without a GPU fault. Every wait between the roles of the
-tensor-core kernels (attention, LM head, decoder-stack projections) is
-bounded: a wait that runs past its budget makes the kernel stop issuing work,
+tensor-core kernels (attention, prefill, LM head, prefix scan, decoder-stack
+projections) is bounded: a wait that runs past its budget makes the kernel stop issuing work,
 let its copies and tensor-core operations in flight finish, free its tensor
 memory and return, with JET_ERR_TIMEOUT in the device status word. A wait
 that ends in time never reaches the budget check, so these tests make one
@@ -194,3 +194,77 @@ def test_prefix_scan_wait_runs_out(cuda, rule):
     torch.cuda.synchronize()
     assert cuda.jet_device_status() == JET_OK
     assert torch.equal(o, ref_o) and torch.equal(s_out, ref_s)
+
+
+@pytest.mark.parametrize("d,prefix", [(64, [300, 90]), (128, [300, 90]), (256, [700, 90]),
+                                      (128, [16] * 64)])
+def test_prefill_wait_runs_out(cuda, d, prefix):
+    # the prefill on SM pairs (both CTAs' roles; a second tile's copies are in flight
+    # when the first wait gives up), and on single SMs with its work list (head size
+    # 64, and many short prefixes)
+    import torch
+    w = dataclasses.replace(jet_synth.WORKLOADS["tiny"], dtype="bf16", Hq=32, Hkv=8, d=d)
+    R = len(prefix)
+    p = jet_synth.custom_problem(w, prefix, [1] * R, [1] * R, [0] * R, seed=62)
+    hl = cuda.jet_layout_build(p.prefix_len, p.n_cand, p.cand_len, p.target_ids, w.V)
+    dims = cuda.make_dims(cuda.DTYPE_BF16, Hq=w.Hq, Hkv=w.Hkv, d=d, D=w.D)
+    q, k, v = (jet_synth.torch_tensor(p, n, device="cuda") for n in ("q_pre", "k_pre", "v_pre"))
+    o = torch.empty(p.total_prefix, w.Hq, d, dtype=torch.bfloat16, device="cuda")
+    ws = torch.empty(cuda.jet_prefill_workspace_bytes(hl.sizes, dims) // 4 + 4,
+                     dtype=torch.float32, device="cuda")
+    lay = hl.to_device("cuda")
+
+    def fn():
+        cuda.jet_prefill_attend(lay, dims, q, k, v, o, ws)
+
+    _times_out_then_repeats(cuda, fn, lambda: o)
+
+
+@pytest.mark.parametrize("lm,D", [("bf16", 1024), ("e4m3", 2048)])
+def test_lm_head_pairs_wait_runs_out(cuda, lm, D):
+    # more than 256 rows and 16 K slices: the LM head on CTA pairs, several units each
+    from paper_2609_33874_gb300.step import ScoringStep, quantize_lm_head
+    w = dataclasses.replace(jet_synth.WORKLOADS["tiny"], dtype="bf16", V=20000, D=D)
+    p = jet_synth.custom_problem(w, [3], [1], [300], np.arange(300) * 7 % w.V, seed=63)
+    hl = cuda.jet_layout_build(p.prefix_len, p.n_cand, p.cand_len, p.target_ids, w.V)
+    dims = cuda.make_dims(cuda.DTYPE_BF16, Hq=w.Hq, Hkv=w.Hkv, d=w.d, D=D)
+    step = ScoringStep(hl, dims, cuda.DECIDE_ARGMAX, lm=lm)
+    hidden = jet_synth.torch_tensor(p, "hidden", device="cuda")
+    w_lm = jet_synth.torch_tensor(p, "w_lm", device="cuda")
+    if lm == "e4m3":
+        w_lm = quantize_lm_head(w_lm)
+    _times_out_then_repeats(cuda, lambda: step.score(hidden, w_lm), lambda: step.tok_logprob)
+
+
+@pytest.mark.parametrize("rule", ["delta", "gla"])
+def test_scan_of_several_items_wait_runs_out(cuda, rule):
+    # more (request, head) items than SMs: each CTA's walk through its items
+    import torch
+    w = dataclasses.replace(jet_synth.WORKLOADS["ordinal_hybrid"], Hl=16, dtype="bf16")
+    pl = [200, 64, 130, 1] * 5
+    R = len(pl)
+    p = jet_synth.custom_problem(w, pl, [1] * R, [1] * R, [0] * R, seed=64)
+    hl = cuda.jet_layout_build(p.prefix_len, p.n_cand, p.cand_len, p.target_ids, w.V)
+    dims = cuda.make_dims(cuda.DTYPE_BF16, Hl=w.Hl, dk=w.dk, dv=w.dv, D=w.D)
+    t = [jet_synth.torch_tensor(p, n, device="cuda")
+         for n in ("lq_pre", "lk_pre", "lv_pre", "alpha_pre", "beta_pre")]
+    out = torch.empty(p.total_prefix, w.Hl, w.dv, dtype=torch.bfloat16, device="cuda")
+    s_out = torch.empty(R, w.Hl, w.dk, w.dv, dtype=torch.float32, device="cuda")
+    lay = hl.to_device("cuda")
+    _times_out_then_repeats(
+        cuda, lambda: cuda.jet_prefill_state(lay, dims, *t, out, s_out, rule=cuda.RULES[rule]),
+        lambda: torch.cat([out.float().flatten(), s_out.flatten()]))
+
+
+def _times_out_then_repeats(cuda, fn, out):
+    """fn with the hook reports the timeout; without it, it does what it did before."""
+    import torch
+    fn()
+    torch.cuda.synchronize()
+    assert cuda.jet_device_status() == JET_OK
+    ref = out().clone()
+    assert _stalled(cuda, fn) == JET_ERR_TIMEOUT
+    fn()
+    torch.cuda.synchronize()
+    assert cuda.jet_device_status() == JET_OK
+    assert torch.equal(out(), ref)
