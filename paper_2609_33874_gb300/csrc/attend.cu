@@ -1,6 +1,6 @@
 // Shared-prefix cascade attention (Sec. 4.1, Fig. 1 "KV-cache text models"):
-// float32 prefix kernel, and the merge kernel shared with the bf16
-// tensor-core prefix kernel (attend_tc.cu). Partials are in base 2:
+// the plan of both types, and the float32 kernels (prefix chunks, then their merge
+// with the candidates' own keys); bf16 runs in attend_tc.cu. Partials are in base 2:
 // m = max of score log2(e), l = sum of 2^(score log2(e) - m).
 //
 // Every row of request r attends to the request's P_r prefix keys; a row fed
@@ -306,19 +306,24 @@ AttnPlan attn_plan(const jet_sizes& n, const jet_dims& d) {
   const int max_splits = std::max(1, (n.max_prefix + gran - 1) / gran);
   int chunk;
   if (tc) {
-    // the persistent kernel (one CTA per SM, longest items first) splits a
-    // request's prefix into near-equal chunks: no shorter than kMinChunkTc keys
-    // (an item's fixed cost - query block in, f32 partial out and read back by
-    // the combine - is worth about five 64-key tiles), and no finer than half
-    // of one SM's share of all key tiles, so that the schedule can balance
+    // the persistent kernel (one CTA per SM; items dealt out by their requests'
+    // lengths, or longest first from a list: `sorted` below) splits a request's
+    // prefix into near-equal chunks: no shorter than kMinChunkTc keys (an item's
+    // fixed cost - query block in, f32 partial out and read back by the combine - is
+    // worth about five 64-key tiles), and no finer than half of one SM's share of all
+    // key tiles, so that the schedule can balance
     const double avg_tiles = double(n.total_prefix) / n.R / 64.0 + 0.5;
     const double share = double(groups) * avg_tiles / kPlanSMs;  // tiles per SM
     int least = kMinChunkTc;
     // a few long prefixes leave most SMs idle at that length: then about
     // kFewItems chunks in all, of at least kLeastChunk keys (one 6,000-key request
-    // with two kv heads: 320 keys 17.5 us, 640 keys 19.8 us, 128 keys 21.3 us;
-    // 32 groups of 512 keys: unsplit 15.0 us, halves 16.9 us with the combine)
-    if (groups <= kFewGroups) {
+    // with two kv heads: 320 keys 17.5 us, 640 keys 19.8 us, 128 keys 21.3 us). Past
+    // kFewGroups the combine costs what shorter chunks gain, and from 19 groups on in
+    // prefixes of up to 448 keys too (d 256; as here and at 640 keys: 8 groups of 1,000
+    // keys 13.2 and 17.7 us, 16 groups 15.2 and 17.9, of 400 12.9 and 13.3; 20 groups
+    // of 200 - 1,200 16.5 and 18.7, of 200 - 600 14.9 and 15.5, of 400 14.0 and 13.4;
+    // 24 groups of 400 14.0 and 13.4, of 700 to 4,000 the same)
+    if (groups <= kFewGroups && (groups <= 18 || n.max_prefix > 448)) {
       const long long even = (long long)(double(groups) * avg_tiles / kFewItems + 0.999) * 64;
       least = int(std::max<long long>(kLeastChunk, std::min<long long>(kMinChunkTc, even)));
     }
