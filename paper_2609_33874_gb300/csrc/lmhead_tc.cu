@@ -797,10 +797,13 @@ cudaError_t launch_head(const jet_layout& lay, const jet_dims& d, const ScorePla
 // each SM takes in: 2,405 rows x 2048 x 151,936 in the whole step 1,492 -> 1,370 us,
 // 355 rows x 4096 353 -> 326 us. e4m3: 355 rows x 4096 195 -> 179 us, 300 rows x
 // 5120 215 -> 190 us. With a single tile the weights' stream from HBM sets the pace
-// (93 % of the copy rate on single CTAs). A limit of one SM (jet_dims.max_sms)
-// leaves no pair.
+// (93 % of the copy rate on single CTAs). An odd limit on the SMs (jet_dims.max_sms)
+// leaves one of them without a pair, which up to seven costs what pairs gain or more
+// (355 rows x 4,096 x 32,000 on 3 SMs 3,067 us in pairs, 2,390 alone; on 5 1,558 and
+// 1,433; on 7 1,062 and 1,033; on 9 790 and 808).
 bool use_pairs(const jet_layout& lay, const jet_dims& d, int esize) {
-  return lay.n.N > kMaxNt && d.max_sms != 1 && k_slices(d, esize) >= kPairSlices;
+  return lay.n.N > kMaxNt && (d.max_sms % 2 == 0 || d.max_sms > 7) &&
+         k_slices(d, esize) >= kPairSlices;
 }
 
 }  // namespace
