@@ -759,7 +759,7 @@ def run_prefill(args):
     flops = float(np.sum(4.0 * w.Hq * w.d * P * (P + 1) / 2))
     nbytes = p.total_prefix * (2 * w.Hq + 2 * w.Hkv) * w.d * 2  # Q, O, K, V once
     roof = _roof(flops, nbytes, ms, peaks)
-    roof.update(kernel="jet_prefill_attend (prefill_pair_kernel, or attend_prefix_tc_kernel for head size 64; causal)",
+    roof.update(kernel="jet_prefill_attend (prefill_pair_kernel; attend_prefix_tc_kernel for head size 64 and short prefixes; causal)",
                 algorithmic_flops=flops, algorithmic_bytes=nbytes, traffic=None,
                 peak_source=peaks["source"])
     parts["attend"] = dict(ms=round(ms, 4), roofline=roof, launches=n_att)

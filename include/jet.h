@@ -224,7 +224,8 @@ jet_status jet_prefix_attend(const jet_layout* lay, const jet_dims* dims, const 
  * bf16 only (else JET_ERR_UNSUPPORTED), d in {64, 128, 256}. Uses the layout's
  * prefix sizes only. ws/ws_bytes: scratch of at least
  * jet_prefill_workspace_bytes() (a work list of 16 bytes per block of
- * 128 / (Hq / Hkv) positions and key/value head).
+ * 128 / (Hq / Hkv) positions and key/value head, which batches of short
+ * prefixes use, and all of head size 64; asked for whatever the batch).
  */
 size_t jet_prefill_workspace_bytes(const jet_sizes* n, const jet_dims* dims);
 jet_status jet_prefill_attend(const jet_layout* lay, const jet_dims* dims, const void* q,
@@ -242,9 +243,9 @@ jet_status jet_prefill_attend(const jet_layout* lay, const jet_dims* dims, const
  *   s_out   [R, Hl, dk, dv] float32   the state after the prefix: the
  *           s_prefix every candidate forks from (Sec. 4.1)
  * Requests and heads run in parallel. bf16 states of 128 x 128 take the
- * chunked form on the tensor cores (64 tokens at a time, one CTA per
- * request and head; an exact rearrangement of the recurrence with float32-
- * like accuracy); float32 and other state shapes run the tokens one after
+ * chunked form on the tensor cores (64 tokens at a time; a CTA works through
+ * one request and head after another; an exact rearrangement of the recurrence
+ * with float32-like accuracy); float32 and other state shapes run the tokens one after
  * another (32- or 64-column slices of the state in parallel).
  */
 jet_status jet_prefill_state(const jet_layout* lay, const jet_dims* dims, int32_t rule,

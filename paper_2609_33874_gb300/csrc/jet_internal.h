@@ -135,8 +135,8 @@ cudaError_t launch_scan_tc(const jet_layout& lay, const jet_dims& d, int rule,
                            const float* s_init, const void* q, const void* k, const void* v,
                            const float* alpha, const float* beta, void* o, float* s_out,
                            int* status, cudaStream_t st);
-// causal self-attention over every request's prefix (bf16, tensor cores);
-// the workspace holds the work list
+// causal self-attention over every request's prefix (bf16, tensor cores): on single
+// SMs with a work list, which the workspace holds, or on pairs of SMs
 size_t prefill_workspace_bytes(const jet_sizes& n, const jet_dims& d);
 cudaError_t launch_prefill_tc(const jet_layout& lay, const jet_dims& d, const void* q,
                               const void* k, const void* v, void* o, void* ws, int* status,

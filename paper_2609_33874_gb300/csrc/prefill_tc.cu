@@ -1,6 +1,7 @@
 // Causal self-attention over every request's prefix (the prefill, Sec. 4.1) on
 // pairs of SMs with the 5th-generation tensor cores; bf16, head dimensions 128
-// and 256 (64 runs on the scoring step's kernel, attend_tc.cu).
+// and 256 (64, and batches of prefixes that fill less than a pair's block, run on
+// single SMs with the scoring step's kernel, attend_tc.cu).
 //
 // What bounds it: every query vector needs its own softmax and the key/value
 // tiles come from L2, and one SM that streams tiles for 128 query vectors

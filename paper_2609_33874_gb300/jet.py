@@ -170,7 +170,7 @@ def _stream(stream) -> Optional[int]:
         import torch
         # the current device's current stream as a raw handle: 0.3 us a call,
         # where building a torch.cuda.Stream object for it takes 3 us (a small
-        # call's whole host time is 8 to 11 us)
+        # call's whole host time is 6 to 8 us)
         return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
