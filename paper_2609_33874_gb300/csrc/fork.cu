@@ -598,17 +598,22 @@ cudaError_t launch_rule(const jet_layout& lay, const jet_dims& d, const float* s
   // No states to write: the prefix state is read once for 16 fed tokens at a
   // time (23 us against 48 at 355 rows of 32 requests x 16 heads), as long as no
   // candidate is longer than such a batch, the value width fills its columns, and
-  // there are tokens to share the read. With at most two fed tokens a request, stepping
-  // is faster: its CTAs read S0 in quarters, seven an SM (64 requests x 16 heads, one
-  // token a request 17.3 us against 24.5 by products, two 22.4 and 26.1, three 30.4
-  // and 27.0; gated linear attention 15.8 and 21.5, 19.1 and 22.8, 25.1 and 23.4). So
-  // it is with up to five tokens and few CTAs (three linear layers and a full one of D
-  // 4,096, one request of four tokens x 4 heads, 16 CTAs: 358 us against 366 by
-  // products; two requests, 32 CTAs: 362 and 367; 16 heads, 64 CTAs: 394 and 383).
+  // there are tokens to share the read. With few fed tokens a request stepping is
+  // faster: its CTAs read S0 in quarters, seven an SM (16 heads; 64 requests, one token
+  // a request 17.3 us against 24.5 by products, 1.9 22.4 and 26.1, 3.0 30.4 and 27.0;
+  // 256 requests, 2.1 tokens 87 and 107, 3.0 110 and 110; 32 requests of 2.4 tokens,
+  // some 15 long, 21.5 and 16.4). So it is with up to five tokens and few CTAs (three
+  // linear layers and a full one of D 4,096, one request of four tokens x 4 heads, 16
+  // CTAs: 358 us against 366 by products; two requests, 32 CTAs: 362 and 367; 16 heads,
+  // 64 CTAs: 394 and 383), and with candidates of more than 12 while it leaves SMs
+  // unfilled, since the products' recurrence goes with the square of a candidate (8
+  // requests x 4 heads, up to 13 a candidate, 128 CTAs: 17.3 us and 21.2; 256 CTAs 21.2
+  // and 22.1, 512 25.5 and 23.2; of 11 a candidate 128 CTAs 16.3 and 16.4).
   const long long steppers = (long long)n.R * d.Hl * (d.dv / kCols);
-  const bool few_tokens = F <= 2LL * n.R || (F <= 5LL * n.R && steppers <= 32);
+  const bool step_states = 10LL * F <= 23LL * n.R || (F <= 5LL * n.R && steppers <= 32) ||
+                          (n.max_len - 1 > 12 && steppers <= 256);
   if (!s_fork && d.dtype == JET_DTYPE_BF16 && n.max_len - 1 <= kRowTok && d.dv % kRowCols == 0 &&
-      !few_tokens)
+      !step_states)
     return launch_rows<DELTA>(lay, d, s_prefix, q, k, v, alpha, beta, q_rows, o, status, st);
   if (d.dtype == JET_DTYPE_F32) {
     return launch_pdl(fork_kernel<float, DELTA>, grid, dim3(kThreads), 0, st, lay.cand_offset,

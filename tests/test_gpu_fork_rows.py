@@ -13,12 +13,13 @@ from gpu_common import check_fork, oracle_layout, run_problem
 pytestmark = pytest.mark.gpu
 
 CASES = [
-    ([1, 1, 2, 17, 16, 2, 1, 9, 9], [4, 4, 1]),     # full batches, one ending at 16 and at 17
+    ([1, 1, 2, 17, 16, 2, 1, 9, 9], [4, 4, 1]),     # 16 fed tokens on few CTAs: stepped
     ([2] * 40 + [1] * 3, [40, 3]),                  # 40 candidates: more than a warp; none fed
     ([1, 18, 3, 2], [3, 1]),                        # 17 fed tokens: the state-stepping form
-    ([3] * 40, [1] * 40),                           # two tokens a request: stepped
-    ([3] * 39 + [4], [1] * 40),                     # and one more: by products
-    ([6] * 2, [1] * 2),                             # five, each CTA its SM: stepped
+    ([3] * 28 + [4] * 12, [1] * 40),                # 2.3 tokens a request: stepped
+    ([3] * 27 + [4] * 13, [1] * 40),                # and one more in all: by products
+    ([6] * 2, [1] * 2),                             # five, few CTAs: stepped
+    ([1, 1, 2, 17, 16, 2, 1, 9, 9] * 16, [4, 4, 1] * 16),  # the first on more CTAs: by products
 ]
 
 
